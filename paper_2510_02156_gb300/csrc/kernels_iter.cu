@@ -205,36 +205,82 @@ __device__ __forceinline__ void inc_log(Ctl *ctl, int c, double v) {
 }
 
 // ------------------------------------------------------------------ begin
-// ||b||, x = x0 or 0, loop state.  One block; sets the WHILE condition.
-__global__ void k_begin(const double *__restrict__ b, int m, const double *__restrict__ x0,
-                        double *__restrict__ x, int n, Ctl *ctl, int use_cond,
-                        cudaGraphConditionalHandle hcond) {
+// ||b||, x = x0 or 0, loop state; the last block sets the WHILE condition.
+// The grid streams b and x (at 2^20 rows one block took 523 us for what every
+// solve, and every inner solve of Algorithm 3, starts with; 152 blocks take 9);
+// the per-block sums of squares are added in block order.
+constexpr int kBeginThreads = 512;
+
+// The loop state of a solve with ||b||^2 = s (one thread).
+__device__ __forceinline__ void begin_state(Ctl *ctl, double bn) {
+    const bool finite = isfinite(bn);
+    ctl->bnorm = bn;
+    ctl->iter = 0;
+    ctl->rr = 0.0;
+    ctl->rrn = bn == 0.0 ? 0.0 : 1.0;
+    ctl->done = bn == 0.0;
+    ctl->halt = !(finite && bn > 0.0 && ctl->maxit > 0);
+    ctl->status = finite ? 0 : kDevNumeric;          // NaN or Inf in b
+    ctl->ticket = 0;
+    ctl->n_in = 0;
+    ctl->n_eq = 0;
+    ctl->outer = 0;
+    ctl->inc_full = 1;             // the first residual of a solve is exact
+    ctl->inc_count = 0;
+    ctl->nlog = 0;
+    ctl->log_full = 0;
+}
+
+// This block's share of ||b||^2 and of x = x0 or 0, for entries ld apart; true
+// in the last block of the column, with the whole sum in *tot (thread 0).
+__device__ __forceinline__ bool begin_share(const double *__restrict__ b, int m, const double *x0, double *x, int n,
+                                            int ld, double *partials, Ctl *ctl, double *tot) {
     __shared__ double red[32];
+    __shared__ int is_last;
+    const int gt = blockIdx.x * blockDim.x + threadIdx.x, gs = gridDim.x * blockDim.x;
     double s = 0.0;
-    for (int i = threadIdx.x; i < m; i += blockDim.x) s = __fma_rn(b[i], b[i], s);
+    for (int i = gt; i < m; i += gs) {
+        const double v = b[(long long)i * ld];
+        s = __fma_rn(v, v, s);
+    }
     s = block_sum(s, red);
-    __shared__ double bn;
-    if (threadIdx.x == 0) bn = sqrt(s);
+    const bool copy = x0 != nullptr && ctl->has_x0;
+    if (!copy)
+        for (int c = gt; c < n; c += gs) x[(long long)c * ld] = 0.0;
+    else if (x0 != x)
+        for (int c = gt; c < n; c += gs) x[(long long)c * ld] = x0[(long long)c * ld];
+    __threadfence();
     __syncthreads();
-    for (int c = threadIdx.x; c < n; c += blockDim.x)
-        x[c] = (bn == 0.0 || x0 == nullptr || !ctl->has_x0) ? 0.0 : x0[c];
     if (threadIdx.x == 0) {
-        const bool finite = isfinite(bn);
-        ctl->bnorm = bn;
-        ctl->iter = 0;
-        ctl->rr = 0.0;
-        ctl->rrn = bn == 0.0 ? 0.0 : 1.0;
-        ctl->done = bn == 0.0;
-        ctl->halt = !(finite && bn > 0.0 && ctl->maxit > 0);
-        ctl->status = finite ? 0 : kDevNumeric;      // NaN or Inf in b
-        ctl->ticket = 0;
-        ctl->n_in = 0;
-        ctl->n_eq = 0;
-        ctl->outer = 0;
-        ctl->inc_full = 1;         // the first residual of a solve is exact
-        ctl->inc_count = 0;
-        ctl->nlog = 0;
-        ctl->log_full = 0;
+        partials[blockIdx.x] = s;
+        __threadfence();
+        is_last = atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!is_last) return false;
+    __threadfence();
+    s = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) s += partials[i];
+    *tot = block_sum(s, red);
+    return true;
+}
+
+// ||b|| = 0: x = 0 whatever x0 holds (the last block, after every other has written).
+__device__ __forceinline__ void begin_zero(double *x, int n, int ld) {
+    for (int c = threadIdx.x; c < n; c += blockDim.x) x[(long long)c * ld] = 0.0;
+}
+
+__global__ void __launch_bounds__(kBeginThreads) k_begin(const double *__restrict__ b, int m, const double *x0,
+                                                         double *x, int n, double *partials, Ctl *ctl, int use_cond,
+                                                         cudaGraphConditionalHandle hcond) {
+    __shared__ double bn;
+    double tot;
+    if (!begin_share(b, m, x0, x, n, 1, partials, ctl, &tot)) return;
+    if (threadIdx.x == 0) bn = sqrt(tot);
+    __syncthreads();
+    if (bn == 0.0) begin_zero(x, n, 1);
+    if (threadIdx.x == 0) {
+        begin_state(ctl, bn);
         if (use_cond) cudaGraphSetConditional(hcond, ctl->halt ? 0u : 1u);
     }
 }
@@ -2917,38 +2963,23 @@ __device__ __forceinline__ VecT<T, VEC> vload_keep(const T *p, unsigned long lon
 }
 
 // k_begin for a block of columns: ||b_j||, x_j = x0_j or 0, loop state; the
-// last column sets the WHILE condition.  Grid (1, nr).
-__global__ void k_mr_begin(const double *__restrict__ b, int m, const double *__restrict__ x0,
-                           double *__restrict__ x, int n, Ctl *ctl0, int nr, unsigned *grp,
-                           int use_cond, cudaGraphConditionalHandle hcond) {
-    __shared__ double red[32];
+// last column sets the WHILE condition.  Grid (g, nr).
+__global__ void __launch_bounds__(kBeginThreads) k_mr_begin(const double *__restrict__ b, int m, const double *x0,
+                                                            double *x, int n, double *partials, Ctl *ctl0, int nr,
+                                                            unsigned *grp, int use_cond,
+                                                            cudaGraphConditionalHandle hcond) {
     __shared__ double bn;
     const int jc = blockIdx.y;
-    Ctl *ctl = ctl0 + jc;
-    double s = 0.0;
-    for (int i = threadIdx.x; i < m; i += blockDim.x) {
-        const double v = b[(long long)i * nr + jc];
-        s = __fma_rn(v, v, s);
-    }
-    s = block_sum(s, red);
-    if (threadIdx.x == 0) bn = sqrt(s);
+    double tot;
+    if (!begin_share(b + jc, m, x0 ? x0 + jc : nullptr, x + jc, n, nr, partials + (long long)jc * gridDim.x, ctl0 + jc,
+                     &tot))
+        return;
+    if (threadIdx.x == 0) bn = sqrt(tot);
     __syncthreads();
-    const bool zero = bn == 0.0 || x0 == nullptr || !ctl->has_x0;
-    for (int c = threadIdx.x; c < n; c += blockDim.x)
-        x[(long long)c * nr + jc] = zero ? 0.0 : x0[(long long)c * nr + jc];
+    if (bn == 0.0) begin_zero(x + jc, n, nr);
+    __syncthreads();
     if (threadIdx.x == 0) {
-        const bool finite = isfinite(bn);
-        ctl->bnorm = bn;
-        ctl->iter = 0;
-        ctl->rr = 0.0;
-        ctl->rrn = bn == 0.0 ? 0.0 : 1.0;
-        ctl->done = bn == 0.0;
-        ctl->halt = !(finite && bn > 0.0 && ctl->maxit > 0);
-        ctl->status = finite ? 0 : kDevNumeric;
-        ctl->ticket = 0;
-        ctl->n_in = 0;
-        ctl->n_eq = 0;
-        ctl->outer = 0;
+        begin_state(ctl0 + jc, bn);
         group_condition(ctl0, nr, grp, use_cond, hcond);
     }
 }
@@ -3512,13 +3543,16 @@ void configure_kernels() {
 
 void launch_begin(rorbk_ctx *h, const double *b, const double *x0, double *x, int use_cond,
                   unsigned long long hcond) {
+    const int nr = std::max(1, h->nr);
+    const int g = (int)std::max<long long>(1, std::min<long long>(std::max(1, h->num_sms / nr),
+                                                                 (std::max(h->m, h->n) + kBeginThreads - 1) / kBeginThreads));
     if (h->nr) {
-        k_mr_begin<<<dim3(1, h->nr), 1024, 0, h->stream>>>(b, (int)h->m, x0, x, (int)h->n, h->ctl, h->nr,
-                                                           h->mr.grp, use_cond, (cudaGraphConditionalHandle)hcond);
+        k_mr_begin<<<dim3(g, nr), kBeginThreads, 0, h->stream>>>(b, (int)h->m, x0, x, (int)h->n, h->partials, h->ctl, nr,
+                                                                 h->mr.grp, use_cond, (cudaGraphConditionalHandle)hcond);
         return;
     }
-    k_begin<<<1, 1024, 0, h->stream>>>(b, (int)h->m, x0, x, (int)h->n, h->ctl, use_cond,
-                                       (cudaGraphConditionalHandle)hcond);
+    k_begin<<<g, kBeginThreads, 0, h->stream>>>(b, (int)h->m, x0, x, (int)h->n, h->partials, h->ctl, use_cond,
+                                                (cudaGraphConditionalHandle)hcond);
 }
 
 void launch_dense_gram(rorbk_ctx *h, Ctl *ctl, int tensor_cores) {
