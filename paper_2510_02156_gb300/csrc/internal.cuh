@@ -63,7 +63,8 @@ struct Ctl {
     int outer_done;
     int has_x0;
     // dynamic block bookkeeping
-    int dynE, dyn_nsh, dyn_nS, dyn_npair, dyn_nraw, pad3_;
+    int dynE, dyn_nsh, dyn_nS, dyn_npair, dyn_nraw;
+    int fac_n;             // order of the system left to the cluster's factor (0: none)
     int halt;              // no further iteration runs (converged, error or maxit)
     int weighted;          // residual-weighted draws (RORBK_DIST_RESIDUAL_WEIGHTED)
     // incremental residual (RORBK_RESIDUAL_INCREMENTAL): the scatters log
@@ -222,6 +223,9 @@ struct rorbk_ctx {
         unsigned long long *raw = nullptr, *skeys = nullptr, *pkeys = nullptr;
         long long pcap = 0, skcap = 0;
         double *g = nullptr;
+        double *gc = nullptr, *z = nullptr;   // the cluster's factor: Gram (sparse A), right-hand side
+        int *fidx = nullptr;
+        int cluster = 0;        // blocks of the cluster that factors (0: none; K fits one warp's component)
     } dyn;
     // a block of nr right-hand sides (rorbk_multi_create; 0: one right-hand
     // side): x, b are row-major n x nr and m x nr, r and r32 hold nr columns in
@@ -275,6 +279,7 @@ void fill_dense_columns(rorbk_ctx *h);        // column indices of a dense A hel
 void configure_kernels();
 int residual_grid(rorbk_ctx *h);   // one resident wave of the residual kernel
 int mres_grid(rorbk_ctx *h, int nr, int fp32);   // one resident wave of the column-block residual
+int chol_cluster_blocks(rorbk_ctx *h);   // blocks of the cluster that factors the dynamic block's Gram
 // the tunable grids (per column), defaults where h->tune holds 0
 int grid_topk(rorbk_ctx *h);
 int grid_collect(rorbk_ctx *h);

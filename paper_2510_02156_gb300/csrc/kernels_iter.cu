@@ -10,9 +10,11 @@
 //   k_topk_collect rows above the 22-bit threshold and the candidates on it;
 //                  the last block completes the exact top-K set
 //   k_dyn_mark     gathers A_I, marks shared columns, Gram diagonal; the last
-//                  block factors G = A_I A_I^T + mu I on the coupled rows and
-//                  solves for y, the first block done forms the next draws
-//   k_dyn_scatter  x += A_I^T y; ends the iteration, sets the loop condition
+//                  block factors G = A_I A_I^T + mu I on the coupled rows' small
+//                  components and solves for y, the first block done forms the
+//                  next draws
+//   k_dyn_scatter  the large components in one cluster, x += A_I^T y; ends the
+//                  iteration, sets the loop condition
 //
 // Compute type T is double (the plain method) or float (the inner solve of
 // the mixed-precision form).  In FP64 every multiply-add is one fused
@@ -21,15 +23,16 @@
 // columns; column-ordered triangular solves), so the iterates reproduce the
 // FP64 definition exactly.  FP64 arithmetic on this part has a long latency,
 // so chains are kept short: the Cholesky of the coupled rows runs per
-// connected component (one warp each), or, for components above 32 rows,
-// along its elimination tree (all columns of one tree level at once); both
-// perform the same operations on every entry in the same order.
+// connected component, one warp each, or, for components above 32 rows, in one
+// thread-block cluster (cluster_chol.cuh); both perform the operations of the
+// whole-matrix factor on every entry in the same order.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
 
 #include <algorithm>
 
+#include "cluster_chol.cuh"
 #include "common.cuh"
 #include "internal.cuh"
 #include "topk_key.cuh"
@@ -1234,7 +1237,10 @@ struct Dyn {
     unsigned long long *skeys;  // [pow2 >= 2 ecap] shared entries sorted by (column, entry)
     unsigned long long *pkeys;  // [pcap] Gram contributions (fallback)
     long long pcap;
-    double *g;                  // [K(K+1)/2] packed Gram fallback
+    double *g;                  // [K(K+1)/2] packed Gram (dense A; coupled rows above kSPackedMax)
+    double *gc;                 // [K(K+1)/2] packed Gram of the rows the cluster factors (sparse A)
+    double *z;                  // [K] right-hand side of the cluster's factor
+    int *fidx;                  // [K] position in I of the rows it factors
     int K, n;                   // sizes of one column's buffers (a block of columns
     long long skcap;            // keeps its columns' buffers one after the other)
 };
@@ -1258,6 +1264,9 @@ __device__ __forceinline__ Dyn dyn_col(Dyn D, int jc) {
     D.skeys += jc * D.skcap;
     D.pkeys += jc * D.pcap;
     D.g += jc * (K * (K + 1) / 2);
+    D.gc += jc * (K * (K + 1) / 2);
+    D.z += jc * K;
+    D.fidx += jc * K;
     return D;
 }
 
@@ -1412,261 +1421,7 @@ __device__ void packed_cholesky(double *G, int nS, int *bad) {
     }
 }
 
-// Elimination tree of the coupled rows (nS <= kSymMax) from the Gram's
-// nonzero pattern, as bitsets: col[j] = rows i > j where L_ij may be
-// nonzero, row[i] = columns j < i where L_ij may be nonzero; level[j] = height
-// of j above the leaves; columns sorted by level.  Returns the cost estimates
-// (cycles) of the level-scheduled and the column-by-column factorisations.
-constexpr int kSymMax = 256;
-constexpr int kSymW = kSymMax / 32;
-
-struct Sym {
-    unsigned *col, *row;        // [kSymMax * kSymW]
-    int16_t *level, *order, *lvl_off;   // [kSymMax], [kSymMax], [kSymMax + 1]
-    int *eoff;                  // [kSymMax + 1] first off-diagonal entry of order[q]
-};
-
-__device__ __forceinline__ int bit_count(const unsigned *w) {
-    int c = 0;
-#pragma unroll
-    for (int q = 0; q < kSymW; ++q) c += __popc(w[q]);
-    return c;
-}
-
-__device__ void symbolic(const double *G, int nS, Sym S, int *s_nlev, int *s_use_levels) {
-    __shared__ int s_cnt[kSymMax + 1];
-    __shared__ long long s_cost_lvl, s_cost_col;
-    const int tid = threadIdx.x, lane = tid & 31;
-    for (int q = tid; q < kSymMax * kSymW; q += blockDim.x) { S.col[q] = 0u; S.row[q] = 0u; }
-    for (int j = tid; j < kSymMax; j += blockDim.x) { S.level[j] = 0; s_cnt[j] = 0; }
-    if (tid == 0) s_cnt[kSymMax] = 0;
-    __syncthreads();
-    for (int q = tid; q < nS * (nS - 1) / 2; q += blockDim.x) {   // entry (i, j), j < i, packed by rows
-        int i = (int)((sqrtf(8.0f * (float)q + 1.0f) + 1.0f) * 0.5f);
-        while (i * (i - 1) / 2 > q) --i;
-        while ((i + 1) * i / 2 <= q) ++i;
-        const int j = q - i * (i - 1) / 2;
-        if (G[pidx(i, j)] != 0.0) atomicOr(&S.col[j * kSymW + (i >> 5)], 1u << (i & 31));
-    }
-    __syncthreads();
-    if (nS <= 64 && tid < 32) {
-        // one warp, every column's structure in registers: lane l holds
-        // columns l and l + 32 as 64-bit row masks (rows below the diagonal)
-        // and their levels.  Column j's parent p is its first row; p takes
-        // j's other rows (fill) and a level above j's.
-        unsigned long long m0 = 0ull, m1 = 0ull;
-        int lv0 = 0, lv1 = 0;
-        if (lane < nS) m0 = ((unsigned long long)S.col[lane * kSymW + 1] << 32) | S.col[lane * kSymW];
-        if (lane + 32 < nS)
-            m1 = ((unsigned long long)S.col[(lane + 32) * kSymW + 1] << 32) | S.col[(lane + 32) * kSymW];
-        for (int j = 0; j < nS; ++j) {
-            const bool hi = j >= 32;                  // uniform across the warp
-            const unsigned long long mj = __shfl_sync(0xffffffffu, hi ? m1 : m0, j & 31);
-            const int lvj = __shfl_sync(0xffffffffu, hi ? lv1 : lv0, j & 31);
-            if (mj) {
-                const int p = __ffsll((long long)mj) - 1;
-                const unsigned long long add = mj & ~(1ull << p);
-                if ((p & 31) == lane) {
-                    if (p < 32) { m0 |= add; lv0 = max(lv0, lvj + 1); }
-                    else { m1 |= add; lv1 = max(lv1, lvj + 1); }
-                }
-            }
-        }
-        if (lane < nS) {
-            S.col[lane * kSymW] = (unsigned)m0;
-            S.col[lane * kSymW + 1] = (unsigned)(m0 >> 32);
-            S.level[lane] = (int16_t)lv0;
-        }
-        if (lane + 32 < nS) {
-            S.col[(lane + 32) * kSymW] = (unsigned)m1;
-            S.col[(lane + 32) * kSymW + 1] = (unsigned)(m1 >> 32);
-            S.level[lane + 32] = (int16_t)lv1;
-        }
-    } else if (tid < 32) {              // one warp: elimination tree and fill
-        for (int j = 0; j < nS; ++j) {
-            const unsigned w = lane < kSymW ? S.col[j * kSymW + lane] : 0u;
-            const unsigned bal = __ballot_sync(0xffffffffu, w != 0u);
-            if (bal) {
-                const int fw = __ffs(bal) - 1;
-                const unsigned wf = __shfl_sync(0xffffffffu, w, fw);
-                const int p = fw * 32 + __ffs(wf) - 1;
-                if (lane < kSymW) {
-                    unsigned add = w;
-                    if (lane == (p >> 5)) add &= ~(1u << (p & 31));
-                    S.col[p * kSymW + lane] |= add;
-                }
-                if (lane == 0) S.level[p] = (int16_t)max((int)S.level[p], (int)S.level[j] + 1);
-            }
-            __syncwarp();
-        }
-    }
-    __syncthreads();
-    // row structures (transpose) and level counts
-    for (int q = tid; q < nS * kSymW; q += blockDim.x) {
-        const int j = q / kSymW, wd = q % kSymW;
-        unsigned w = S.col[q];
-        while (w) {
-            const int bitp = __ffs(w) - 1;
-            w &= w - 1;
-            const int i = wd * 32 + bitp;
-            atomicOr(&S.row[i * kSymW + (j >> 5)], 1u << (j & 31));
-        }
-    }
-    for (int j = tid; j < nS; j += blockDim.x) atomicAdd(&s_cnt[S.level[j]], 1);
-    __syncthreads();
-    if (tid == 0) {                     // levels are below nS
-        int nl = 0, acc = 0;
-        for (int L = 0; L < nS; ++L) {
-            if (s_cnt[L]) nl = L + 1;
-            const int c = s_cnt[L];
-            S.lvl_off[L] = (int16_t)acc;
-            acc += c;
-            s_cnt[L] = 0;
-        }
-        for (int L = nS; L <= kSymMax; ++L) S.lvl_off[L] = (int16_t)acc;
-        *s_nlev = nl;
-        s_cost_lvl = 0;
-        s_cost_col = 0;
-    }
-    __syncthreads();
-    for (int j = tid; j < nS; j += blockDim.x) {
-        const int L = S.level[j];
-        S.order[S.lvl_off[L] + atomicAdd(&s_cnt[L], 1)] = (int16_t)j;
-    }
-    __syncthreads();
-    {   // off-diagonal entries of each column, in level order
-        __shared__ int sc2[33];
-        int carry = 0;
-        for (int base = 0; base < nS; base += blockDim.x) {
-            const int q = base + tid;
-            const int c = q < nS ? bit_count(S.col + S.order[q] * kSymW) : 0;
-            int total;
-            const int pre = block_exclusive_scan(c, sc2, &total);
-            if (q < nS) S.eoff[q] = carry + pre;
-            carry += total;
-        }
-        if (tid == 0) S.eoff[nS] = carry;
-        __syncthreads();
-    }
-    // cost model (cycles): FP64 fma ~70, sqrt/div ~500 each, barrier ~100;
-    // one warp per level
-    {
-        const int warp = tid >> 5, nwarps = blockDim.x >> 5;
-        long long lvl = 0;
-        for (int L = warp; L < *s_nlev; L += nwarps) {
-            int mr = 0, mc = 0;
-            for (int q = S.lvl_off[L] + lane; q < S.lvl_off[L + 1]; q += 32) {
-                const int j = S.order[q];
-                mr = max(mr, bit_count(S.row + j * kSymW));
-                mc = max(mc, bit_count(S.col + j * kSymW));
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                mr = max(mr, __shfl_xor_sync(0xffffffffu, mr, o));
-                mc = max(mc, __shfl_xor_sync(0xffffffffu, mc, o));
-            }
-            lvl += (long long)(2 * mr + mc) * 90 + 2300;
-        }
-        if (lane == 0 && lvl) atomicAdd((unsigned long long *)&s_cost_lvl, (unsigned long long)lvl);
-    }
-    __syncthreads();
-    if (tid == 0) {
-        s_cost_col = (long long)nS * (1300 + 2 * 800);
-        *s_use_levels = s_cost_lvl < s_cost_col;
-    }
-    __syncthreads();
-}
-
-// Left-looking Cholesky by tree levels: every column of a level at once.
-// Entry (a, b) receives its updates L_aj L_bj over the columns j of row b in
-// ascending order (the right-looking order).  Diagonals first (one thread per
-// column: L_bb = sqrt(.)), then the off-diagonals (one thread per entry:
-// L_ab = (.) / L_bb), so every FP64 instruction carries as many columns or
-// entries as the level has.
-__device__ __forceinline__ int kth_bit(const unsigned *w, int k) {
-    for (int wd = 0; wd < kSymW; ++wd) {
-        const int c = __popc(w[wd]);
-        if (k < c) return wd * 32 + (int)__fns(w[wd], 0, k + 1);
-        k -= c;
-    }
-    return -1;
-}
-
-template <bool RC>
-__device__ void level_cholesky(double *G, int nS, Sym S, int nlev, int *bad) {
-    for (int L = 0; L < nlev; ++L) {
-        const int q0 = S.lvl_off[L], q1 = S.lvl_off[L + 1];
-        for (int q = q0 + threadIdx.x; q < q1; q += blockDim.x) {
-            const int b = S.order[q];
-            const unsigned *rb = S.row + b * kSymW;
-            double v = G[pidx(b, b)];
-            for (int wd = 0; wd < kSymW; ++wd)
-                for (unsigned w = rb[wd]; w; w &= w - 1) {
-                    const int j = wd * 32 + __ffs(w) - 1;
-                    const double lbj = G[pidx(b, j)];
-                    v = __fma_rn(-lbj, lbj, v);
-                }
-            if (!(v > 0.0)) { *bad = 1; v = 1.0; }
-            G[pidx(b, b)] = chol_diag<RC>(v);
-        }
-        __syncthreads();
-        const int e0 = S.eoff[q0], e1 = S.eoff[q1];
-        for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-            int lo = q0, hi = q1;                       // last q with eoff[q] <= e
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (S.eoff[mid] <= e) lo = mid; else hi = mid;
-            }
-            const int b = S.order[lo];
-            const int a = kth_bit(S.col + b * kSymW, e - S.eoff[lo]);
-            const unsigned *rb = S.row + b * kSymW;
-            double v = G[pidx(a, b)];
-            for (int wd = 0; wd < kSymW; ++wd)
-                for (unsigned w = rb[wd]; w; w &= w - 1) {
-                    const int j = wd * 32 + __ffs(w) - 1;
-                    v = __fma_rn(-G[pidx(a, j)], G[pidx(b, j)], v);
-                }
-            G[pidx(a, b)] = chol_div<RC>(v, G[pidx(b, b)]);
-        }
-        __syncthreads();
-    }
-}
-
-// z <- L^{-T} L^{-1} z on the coupled rows, by tree levels (forward:
-// ascending levels, row sums over ascending columns; backward: descending
-// levels, sums over descending rows), one thread per row.
-template <bool RC>
-__device__ void level_solve(const double *G, int nS, Sym S, int nlev, double *z) {
-    for (int L = 0; L < nlev; ++L) {
-        for (int q = S.lvl_off[L] + threadIdx.x; q < S.lvl_off[L + 1]; q += blockDim.x) {
-            const int b = S.order[q];
-            double v = z[b];
-            const unsigned *rb = S.row + b * kSymW;
-            for (int wd = 0; wd < kSymW; ++wd)
-                for (unsigned w = rb[wd]; w; w &= w - 1) {
-                    const int j = wd * 32 + __ffs(w) - 1;
-                    v = __fma_rn(-G[pidx(b, j)], z[j], v);
-                }
-            z[b] = chol_div<RC>(v, G[pidx(b, b)]);
-        }
-        __syncthreads();
-    }
-    for (int L = nlev - 1; L >= 0; --L) {
-        for (int q = S.lvl_off[L] + threadIdx.x; q < S.lvl_off[L + 1]; q += blockDim.x) {
-            const int b = S.order[q];
-            double v = z[b];
-            const unsigned *cb = S.col + b * kSymW;
-            for (int wd = kSymW - 1; wd >= 0; --wd)
-                for (unsigned w = cb[wd]; w; ) {
-                    const int hb = 31 - __clz(w);
-                    w &= ~(1u << hb);
-                    const int c = wd * 32 + hb;
-                    v = __fma_rn(-G[pidx(c, b)], z[c], v);
-                }
-            z[b] = chol_div<RC>(v, G[pidx(b, b)]);
-        }
-        __syncthreads();
-    }
-}
+constexpr int kSymMax = 256;            // coupled rows up to which components are looked for
 
 // Column-by-column solves (right-looking order) with zero columns skipped.
 template <bool RC>
@@ -1711,19 +1466,21 @@ __device__ void column_solve(const double *G, int nS, double *z, unsigned char *
 // column solves (packed_cholesky, column_solve; zero multipliers skipped as
 // there).  The components come from union-find over the Gram's nonzero pairs
 // (roots hooked to the smaller root, then pointer jumping), their members
-// listed ascending; one warp factors and solves each.  Returns false, with G
-// and z untouched, when a component has more than kCompMax rows or the
-// union-find did not settle; the caller then takes the other paths.
+// listed ascending; one warp factors and solves each of up to kCompMax rows.
+// Returns the number of rows in larger components and lists them ascending in
+// big; G and z are untouched there (a cluster factors them in k_dyn_scatter).  All
+// rows are listed when the union-find did not settle.
 constexpr int kCompMax = 32;
 template <bool RC>
-__device__ bool component_factor(double *G, int nS, const unsigned long long *pkeys, int npk,
-                                 const int16_t *spos, double *z, int *bad) {
+__device__ int component_factor(double *G, int nS, const unsigned long long *pkeys, int npk,
+                                const int16_t *spos, double *z, int *bad, int16_t *big) {
     __shared__ int par[kSymMax], cid[kSymMax], csz[kSymMax], cst[kSymMax + 1], memb[kSymMax];
     __shared__ int sc[33];
-    __shared__ int s_changed, s_max, s_nc;
+    __shared__ int s_changed, s_nc;
+    __shared__ double rdiag[kSymMax];                         // reciprocals of the factor's diagonal
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
     for (int q = tid; q < nS; q += blockDim.x) { par[q] = q; csz[q] = 0; }
-    if (tid == 0) { s_changed = 1; s_max = 0; }
+    if (tid == 0) s_changed = 1;
     __syncthreads();
     for (int rnd = 0; rnd < 64 && s_changed; ++rnd) {
         __syncthreads();
@@ -1748,12 +1505,15 @@ __device__ bool component_factor(double *G, int nS, const unsigned long long *pk
         }
         __syncthreads();
     }
-    if (s_changed) return false;
+    if (s_changed || nS > (int)blockDim.x) {                  // nS <= kSymMax <= blockDim.x
+        for (int q = tid; q < nS; q += blockDim.x) big[q] = (int16_t)q;
+        __syncthreads();
+        return nS;
+    }
     // components numbered by their roots, sizes, members ascending
     const int isroot = tid < nS && par[tid] == tid;
     int nc;
-    const int pre = nS <= (int)blockDim.x ? block_exclusive_scan(isroot, sc, &nc) : 0;
-    if (nS > (int)blockDim.x) return false;                   // not reached: nS <= kSymMax
+    const int pre = block_exclusive_scan(isroot, sc, &nc);
     if (isroot) cid[tid] = pre;
     __syncthreads();
     for (int q = tid; q < nS; q += blockDim.x) atomicAdd(&csz[cid[par[q]]], 1);
@@ -1763,9 +1523,11 @@ __device__ bool component_factor(double *G, int nS, const unsigned long long *pk
     const int st = block_exclusive_scan(size, sc, &tot);
     if (tid < nc) cst[tid] = st;
     if (tid == 0) { cst[nc] = tot; s_nc = nc; }
-    if (size) atomicMax(&s_max, size);
     __syncthreads();
-    if (s_max > kCompMax) return false;
+    const int inbig = tid < nS && csz[cid[par[tid]]] > kCompMax;
+    int nbig;
+    const int bpos = block_exclusive_scan(inbig, sc, &nbig);
+    if (inbig) big[bpos] = (int16_t)tid;
     for (int q = tid; q < nS; q += blockDim.x) {
         const int root = par[q];
         int rank = 0;
@@ -1773,25 +1535,47 @@ __device__ bool component_factor(double *G, int nS, const unsigned long long *pk
         memb[cst[cid[root]] + rank] = q;
     }
     __syncthreads();
-    // one warp per component: right-looking factor, then the two solves
+    // one warp per component: right-looking factor with the forward solve beside
+    // it (lane i holds z_i; at column j lane j divides z_j while the lanes after
+    // it divide their rows' entries), then the backward solve.  Every lane forms
+    // the pivot itself, and the quotients come from its reciprocal
+    // (cluster_chol.cuh): about 900 cycles per column where a square root, a
+    // division and the hand-over between lanes took 1,900, and 300 per backward
+    // step instead of 800
     for (int c = wid; c < s_nc; c += nw) {
         const int *M = memb + cst[c];
         const int n = cst[c + 1] - cst[c];
+        if (n > kCompMax) continue;
+        const int mi = M[min(lane, n - 1)];                   // this lane's row
+        double zi = lane < n ? z[mi] : 0.0;
         for (int j = 0; j < n; ++j) {
             const int mj = M[j];
-            if (lane == 0) {
-                double d = G[pidx(mj, mj)];
-                if (!(d > 0.0)) { *bad = 1; d = 1.0; }
-                G[pidx(mj, mj)] = chol_diag<RC>(d);
+            double d = G[pidx(mj, mj)];
+            const double v = lane == j ? zi : lane > j && lane < n ? G[pidx(mi, mj)] : 0.0;
+            if (!positive(d)) {
+                if (lane == 0) *bad = 1;
+                d = 1.0;
             }
-            __syncwarp();
-            const double l = G[pidx(mj, mj)];
-            int any = 0;
-            for (int i = j + 1 + lane; i < n; i += 32) {
-                const double v = G[pidx(M[i], mj)];
-                if (v != 0.0) { G[pidx(M[i], mj)] = chol_div<RC>(v, l); any = 1; }
+            double q, dg, rl;
+            if constexpr (RC) {
+                dg = rl = rsqrt(d);
+                q = v * rl;
+            } else {
+                const Pivot pv = pivot(d);
+                q = pivot_div(v, pv);
+                dg = pv.l;
+                rl = pv.rl;
             }
-            if (!__any_sync(0xffffffffu, any)) continue;
+            const bool below = lane > j && lane < n;
+            if (below) G[pidx(mi, mj)] = q;
+            if (lane == j) {
+                G[pidx(mj, mj)] = dg;
+                rdiag[mj] = rl;
+                zi = q;
+            }
+            if (!__any_sync(0xffffffffu, below && nonzero(q))) continue;
+            const double wj = __shfl_sync(0xffffffffu, q, j);
+            if (below) zi = sub_prod(zi, q, wj);
             __syncwarp();
             const int t = n - j - 1;                          // trailing rows j+1 .. n-1
             for (int e = lane; e < t * (t + 1) / 2; e += 32) {
@@ -1800,38 +1584,24 @@ __device__ bool component_factor(double *G, int nS, const unsigned long long *pk
                 while ((ai + 1) * (ai + 2) / 2 <= e) ++ai;
                 const int bi = e - ai * (ai + 1) / 2;
                 const int a = M[j + 1 + ai], b = M[j + 1 + bi];
-                const double la = G[pidx(a, mj)];
-                if (la == 0.0) continue;
-                const double lb = G[pidx(b, mj)];
-                if (lb != 0.0) G[pidx(a, b)] = __fma_rn(-la, lb, G[pidx(a, b)]);
+                G[pidx(a, b)] = sub_prod(G[pidx(a, b)], G[pidx(a, mj)], G[pidx(b, mj)]);
             }
             __syncwarp();
         }
-        for (int j = 0; j < n; ++j) {                        // forward
-            const int mj = M[j];
-            if (lane == 0) z[mj] = chol_div<RC>(z[mj], G[pidx(mj, mj)]);
-            __syncwarp();
-            const double zj = z[mj];
-            for (int i = j + 1 + lane; i < n; i += 32) {
-                const double lij = G[pidx(M[i], mj)];
-                if (lij != 0.0) z[M[i]] = __fma_rn(-lij, zj, z[M[i]]);
-            }
-            __syncwarp();
-        }
+        __syncwarp();
         for (int j = n - 1; j >= 0; --j) {                   // backward
             const int mj = M[j];
-            if (lane == 0) z[mj] = chol_div<RC>(z[mj], G[pidx(mj, mj)]);
-            __syncwarp();
-            const double zj = z[mj];
-            for (int i = lane; i < j; i += 32) {
-                const double lji = G[pidx(mj, M[i])];
-                if (lji != 0.0) z[M[i]] = __fma_rn(-lji, zj, z[M[i]]);
-            }
-            __syncwarp();
+            double zj = __shfl_sync(0xffffffffu, zi, j);
+            const double l = G[pidx(mj, mj)], rl = rdiag[mj];
+            if constexpr (RC) zj = zj * l;
+            else zj = quotient_rn(zj, __dmul_rn(zj, rl), l, rl, divisor_ok(l));
+            if (lane == j) zi = zj;
+            if (lane < j) zi = sub_prod(zi, G[pidx(mj, mi)], zj);
         }
+        if (lane < n) z[mi] = zi;
     }
     __syncthreads();
-    return true;
+    return nbig;
 }
 
 // The factor step of the dynamic update, run by the last block of
@@ -1841,31 +1611,25 @@ __device__ bool component_factor(double *G, int nS, const unsigned long long *pk
 // (y_a = (r_a / L_aa) / L_aa outside S).
 template <typename T, bool MC>
 __device__ void dyn_factor(const T *__restrict__ r, int K, Dyn D, Ctl *ctl,
-                           unsigned long long *dsm, const Cols &cl) {
+                           unsigned long long *dsm, const Cols &cl, int fac_max) {
     constexpr bool RC = sizeof(T) == sizeof(float);   // the mixed form's inner solve
-    __shared__ int s_nsh, s_npk, s_nS, s_bad, s_fill, s_fill2, s_nlev, s_uselev;
+    __shared__ int s_nsh, s_npk, s_nS, s_bad, s_fill, s_fill2;
     __shared__ int sc[33];
     unsigned long long *sk = dsm;                                   // kShCap
     unsigned long long *pk = sk + kShCap;                           // kPairCap
     double *z = (double *)(pk + kPairCap);                          // kMaxDynRows
     double *Gs = z + kMaxDynRows;                                   // kGPack
-    Sym S;
-    S.col = (unsigned *)(Gs + kGPack);                              // kSymMax * kSymW
-    S.row = S.col + kSymMax * kSymW;                                // kSymMax * kSymW
-    S.level = (int16_t *)(S.row + kSymMax * kSymW);                 // kSymMax
-    S.order = S.level + kSymMax;                                    // kSymMax
-    S.lvl_off = S.order + kSymMax;                                  // kSymMax + 1
-    S.eoff = (int *)(S.lvl_off + kSymMax + 2);                      // kSymMax + 1
-    int16_t *spos = (int16_t *)(S.eoff + kSymMax + 2);              // kMaxDynRows
+    int16_t *spos = (int16_t *)(Gs + kGPack);                       // kMaxDynRows
     int16_t *sidx = spos + kMaxDynRows;                             // kMaxDynRows
-    unsigned char *flag = (unsigned char *)(sidx + kMaxDynRows);    // kMaxDynRows
+    int16_t *big = sidx + kMaxDynRows;                              // kMaxDynRows
+    unsigned char *flag = (unsigned char *)(big + kMaxDynRows);     // kMaxDynRows
     unsigned char *cz = flag + kMaxDynRows;
     unsigned char *rz = cz + kMaxDynRows;
     const int tid = threadIdx.x;
     const int E = ctl->dynE;
     const int nraw = ctl->dyn_nraw;
     for (int a = tid; a < K; a += blockDim.x) { flag[a] = 0; cz[a] = 0; rz[a] = 0; }
-    if (tid == 0) { s_nsh = 0; s_npk = 0; s_bad = 0; s_fill = 0; s_fill2 = 0; }
+    if (tid == 0) { s_nsh = 0; s_npk = 0; s_bad = 0; s_fill = 0; s_fill2 = 0; ctl->fac_n = 0; }
     if (nraw > 2 * D.ecap || nraw >= (1 << 22)) {   // positions are packed in 22 bits
         if (tid == 0) set_status(&ctl->status, kDevBounds);
         return;
@@ -1958,7 +1722,7 @@ __device__ void dyn_factor(const T *__restrict__ r, int K, Dyn D, Ctl *ctl,
     if (tid == 0) s_nS = cnt;
     __syncthreads();
     const int nS = s_nS;
-    double *G = nS <= kSPackedMax ? Gs : D.g;
+    double *G = nS <= kSPackedMax ? Gs : nS <= kSymMax ? D.g : D.gc;
     for (long long q = tid; q < (long long)nS * (nS + 1) / 2; q += blockDim.x) G[q] = 0.0;
     __syncthreads();
     for (int i = tid; i < nS; i += blockDim.x) G[pidx(i, i)] = D.gdiag[sidx[i]];
@@ -1977,20 +1741,32 @@ __device__ void dyn_factor(const T *__restrict__ r, int K, Dyn D, Ctl *ctl,
     __syncthreads();
     for (int q = tid; q < nS; q += blockDim.x) z[q] = (double)r[rpos<MC>(cl, D.I[sidx[q]])];
     __syncthreads();
-    bool by_comp = false;
-    if (nS > 0 && nS <= kSymMax) by_comp = component_factor<RC>(G, nS, pkeys, npk, spos, z, &s_bad);
-    if (by_comp) {
-        if (tid == 0) s_uselev = 0;
-    } else if (nS > 0) {
-        if (nS <= kSymMax) symbolic(G, nS, S, &s_nlev, &s_uselev);
-        else if (tid == 0) s_uselev = 0;
+    // small components here, one warp each; the rows of the larger ones are
+    // left to the cluster (k_dyn_scatter), or, above its largest order, factored
+    // here column by column
+    int nB = nS;
+    if (nS > kSymMax) {
+        for (int q = tid; q < nS; q += blockDim.x) big[q] = (int16_t)q;
         __syncthreads();
-        if (s_uselev) {
-            level_cholesky<RC>(G, nS, S, s_nlev, &s_bad);
-            level_solve<RC>(G, nS, S, s_nlev, z);
+    } else if (nS > 0) {
+        nB = component_factor<RC>(G, nS, pkeys, npk, spos, z, &s_bad, big);
+    }
+    if (nB > 0) {
+        if (G != D.gc)
+            for (int i = tid >> 5; i < nB; i += blockDim.x >> 5)
+                for (int j = tid & 31; j <= i; j += 32) D.gc[pidx(i, j)] = G[pidx(big[i], big[j])];
+        for (int q = tid; q < nB; q += blockDim.x) {
+            D.z[q] = z[big[q]];
+            D.fidx[q] = sidx[big[q]];
+        }
+        if (nB <= fac_max) {
+            if (tid == 0) ctl->fac_n = nB;
         } else {
-            packed_cholesky<RC>(G, nS, &s_bad);
-            column_solve<RC>(G, nS, z, cz, rz);
+            __syncthreads();
+            packed_cholesky<RC>(D.gc, nB, &s_bad);
+            column_solve<RC>(D.gc, nB, D.z, cz, rz);
+            for (int q = tid; q < nB; q += blockDim.x) z[big[q]] = D.z[q];
+            __syncthreads();
         }
     }
     for (int q = tid; q < nS; q += blockDim.x) D.y[sidx[q]] = z[q];
@@ -2002,7 +1778,7 @@ __device__ void dyn_factor(const T *__restrict__ r, int K, Dyn D, Ctl *ctl,
         ctl->dyn_npair = npk;
         if (ctl->tr_dyn && ctl->iter < ctl->trace_cap) {
             int *t = ctl->tr_dyn + 4 * ctl->iter;
-            t[0] = E; t[1] = nsh; t[2] = nS; t[3] = nS > 0 && nS <= kSymMax && s_uselev ? s_nlev : -1;
+            t[0] = E; t[1] = nsh; t[2] = nS; t[3] = npk;
         }
         if (s_bad) set_status(&ctl->status, kDevNotSpd);
     }
@@ -2051,7 +1827,8 @@ __device__ void plan_next(const Plan &pl, Ctl *ctl) {
 
 template <typename T, bool MC = false>
 __global__ void __launch_bounds__(512, 1) k_dyn_mark(Mat<T> A, const T *__restrict__ r, Dyn D,
-                                                  Ctl *ctl, int check_done, Cols cl, Plan pl) {
+                                                  Ctl *ctl, int check_done, Cols cl, Plan pl,
+                                                  int fac_max) {
     extern __shared__ unsigned long long dsm_u64[];
     __shared__ int is_last;
     __shared__ unsigned s_tk;
@@ -2077,13 +1854,13 @@ __global__ void __launch_bounds__(512, 1) k_dyn_mark(Mat<T> A, const T *__restri
         double g = A.rn[i];                          // the row's fused chain, formed at set-up
         g = __dadd_rn(g, A.mu);
         D.gdiag[a] = g;
-        if (!(g > 0.0)) { set_status(&ctl->status, kDevNotSpd); g = 1.0; }
+        if (!positive(g)) { set_status(&ctl->status, kDevNotSpd); g = 1.0; }
         if constexpr (sizeof(T) == sizeof(float)) {    // mixed form: rsqrt, products
             const double il = rsqrt(g);
             D.y[a] = ((double)r[rpos<MC>(cl, i)] * il) * il;
         } else {
-            const double l = sqrt(g);
-            D.y[a] = ((double)r[rpos<MC>(cl, i)] / l) / l;
+            const Pivot pv = pivot(g);
+            D.y[a] = pivot_div(pivot_div((double)r[rpos<MC>(cl, i)], pv), pv);
         }
     }
     for (int e = gt; e < E; e += gs) {
@@ -2129,8 +1906,23 @@ __global__ void __launch_bounds__(512, 1) k_dyn_mark(Mat<T> A, const T *__restri
         return;
     }
     __threadfence();
-    dyn_factor<T, MC>(r, K, D, ctl, dsm_u64, cl);
+    dyn_factor<T, MC>(r, K, D, ctl, dsm_u64, cl, fac_max);
     if (threadIdx.x == 0) ctl->ticket = 0;
+}
+
+// Factor and solves of the Gram of a dense A's rows of I (order K, right-hand
+// side r_I), or of the n x n form (order n, right-hand side z0), by one cluster.
+template <typename T>
+__global__ void __launch_bounds__(kCcThreads, 2) k_dense_chol(const T *__restrict__ r, int K, Dyn D, Ctl *ctl,
+                                                              const double *__restrict__ z0) {
+    extern __shared__ unsigned long long dsm_u64[];
+    __shared__ int s_bad;
+    if (ctl->done || ctl->status || ctl->halt) return;
+    if (threadIdx.x == 0) s_bad = 0;
+    cluster_chol_solve<false>(
+        D.g, D.z, K, (double *)dsm_u64, &s_bad, [&](int c) { return z0 ? z0[c] : (double)r[D.I[c]]; },
+        [&](int i, double v) { D.y[i] = v; });
+    if (threadIdx.x == 0 && cluster_rank() == 0 && s_bad) set_status(&ctl->status, kDevNotSpd);
 }
 
 // End of an iteration: trace x, advance, loop condition (one block).
@@ -2157,11 +1949,19 @@ __device__ void end_iteration(const T *x, int n, Ctl *ctl, int use_cond,
 // x += A_I^T y: a column used by one row of I takes its single product; a
 // shared column is summed over its rows in ascending order by the entry that
 // owns it.  The last block clears the column marks and ends the iteration.
+//
+// Rows of I in components too large for one warp are solved first: their packed
+// Gram (D.gc) and right-hand side (D.z), left by k_dyn_mark, are factored by the
+// grid's first cluster (cluster_chol.cuh), which then scatters alone while the
+// other blocks leave.  A launch of its own for the factor would cost every
+// iteration that needs none (2 us of 140 in the steady state of the 2^20
+// power-law system); a scatter by 16 blocks instead of all costs nothing visible.
 template <typename T, bool LOG = false, bool MC = false>
-__global__ void __launch_bounds__(512) k_dyn_scatter(T *x, int n, Dyn D, Ctl *ctl, int count_iter,
-                                                     int use_cond,
-                                                     cudaGraphConditionalHandle hcond, Cols cl) {
-    __shared__ int is_last;
+__global__ void __launch_bounds__(kCcThreads, 2) k_dyn_scatter(T *x, int n, Dyn D, Ctl *ctl, int count_iter,
+                                                               int use_cond,
+                                                               cudaGraphConditionalHandle hcond, Cols cl) {
+    extern __shared__ unsigned long long dsm_u64[];
+    __shared__ int is_last, s_bad;
     if constexpr (MC) {
         ctl += blockIdx.y;
         x += blockIdx.y;
@@ -2173,21 +1973,34 @@ __global__ void __launch_bounds__(512) k_dyn_scatter(T *x, int n, Dyn D, Ctl *ct
         if (count_iter && blockIdx.x == 0) end_iteration<T>(x, n, ctl, use_cond, hcond, ld, grp);
         return;
     }
-    const int E = ctl->dynE, nsh = ctl->dyn_nsh;
+    const int E = ctl->dynE, nsh = ctl->dyn_nsh, nF = ctl->fac_n;
+    int bid = blockIdx.x, nblk = gridDim.x;
+    if (nF) {                                        // the same for every block
+        const int C = (int)cluster_blocks();
+        if (bid >= C) return;
+        nblk = C;
+        if (threadIdx.x == 0) s_bad = 0;
+        cluster_chol_solve<sizeof(T) == sizeof(float)>(
+            D.gc, D.z, nF, (double *)dsm_u64, &s_bad, [&](int c) { return __ldcg(&D.z[c]); },
+            [&](int i, double v) { D.y[D.fidx[i]] = v; });
+        if (threadIdx.x == 0 && bid == 0 && s_bad) set_status(&ctl->status, kDevNotSpd);
+        cluster_sync_all();                          // y and the status
+    }
+    const bool ok = !nF || *(volatile int *)&ctl->status == 0;
     const bool lg = LOG && count_iter;               // log x's changes
     const unsigned ep = *D.epoch;
-    const int gt = blockIdx.x * blockDim.x + threadIdx.x, gs = gridDim.x * blockDim.x;
-    for (int e = gt; e < E; e += gs) {
+    const int gt = bid * blockDim.x + threadIdx.x, gs = nblk * blockDim.x;
+    for (int e = ok ? gt : E; e < E; e += gs) {
         const int c = D.ecol[e];
         if (D.shared[c] != ep) {
-            const T d = Ar<T>::fma(as<T>(D.eval[e]), as<T>(D.y[D.erow[e]]), T(0));
+            const T d = Ar<T>::fma(as<T>(D.eval[e]), as<T>(__ldcg(&D.y[D.erow[e]])), T(0));
             x[(long long)c * ld] = Ar<T>::add(x[(long long)c * ld], d);
             if (lg) inc_log(ctl, c, (double)d);
         } else if ((unsigned)D.skeys[D.segpos[c]] == (unsigned)e) {
             T acc = T(0);
             for (int u = D.segpos[c]; u < nsh && (int)(D.skeys[u] >> 32) == c; ++u) {
                 const unsigned e2 = (unsigned)D.skeys[u];
-                acc = Ar<T>::fma(as<T>(D.eval[e2]), as<T>(D.y[D.erow[e2]]), acc);
+                acc = Ar<T>::fma(as<T>(D.eval[e2]), as<T>(__ldcg(&D.y[D.erow[e2]])), acc);
             }
             x[(long long)c * ld] = Ar<T>::add(x[(long long)c * ld], acc);
             if (lg) inc_log(ctl, c, (double)acc);
@@ -2195,7 +2008,7 @@ __global__ void __launch_bounds__(512) k_dyn_scatter(T *x, int n, Dyn D, Ctl *ct
     }
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) is_last = atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1;
+    if (threadIdx.x == 0) is_last = atomicAdd(&ctl->ticket, 1u) == (unsigned)nblk - 1u;
     __syncthreads();
     if (!is_last) return;
     __threadfence();
@@ -2667,12 +2480,12 @@ __global__ void __launch_bounds__(256) k_dchol_panel_rows(const T *__restrict__ 
         if (dt >= 0) {
             for (int q = jj + 1 + dt; q < w; q += dn) {
                 const double u = Ld[q][jj];
-                if (u != 0.0) Ld[q][jj] = u / l;
+                if (nonzero(u)) Ld[q][jj] = u / l;
             }
             if (dt == dn - 1) zd[jj] = zd[jj] / l;
         } else if (own) {
             v = Lr[jj];
-            if (v != 0.0) v = v / l;
+            if (nonzero(v)) v = v / l;
             Lr[jj] = v;
         }
         __syncthreads();
@@ -2682,19 +2495,19 @@ __global__ void __launch_bounds__(256) k_dchol_panel_rows(const T *__restrict__ 
                 const int jj2 = jj + 1 + q / w, a = q % w;
                 if (a < jj2) continue;
                 const double la = Ld[a][jj], lb = Ld[jj2][jj];
-                if (la != 0.0 && lb != 0.0) Ld[a][jj2] = __fma_rn(-la, lb, Ld[a][jj2]);
+                if (nonzero(la) && nonzero(lb)) Ld[a][jj2] = __fma_rn(-la, lb, Ld[a][jj2]);
             }
             for (int q = jj + 1 + dt; q < w; q += dn) {
                 const double lij = Ld[q][jj];
-                if (lij != 0.0) zd[q] = __fma_rn(-lij, wj, zd[q]);
+                if (nonzero(lij)) zd[q] = __fma_rn(-lij, wj, zd[q]);
             }
         } else if (own) {
 #pragma unroll
             for (int j2 = jj + 1; j2 < kPW; ++j2) {
                 const double bb = Ld[j2][jj];
-                if (j2 < w && v != 0.0 && bb != 0.0) Lr[j2] = __fma_rn(-v, bb, Lr[j2]);
+                if (j2 < w && nonzero(v) && nonzero(bb)) Lr[j2] = __fma_rn(-v, bb, Lr[j2]);
             }
-            if (v != 0.0) zi = __fma_rn(-v, wj, zi);
+            if (nonzero(v)) zi = __fma_rn(-v, wj, zi);
         }
         __syncthreads();
     }
@@ -2744,7 +2557,7 @@ __global__ void __launch_bounds__(256) k_dchol_trail(int K, int j0, Dyn D, Ctl *
     double g = D.g[pidx(a, b)];
     for (int jj = 0; jj < w; ++jj) {
         const double la = La[ta][jj], lb = Lb[tb][jj];
-        if (la != 0.0 && lb != 0.0) g = __fma_rn(-la, lb, g);
+        if (nonzero(la) && nonzero(lb)) g = __fma_rn(-la, lb, g);
     }
     D.g[pidx(a, b)] = g;
 }
@@ -2762,7 +2575,7 @@ __global__ void __launch_bounds__(1024) k_dchol_back(int K, Dyn D, Ctl *ctl) {
         const double zj = z[j];
         for (int i = tid; i < j; i += blockDim.x) {
             const double lji = D.g[pidx(j, i)];
-            if (lji != 0.0) z[i] = __fma_rn(-lji, zj, z[i]);
+            if (nonzero(lji)) z[i] = __fma_rn(-lji, zj, z[i]);
         }
         __syncthreads();
     }
@@ -3397,15 +3210,14 @@ __global__ void __launch_bounds__(256) k_mr_outer_update(double *__restrict__ x,
 static size_t collect_smem_bytes() { return (size_t)kEqCap * (8 + 4) + (size_t)kMaxDynRows * 4; }
 static size_t factor_smem_bytes() {
     return (size_t)(kShCap + kPairCap) * 8 + (size_t)kMaxDynRows * 8 + (size_t)kGPack * 8 +
-           (size_t)2 * kSymMax * kSymW * 4 + (size_t)(3 * kSymMax + 2) * 2 + (size_t)(kSymMax + 2) * 4 +
-           (size_t)kMaxDynRows * (2 + 2 + 1 + 1 + 1) + 64;
+           (size_t)kMaxDynRows * (3 * 2 + 1 + 1 + 1) + 64;
 }
 
 static Dyn dyn_bufs(rorbk_ctx *h) {
     return Dyn{h->dyn.I, h->dyn.estart, h->dyn.gdiag, h->dyn.y, h->dyn.ecol, h->dyn.eval,
                h->dyn.erow, h->dyn.ecap, h->dyn.owner, h->dyn.shared, h->dyn.segpos,
                h->dyn.epoch, h->dyn.raw, h->dyn.skeys, h->dyn.pkeys, h->dyn.pcap, h->dyn.g,
-               h->K, (int)h->n, h->dyn.skcap};
+               h->dyn.gc, h->dyn.z, h->dyn.fidx, h->K, (int)h->n, h->dyn.skcap};
 }
 
 // The sparse path's plan of the next draws (the dense path samples its own).
@@ -3431,7 +3243,11 @@ int grid_topk(rorbk_ctx *h) {
 }
 int grid_collect(rorbk_ctx *h) { return tuned(h->tune.collect, grid_topk(h) / 2); }
 int grid_mark(rorbk_ctx *h) { return tuned(h->tune.mark, h->num_sms / std::max(1, h->nr)); }
-int grid_scatter(rorbk_ctx *h) { return tuned(h->tune.scatter, 2 * h->num_sms / std::max(1, h->nr)); }
+// (about one block per SM, in whole clusters)
+int grid_scatter(rorbk_ctx *h) {
+    const int C = std::max(1, h->dyn.cluster);
+    return tuned(h->tune.scatter, std::max(1, h->num_sms / std::max(1, h->nr) / C) * C);
+}
 
 int residual_grid(rorbk_ctx *h) {
     int per_sm = 0, per_sm32 = 0;
@@ -3491,6 +3307,16 @@ int mres_grid(rorbk_ctx *h, int nr, int fp32) {
     return per_sm * h->num_sms;
 }
 
+// Clusters of 16 blocks are above the portable size; the dynamic shared memory
+// holds the panel of the largest order.
+template <typename K>
+static void configure_cluster(K *kernel) {
+    size_t sm = 0;
+    for (int C = 1; C <= kCcMaxCluster; C *= 2) sm = std::max(sm, cc_smem_bytes(cc_max_order(C), C));
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
+
 void configure_kernels() {
     cudaFuncSetAttribute(k_static<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)static_smem_bytes<double>());
@@ -3516,6 +3342,14 @@ void configure_kernels() {
                          (int)factor_smem_bytes());
     cudaFuncSetAttribute(k_dyn_mark<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)factor_smem_bytes());
+    configure_cluster(k_dyn_scatter<double, false, false>);
+    configure_cluster(k_dyn_scatter<float, false, false>);
+    configure_cluster(k_dyn_scatter<double, true, false>);
+    configure_cluster(k_dyn_scatter<float, true, false>);
+    configure_cluster(k_dyn_scatter<double, false, true>);
+    configure_cluster(k_dyn_scatter<float, false, true>);
+    configure_cluster(k_dense_chol<double>);
+    configure_cluster(k_dense_chol<float>);
     cudaFuncSetAttribute(k_dyn_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gram_tc_smem());
     cudaFuncSetAttribute(k_sd_rows_tiled<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)sd_rows_smem<double>());
@@ -3572,6 +3406,84 @@ void launch_dense_gram(rorbk_ctx *h, Ctl *ctl, int tensor_cores) {
     }
 }
 
+// A launch in clusters of C blocks.
+template <typename... A, typename... B>
+static cudaError_t cluster_launch(cudaStream_t st, void (*kernel)(A...), dim3 grid, int C, size_t smem, B... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kCcThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)C;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// Blocks of the cluster that factors a Gram of order up to K (0: none is
+// needed or none can be resident).  Measured at order 256: 344 us with 16
+// blocks, 393 us with 8 (the trailing updates); at order 100 both take 127 us,
+// so 8 serve orders up to 128 and a block of columns, whose clusters run side
+// by side.  Orders up to 64 have one small trailing update: 4 blocks.
+int chol_cluster_blocks(rorbk_ctx *h) {
+    const bool dense = h->format == RORBK_FORMAT_DENSE || h->K >= h->n;
+    const int K = h->K >= h->n ? (int)h->n : h->K;
+    if (!dense && K <= kCompMax) return 0;
+    const bool half = K <= 128 || (h->nr && K <= cc_max_order(8));
+    for (int C = K <= 64 ? 4 : half ? 8 : kCcMaxCluster; C >= 1; C /= 2) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(C);
+        cfg.blockDim = dim3(kCcThreads);
+        cfg.dynamicSmemBytes = cc_smem_bytes(std::min(K, cc_max_order(C)), C);
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)C;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, k_dyn_scatter<double, false, true>, &cfg);
+        if (e == cudaSuccess && n > 0) return C;
+        cudaGetLastError();
+    }
+    return 0;
+}
+// The largest order the handle's cluster factors.
+static int fac_max(rorbk_ctx *h) { return h->dyn.cluster ? cc_max_order(h->dyn.cluster) : 0; }
+
+// Factor and solves of the dense Gram of order K in D.g: one cluster up to its
+// largest order, above it the grid-wide panels (a trailing update of that
+// size wants every SM).
+template <typename T>
+static void launch_dense_chol(rorbk_ctx *h, const T *r, int K, const double *z0, Ctl *ctl) {
+    if (K <= fac_max(h)) {
+        const int C = h->dyn.cluster;
+        cluster_launch(h->stream, k_dense_chol<T>, dim3(C), C, cc_smem_bytes(K, C), r, K, dyn_bufs(h), ctl, z0);
+        return;
+    }
+    for (int j0 = 0; j0 < K; j0 += kPW) {
+        const int below = K - j0 - std::min(kPW, K - j0);
+        k_dchol_panel_rows<T><<<std::max(1, (below + 31) / 32), 256, 0, h->stream>>>(r, K, j0, dyn_bufs(h), ctl, z0);
+        const int rest = K - std::min(K, j0 + kPW), tt = (rest + 15) / 16;
+        if (rest > 0) k_dchol_trail<<<tt * (tt + 1) / 2, 256, 0, h->stream>>>(K, j0, dyn_bufs(h), ctl);
+    }
+    k_dchol_back<<<1, 1024, 0, h->stream>>>(K, dyn_bufs(h), ctl);
+}
+
+// The sparse dynamic update's factor of large components and its scatter:
+// whole clusters (the grid is rounded up to them).
+template <typename T, bool LOG, bool MC>
+static void launch_dyn_scatter(rorbk_ctx *h, T *x, Ctl *ctl, int count_iter, int use_cond, unsigned long long hcond,
+                               const Cols &cl) {
+    const int C = std::max(1, h->dyn.cluster), g = (grid_scatter(h) + C - 1) / C * C;
+    const size_t smem = h->dyn.cluster ? cc_smem_bytes(std::min(h->K, cc_max_order(C)), C) : 0;
+    cluster_launch(h->stream, k_dyn_scatter<T, LOG, MC>, dim3(g, std::max(1, h->nr)), C, smem, x, (int)h->n,
+                   dyn_bufs(h), ctl, count_iter, use_cond, (cudaGraphConditionalHandle)hcond, cl);
+}
+
 template <typename T>
 static void launch_dynamic_tail(rorbk_ctx *h, const T *r, T *x, Ctl *ctl, int check_done,
                                 int count_iter, int use_cond, unsigned long long hcond, int inc = 0) {
@@ -3587,14 +3499,7 @@ static void launch_dynamic_tail(rorbk_ctx *h, const T *r, T *x, Ctl *ctl, int ch
         k_dynw_gram<<<(int)std::max<long long>(1, std::min<long long>(8LL * h->num_sms, (np + 255) / 256)), 256, 0,
                       h->stream>>>(dw, n, K, h->mu, dyn_bufs(h), ctl);
         k_dynw_rhs<T><<<std::max(1, (n + 63) / 64), 64, 0, h->stream>>>(dw, r, n, K, dyn_bufs(h), hz, ctl);
-        for (int j0 = 0; j0 < n; j0 += kPW) {
-            const int below = n - j0 - std::min(kPW, n - j0);
-            k_dchol_panel_rows<T><<<std::max(1, (below + 31) / 32), 256, 0, h->stream>>>(r, n, j0, dyn_bufs(h),
-                                                                                       ctl, hz);
-            const int rest = n - std::min(n, j0 + kPW), tt = (rest + 15) / 16;
-            if (rest > 0) k_dchol_trail<<<tt * (tt + 1) / 2, 256, 0, h->stream>>>(n, j0, dyn_bufs(h), ctl);
-        }
-        k_dchol_back<<<1, 1024, 0, h->stream>>>(n, dyn_bufs(h), ctl);
+        launch_dense_chol<T>(h, r, n, hz, ctl);
         const int g = std::max(1, std::min(8 * h->num_sms, (n + 63) / 64));
         k_dyn_dense_scatter<T><<<g, 64, 0, h->stream>>>(h->val, h->val32, x, n, K, dyn_bufs(h), ctl, count_iter,
                                                           use_cond, (cudaGraphConditionalHandle)hcond, 1);
@@ -3604,15 +3509,7 @@ static void launch_dynamic_tail(rorbk_ctx *h, const T *r, T *x, Ctl *ctl, int ch
         const int K = h->K;
         // mixed precision: the TF32 tensor-core Gram (FP32 partials added in FP64)
         launch_dense_gram(h, ctl, sizeof(T) == sizeof(float) && h->gram_part);
-        for (int j0 = 0; j0 < K; j0 += kPW) {
-            const int below = K - j0 - std::min(kPW, K - j0);
-            k_dchol_panel_rows<T><<<std::max(1, (below + 31) / 32), 256, 0, h->stream>>>(r, K, j0,
-                                                                                       dyn_bufs(h), ctl,
-                                                                                       nullptr);
-            const int rest = K - std::min(K, j0 + kPW), tt = (rest + 15) / 16;
-            if (rest > 0) k_dchol_trail<<<tt * (tt + 1) / 2, 256, 0, h->stream>>>(K, j0, dyn_bufs(h), ctl);
-        }
-        k_dchol_back<<<1, 1024, 0, h->stream>>>(K, dyn_bufs(h), ctl);
+        launch_dense_chol<T>(h, r, K, nullptr, ctl);
         const int g = std::max(1, std::min(8 * h->num_sms, (int)((h->n + 63) / 64)));
         k_dyn_dense_scatter<T><<<g, 64, 0, h->stream>>>(h->val, h->val32, x, (int)h->n, K, dyn_bufs(h),
                                                           ctl, count_iter, use_cond,
@@ -3622,10 +3519,10 @@ static void launch_dynamic_tail(rorbk_ctx *h, const T *r, T *x, Ctl *ctl, int ch
     Mat<T> A = make_mat<T>(h);
     k_dyn_mark<T><<<grid_mark(h), 512, factor_smem_bytes(), h->stream>>>(A, r, dyn_bufs(h), ctl,
                                                                         check_done, one_col((int)h->m),
-                                                                        count_iter ? plan_of(h) : Plan{});
-    (inc ? k_dyn_scatter<T, true> : k_dyn_scatter<T, false>)<<<grid_scatter(h), 512, 0, h->stream>>>(
-        x, (int)h->n, dyn_bufs(h), ctl, count_iter, use_cond, (cudaGraphConditionalHandle)hcond,
-        one_col((int)h->m));
+                                                                        count_iter ? plan_of(h) : Plan{},
+                                                                        fac_max(h));
+    if (inc) launch_dyn_scatter<T, true, false>(h, x, ctl, count_iter, use_cond, hcond, one_col((int)h->m));
+    else launch_dyn_scatter<T, false, false>(h, x, ctl, count_iter, use_cond, hcond, one_col((int)h->m));
 }
 
 template <typename T>
@@ -3738,9 +3635,8 @@ static void launch_mr_iteration_t(rorbk_ctx *h, const T *b, T *x, T *r, Ctl *ctl
     k_topk_collect<T, true><<<dim3(grid_collect(h), nr), 512, collect_smem_bytes(), st>>>(
         r, m, K, h->rowptr, h->in_list, h->eq_list, dyn_bufs(h), ctl, 1, cl);
     k_dyn_mark<T, true><<<dim3(grid_mark(h), nr), 512, factor_smem_bytes(), st>>>(
-        A, r, dyn_bufs(h), ctl, 1, cl, plan_of(h));
-    k_dyn_scatter<T, false, true><<<dim3(grid_scatter(h), nr), 512, 0, st>>>(
-        x, (int)h->n, dyn_bufs(h), ctl, 1, use_cond, (cudaGraphConditionalHandle)hcond, cl);
+        A, r, dyn_bufs(h), ctl, 1, cl, plan_of(h), fac_max(h));
+    launch_dyn_scatter<T, false, true>(h, x, ctl, 1, use_cond, hcond, cl);
 }
 
 void launch_residual_multi(rorbk_ctx *h, int fp32, const void *B, const void *X, void *R) {

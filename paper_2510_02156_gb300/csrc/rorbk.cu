@@ -294,8 +294,14 @@ static rorbk_status alloc_workspace(rorbk_ctx *h) {
         D.skeys = (unsigned long long *)dev_alloc(h, nr * np2 * sizeof(unsigned long long));
         D.pkeys = (unsigned long long *)dev_alloc(h, nr * D.pcap * sizeof(unsigned long long));
         D.g = (double *)dev_alloc(h, nr * ((size_t)h->K * (h->K + 1) / 2) * sizeof(double));
+        D.z = (double *)dev_alloc(h, nr * h->K * sizeof(double));
+        D.fidx = (int *)dev_alloc(h, nr * h->K * sizeof(int));
+        if (h->format == RORBK_FORMAT_CSR)
+            D.gc = (double *)dev_alloc(h, nr * ((size_t)h->K * (h->K + 1) / 2) * sizeof(double));
+        D.cluster = chol_cluster_blocks(h);
         if (!D.I || !D.estart || !D.gdiag || !D.y || !D.ecol || !D.eval || !D.erow || !D.owner ||
-            !D.shared || !D.epoch || !D.segpos || !D.raw || !D.skeys || !D.pkeys || !D.g)
+            !D.shared || !D.epoch || !D.segpos || !D.raw || !D.skeys || !D.pkeys || !D.g || !D.z || !D.fidx ||
+            (h->format == RORBK_FORMAT_CSR && !D.gc))
             return fail(h, RORBK_ERR_OOM, "dynamic-block workspace");
         cudaMemsetAsync(D.owner, 0, nr * n * sizeof(unsigned long long), s);   // epoch 0: never
         cudaMemsetAsync(D.shared, 0, nr * n * sizeof(unsigned), s);
