@@ -58,6 +58,12 @@ template <> __device__ __forceinline__ double wide<double>(float v) { return wid
 template <> __device__ __forceinline__ float wide<float>(float v) { return v; }
 template <typename T> __device__ __forceinline__ T wide(double v) { return (T)v; }
 
+}  // namespace rorbk
+
+#include "dense_rows.cuh"
+
+namespace rorbk {
+
 // VEC values of T in one aligned load (16 bytes at most).
 template <typename T, int VEC>
 struct VecT {
@@ -463,6 +469,7 @@ __global__ void __launch_bounds__(1024, 1) k_static(Mat<T> A, const T *__restric
     if (force_tau < 0 && (ctl->done || ctl->halt)) return;
     const bool lg = LOG && force_tau < 0;            // log x's changes
     const int nst = force_tau >= 0 ? 1 : ctl->n_static;
+    if (l_begin > 0 && l_begin >= nst) return;        // a dense A's updates ran as grid launches
     const int a = threadIdx.x;
     unsigned long long *bar = dsm_u64;                // two mbarriers
     unsigned char *sbase = (unsigned char *)(dsm_u64 + 8);
@@ -708,111 +715,15 @@ __device__ __forceinline__ void hist_add(unsigned *hist, unsigned bin, bool acti
 // column order.  Longest slices come first.  V is the stored value type (an
 // FP32-stored system is read as FP32 and widened exactly).
 // finalize: 1 = convergence test + first radix level (iteration), 2 = ||r||^2
-// only (single-step API).  DN: A is dense, so entry j of a row is in column j
-// and the column indices are not read (x_j is the same for the warp's lanes).
-constexpr int kDnAhead = 8;      // dense residual: 16-byte loads per lane in flight
+// only (single-step API), 3 = convergence test only.
 
-// (a dense A: three blocks per SM, so that each lane keeps kDnAhead loads in
-// flight without spilling)
-template <typename T, typename V, bool DN = false>
-__global__ void __launch_bounds__(256, DN ? 3 : 4) k_residual(Mat<T> A, const T *__restrict__ b,
-                                                  const T *__restrict__ x, T *__restrict__ r,
-                                                  double *partials, unsigned *hist1, Ctl *ctl,
-                                                  int finalize) {
-    __shared__ unsigned hist[kHistBins];
+// The end of a residual pass, by the whole block: its share of the first radix
+// histogram and of ||r||^2; the last block adds the shares in block order, runs
+// the convergence test and selects the first radix bin.
+__device__ __forceinline__ void residual_finish(double rr, unsigned *hist, double *partials, unsigned *hist1, Ctl *ctl,
+                                                int K, int finalize) {
     __shared__ double red[32];
     __shared__ int is_last;
-    if ((finalize == 1 || finalize == 3) && (ctl->done || ctl->halt)) return;
-    if (finalize == 1 && ctl->inc && !ctl->inc_full) return;   // r came from the change log
-    const V *__restrict__ val = sell_values<V, T>(A);
-    const int lane = threadIdx.x & 31;
-    const int nwb = blockDim.x >> 5;
-    for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) hist[i] = 0u;
-    double rr = 0.0;
-    __syncthreads();
-    // One resident wave of blocks; slices (longest first) are dealt to the
-    // warps in snake order, warps of consecutive ids sitting on different SMs,
-    // so every warp gets a mix of long and short slices.
-    const int W = gridDim.x * nwb;
-    const int g = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-    for (int rnd = 0;; ++rnd) {
-        const int sl = rnd * W + ((rnd & 1) ? W - 1 - g : g);
-        if (sl >= A.nslices) break;
-        const long long base = A.sptr[sl] + lane;
-        const int L = A.slen[sl];
-        const int slot = sl * 32 + lane;
-        const int row = A.srow[slot], len = A.srlen[slot];
-        T acc = T(0);
-        if constexpr (DN) {
-            // a dense A: entry j of lane l is at 32 VW (j / VW) + VW l + j % VW
-            // of the slice, so each load brings VW consecutive entries of the
-            // lane's own row (16 bytes); kDnAhead such loads are in flight while
-            // the chain runs over the previous ones, columns ascending as ever
-            constexpr int VW = 16 / sizeof(V);
-            const V *vb = val + A.sptr[sl] + VW * lane;
-            VecT<V, VW> vq[kDnAhead];
-#pragma unroll
-            for (int q = 0; q < kDnAhead; ++q)
-                if (q * VW < len) vq[q] = vload<V, VW, true>(vb + 32LL * VW * q);
-            for (int q0 = 0; q0 * VW < L; q0 += kDnAhead) {
-                VecT<V, VW> vc[kDnAhead];
-#pragma unroll
-                for (int q = 0; q < kDnAhead; ++q) vc[q] = vq[q];
-#pragma unroll
-                for (int q = 0; q < kDnAhead; ++q)
-                    if ((q0 + kDnAhead + q) * VW < len)
-                        vq[q] = vload<V, VW, true>(vb + 32LL * VW * (q0 + kDnAhead + q));
-#pragma unroll
-                for (int q = 0; q < kDnAhead; ++q)
-#pragma unroll
-                    for (int u = 0; u < VW; ++u) {
-                        const int j = (q0 + q) * VW + u;
-                        if (j < len) acc = Ar<T>::fma(wide<T>(vc[q].v[u]), x[j], acc);
-                    }
-            }
-        } else {
-        // software pipeline, 8 deep: the x gathers of chunk k and the index /
-        // value loads of chunk k+1 are in flight while chunk k's chain runs
-        int cn[8];
-        V vn[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const bool in = u < len;
-            const long long d = base + 32LL * u;
-            cn[u] = in ? A.scol[d] : 0;
-            vn[u] = in ? val[d] : V(0);
-        }
-        for (int c0 = 0; c0 < L; c0 += 8) {
-            T xv[8];
-            V vc[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                xv[u] = c0 + u < len ? x[cn[u]] : T(0);
-                vc[u] = vn[u];
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int j = c0 + 8 + u;
-                const bool in = j < len;
-                const long long d = base + 32LL * j;
-                cn[u] = in ? A.scol[d] : 0;
-                vn[u] = in ? val[d] : V(0);
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (c0 + u < len) acc = Ar<T>::fma(wide<T>(vc[u]), xv[u], acc);
-        }
-        }
-        const bool act = row >= 0;
-        unsigned bin = 0;
-        if (act) {
-            const T ri = Ar<T>::sub(b[row], acc);
-            r[row] = ri;
-            rr = __fma_rn((double)ri, (double)ri, rr);
-            bin = (unsigned)(abs_key(ri) >> 52);
-        }
-        if (finalize == 1) hist_add(hist, bin, act);
-    }
     __syncthreads();
     if (finalize == 1)
         for (int i = threadIdx.x; i < kHistBins; i += blockDim.x)
@@ -856,12 +767,126 @@ __global__ void __launch_bounds__(256, DN ? 3 : 4) k_residual(Mat<T> A, const T 
     if (finalize == 1) {
         int bin, above;
         if (!stop) {
-            select_bin(hist1, A.K, &bin, &above);
+            select_bin(hist1, K, &bin, &above);
             if (threadIdx.x == 0) { ctl->sel1 = bin; ctl->above1 = above; }
         } else {
             for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) hist1[i] = 0u;
         }
     }
+}
+
+template <typename T, typename V>
+__global__ void __launch_bounds__(256, 4) k_residual(Mat<T> A, const T *__restrict__ b,
+                                                  const T *__restrict__ x, T *__restrict__ r,
+                                                  double *partials, unsigned *hist1, Ctl *ctl,
+                                                  int finalize) {
+    __shared__ unsigned hist[kHistBins];
+    if ((finalize == 1 || finalize == 3) && (ctl->done || ctl->halt)) return;
+    if (finalize == 1 && ctl->inc && !ctl->inc_full) return;   // r came from the change log
+    const V *__restrict__ val = sell_values<V, T>(A);
+    const int lane = threadIdx.x & 31;
+    const int nwb = blockDim.x >> 5;
+    for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) hist[i] = 0u;
+    double rr = 0.0;
+    __syncthreads();
+    // One resident wave of blocks; slices (longest first) are dealt to the
+    // warps in snake order, warps of consecutive ids sitting on different SMs,
+    // so every warp gets a mix of long and short slices.
+    const int W = gridDim.x * nwb;
+    const int g = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    for (int rnd = 0;; ++rnd) {
+        const int sl = rnd * W + ((rnd & 1) ? W - 1 - g : g);
+        if (sl >= A.nslices) break;
+        const long long base = A.sptr[sl] + lane;
+        const int L = A.slen[sl];
+        const int slot = sl * 32 + lane;
+        const int row = A.srow[slot], len = A.srlen[slot];
+        T acc = T(0);
+        // software pipeline, 8 deep: the x gathers of chunk k and the index /
+        // value loads of chunk k+1 are in flight while chunk k's chain runs
+        int cn[8];
+        V vn[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const bool in = u < len;
+            const long long d = base + 32LL * u;
+            cn[u] = in ? A.scol[d] : 0;
+            vn[u] = in ? val[d] : V(0);
+        }
+        for (int c0 = 0; c0 < L; c0 += 8) {
+            T xv[8];
+            V vc[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                xv[u] = c0 + u < len ? x[cn[u]] : T(0);
+                vc[u] = vn[u];
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int j = c0 + 8 + u;
+                const bool in = j < len;
+                const long long d = base + 32LL * j;
+                cn[u] = in ? A.scol[d] : 0;
+                vn[u] = in ? val[d] : V(0);
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (c0 + u < len) acc = Ar<T>::fma(wide<T>(vc[u]), xv[u], acc);
+        }
+        const bool act = row >= 0;
+        unsigned bin = 0;
+        if (act) {
+            const T ri = Ar<T>::sub(b[row], acc);
+            r[row] = ri;
+            rr = __fma_rn((double)ri, (double)ri, rr);
+            bin = (unsigned)(abs_key(ri) >> 52);
+        }
+        if (finalize == 1) hist_add(hist, bin, act);
+    }
+    residual_finish(rr, hist, partials, hist1, ctl, A.K, finalize);
+}
+
+// r = b - A x for a dense A: one warp per 32 consecutive rows on its own ring of
+// stages (dense_rows.cuh), row-major values, one block per SM.  W warps per block
+// run chains, with 24 / W stages each: as many as there are groups of rows per
+// SM, so that a short A (few chains) keeps more bytes of each in flight.
+constexpr int kDrStages = 24;       // stages per block, about 9 KB each
+
+template <typename T, typename V>
+__host__ __device__ constexpr size_t dense_res_smem() { return (size_t)kDrStages * DenseStage<T, V>::bytes; }
+
+template <typename T, typename V, int W>
+__global__ void __launch_bounds__(256, 1) k_residual_dense(const V *__restrict__ val, int m, int n, int K,
+                                                          const T *__restrict__ b, const T *__restrict__ x,
+                                                          T *__restrict__ r, double *partials, unsigned *hist1,
+                                                          Ctl *ctl, int finalize) {
+    extern __shared__ __align__(16) unsigned char dr_ring[];
+    __shared__ unsigned hist[kHistBins];
+    if ((finalize == 1 || finalize == 3) && (ctl->done || ctl->halt)) return;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) hist[i] = 0u;
+    __syncthreads();
+    double rr = 0.0;
+    constexpr int ST = kDrStages / W;
+    if (wid < W) {
+        const bool vec = ((long long)n * (int)sizeof(V)) % 16 == 0;
+        const int nsl = (m + 31) / 32, Wt = gridDim.x * W, g = wid * gridDim.x + blockIdx.x;
+        unsigned char *ring = dr_ring + (size_t)wid * ST * DenseStage<T, V>::bytes;
+        for (int sl = g; sl < nsl; sl += Wt) {
+            const int row0 = sl * 32, rows = min(32, m - row0);
+            const T acc = dense_chain<T, V, ST>(val + (long long)row0 * n, rows, n, x, ring, vec);
+            const bool act = lane < rows;
+            unsigned bin = 0;
+            if (act) {
+                const T ri = Ar<T>::sub(b[row0 + lane], acc);
+                r[row0 + lane] = ri;
+                rr = __fma_rn((double)ri, (double)ri, rr);
+                bin = (unsigned)(abs_key(ri) >> 52);
+            }
+            if (finalize == 1) hist_add(hist, bin, act);
+        }
+    }
+    residual_finish(rr, hist, partials, hist1, ctl, K, finalize);
 }
 
 // Incremental residual, first kernel: r -= A dx from the iteration's change log,
@@ -1300,15 +1325,54 @@ __device__ void publish_rows(const int *rowptr, const int *sI, int K, Dyn D, Ctl
     }
 }
 
+// What the dynamic update (sparse A) or the top-K pass (dense A) needs to form the next iteration's draws ahead of
+// them (cdf == nullptr: not formed).
+struct Plan {
+    const double *cdf;
+    int k;
+    const int *off, *s_ptr, *blk_nz;
+    const long long *w_ptr;
+};
+
+// The next iteration's draws and their blocks' ranges, which depend on
+// neither x nor r, formed by one block of a pass while its last block works
+// alone (so that the next sampled updates start at once).  The
+// residual-weighted draws are formed by k_static itself.
+__device__ void plan_next(const Plan &pl, Ctl *ctl) {
+    if (ctl->weighted || ctl->n_static > kPreDraws) return;
+    __shared__ int taus[64], s_cnt[64];
+    __shared__ double s_target[64];
+    const int nst = ctl->n_static;
+    const long long next = ctl->iter_base + ctl->iter + 1;
+    sample_blocks_block<8>(pl.cdf, pl.k, ctl->seed, ctl->sysid, (uint64_t)next, nst, s_target, s_cnt, taus);
+    const int a = threadIdx.x;
+    if (a < nst) {
+        const int tau = taus[a];
+        ctl->pre_tau[a] = tau;
+        ctl->pre_r0[a] = pl.off[tau];
+        ctl->pre_s[a] = pl.off[tau + 1] - pl.off[tau];
+        ctl->pre_sb[a] = pl.s_ptr[tau];
+        ctl->pre_nS[a] = pl.s_ptr[tau + 1] - pl.s_ptr[tau];
+        ctl->pre_wb[a] = pl.w_ptr[tau];
+        ctl->pre_p0[a] = pl.blk_nz[tau];
+        ctl->pre_pend[a] = pl.blk_nz[tau + 1];
+    }
+    __syncthreads();
+    if (a == 0) {
+        __threadfence();
+        ctl->pre_it = next + 1;
+    }
+}
+
 // Rows above the 22-bit threshold and the candidates on it; the last block
 // completes the exact top-K set and publishes it.
 template <typename T, bool MC = false>
 __global__ void __launch_bounds__(512) k_topk_collect(const T *__restrict__ r, int m, int K,
                                                       const int *rowptr, int *in_list,
                                                       int *eq_list, Dyn D, Ctl *ctl,
-                                                      int check_done, Cols cl) {
+                                                      int check_done, Cols cl, Plan pl) {
     extern __shared__ unsigned long long dsm_u64[];
-    __shared__ int is_last;
+    __shared__ int is_last, is_first;
     if constexpr (MC) {
         ctl += blockIdx.y;
         r += blockIdx.y * cl.rs;
@@ -1345,9 +1409,16 @@ __global__ void __launch_bounds__(512) k_topk_collect(const T *__restrict__ r, i
     }
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) is_last = atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1;
+    if (threadIdx.x == 0) {
+        const unsigned tk = atomicAdd(&ctl->ticket, 1u);
+        is_last = tk == gridDim.x - 1;
+        is_first = tk == 0;
+    }
     __syncthreads();
-    if (!is_last) return;
+    if (!is_last) {
+        if (is_first && pl.cdf) plan_next(pl, ctl);
+        return;
+    }
     __threadfence();
     unsigned long long *skey = dsm_u64;
     int *sidx = (int *)(skey + kEqCap);
@@ -1786,45 +1857,6 @@ __device__ void dyn_factor(const T *__restrict__ r, int K, Dyn D, Ctl *ctl,
 
 // Gathers the nonzeros of A_I (row order), marks each column's lowest entry
 // and entry count, forms ||A_i||^2 + mu; the last block factors.
-// What the dynamic update needs to form the next iteration's draws ahead of
-// them (cdf == nullptr: not formed).
-struct Plan {
-    const double *cdf;
-    int k;
-    const int *off, *s_ptr, *blk_nz;
-    const long long *w_ptr;
-};
-
-// The next iteration's draws and their blocks' ranges, which depend on
-// neither x nor r, formed by one block of the dynamic update while its last
-// block factors (so that the next sampled updates start at once).  The
-// residual-weighted draws are formed by k_static itself.
-__device__ void plan_next(const Plan &pl, Ctl *ctl) {
-    if (ctl->weighted || ctl->n_static > kPreDraws) return;
-    __shared__ int taus[64], s_cnt[64];
-    __shared__ double s_target[64];
-    const int nst = ctl->n_static;
-    const long long next = ctl->iter_base + ctl->iter + 1;
-    sample_blocks_block<8>(pl.cdf, pl.k, ctl->seed, ctl->sysid, (uint64_t)next, nst, s_target, s_cnt, taus);
-    const int a = threadIdx.x;
-    if (a < nst) {
-        const int tau = taus[a];
-        ctl->pre_tau[a] = tau;
-        ctl->pre_r0[a] = pl.off[tau];
-        ctl->pre_s[a] = pl.off[tau + 1] - pl.off[tau];
-        ctl->pre_sb[a] = pl.s_ptr[tau];
-        ctl->pre_nS[a] = pl.s_ptr[tau + 1] - pl.s_ptr[tau];
-        ctl->pre_wb[a] = pl.w_ptr[tau];
-        ctl->pre_p0[a] = pl.blk_nz[tau];
-        ctl->pre_pend[a] = pl.blk_nz[tau + 1];
-    }
-    __syncthreads();
-    if (a == 0) {
-        __threadfence();
-        ctl->pre_it = next + 1;
-    }
-}
-
 template <typename T, bool MC = false>
 __global__ void __launch_bounds__(512, 1) k_dyn_mark(Mat<T> A, const T *__restrict__ r, Dyn D,
                                                   Ctl *ctl, int check_done, Cols cl, Plan pl,
@@ -2072,88 +2104,73 @@ __global__ void __launch_bounds__(1024) k_wcdf(const double *__restrict__ w, int
 }
 
 // ---- the static updates of a dense A --------------------------------------
-// A block of a dense A (s rows of n entries) is far larger than a stage, and
-// one block of threads reading it row by row runs short of loads in flight.
-// Each of the first kDenseStatic updates of an iteration therefore runs as
-// three grid launches with the arithmetic of k_static's direct path: the
-// block's residual (one lane per row, the row's chain in column order),
-// y = W_tau r_tau, and x += A_tau^T y (one thread per column segment, rows
-// ascending).  Every launch draws the same tau from the Philox stream.
+// A block of a dense A (s rows of n entries) is far larger than a stage of
+// k_static, and one block of threads reading it row by row runs short of loads
+// in flight.  Each of the first kDenseStatic updates of an iteration therefore
+// runs as three grid launches with the arithmetic of k_static's direct path:
+// the block's residual (one lane per row, the row's chain in column order),
+// y = W_tau r_tau, and x += A_tau^T y (one thread per column, rows ascending).
 constexpr int kDenseStatic = 3;
 
-// The block's residual r_tau = b_tau - A_tau x, tiled for load parallelism:
-// grid block g takes rows 32g..32g+31 of the block.  Its 256 threads copy a
-// tile of those rows' next kSdCols columns (coalesced along the columns) into
-// shared memory, transposed, while lane a of warp 0 runs row a's chain
-// acc = fma(a_aj, x_j, acc) over the previous tile, columns ascending -- the
-// operations of k_static's direct path in the same order.
-constexpr int kSdCols = 256;     // = blockDim: thread t copies column t of each row
-
+// Draw l of this iteration: the one formed ahead by the previous iteration's
+// top-K pass, or searched in the running sum.
 template <typename T>
-__host__ __device__ constexpr size_t sd_rows_smem() { return ((size_t)kSdCols * 33 + kSdCols) * sizeof(T); }
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_sd_rows_tiled(Mat<T> A, const T *__restrict__ b,
-                                                      const T *__restrict__ x, T *rloc, Ctl *ctl,
-                                                      int l) {
-    extern __shared__ unsigned long long sd_dsm[];
-    T *tile = (T *)sd_dsm;                        // [kSdCols][33]: column-major tile
-    T *xs = tile + kSdCols * 33;                  // [kSdCols]
-    __shared__ long long rbase[32];
-    if (ctl->done || ctl->halt || l >= ctl->n_static) return;
+__device__ __forceinline__ int drawn_block(const Mat<T> &A, const Ctl *ctl, int l) {
     const long long it = ctl->iter_base + ctl->iter;
-    const int tau = sample_block(ctl->scdf ? ctl->scdf : A.cdf, A.k, ctl->seed, ctl->sysid, (uint64_t)it, (uint64_t)l);
-    if (blockIdx.x == 0 && threadIdx.x == 0 && ctl->tr_tau && ctl->iter < ctl->trace_cap)
+    if (ctl->pre_it == it + 1 && ctl->n_static <= kPreDraws) return ctl->pre_tau[l];
+    return sample_block(ctl->scdf ? ctl->scdf : A.cdf, A.k, ctl->seed, ctl->sysid, (uint64_t)it, (uint64_t)l);
+}
+
+// The block's residual r_tau = b_tau - A_tau x: grid block g is one warp that
+// takes rows 32g .. 32g + 31 on a ring of 8 stages (dense_rows.cuh: seven stages
+// of FP32 links take longer than a load).  256 x 2,048: 95 -> 93 us in FP64
+// (2,048 links of 64 cycles are 66), 37 -> 22 us in FP32; 256 x 100,000 in FP32:
+// 1,537 -> 735 us.
+constexpr int kSdStages = 8;
+template <typename T>
+__host__ __device__ constexpr size_t sd_rows_smem() { return (size_t)kSdStages * DenseStage<T, T>::bytes; }
+
+template <typename T>
+__global__ void __launch_bounds__(32) k_sd_rows(Mat<T> A, const T *__restrict__ b, const T *__restrict__ x, T *rloc,
+                                                Ctl *ctl, int l) {
+    extern __shared__ __align__(16) unsigned char dr_ring[];
+    if (ctl->done || ctl->halt || l >= ctl->n_static) return;
+    const int tau = drawn_block(A, ctl, l), lane = threadIdx.x;
+    if (blockIdx.x == 0 && lane == 0 && ctl->tr_tau && ctl->iter < ctl->trace_cap)
         ctl->tr_tau[ctl->iter * ctl->n_static + l] = tau;
     const int r0 = A.off[tau], s = A.off[tau + 1] - r0;
     const int row0 = blockIdx.x * 32;
     if (row0 >= s) return;
-    const int rows = min(32, s - row0), n = A.n, tid = threadIdx.x;
-    if (tid < 32) rbase[tid] = tid < rows ? (long long)A.rowptr[r0 + row0 + tid] : 0;
-    __syncthreads();
-    T pre[32];
-#pragma unroll
-    for (int u = 0; u < 32; ++u) pre[u] = (u < rows && tid < n) ? A.val[rbase[u] + tid] : T(0);
-    T acc = T(0);
-    for (int c0 = 0; c0 < n; c0 += kSdCols) {
-#pragma unroll
-        for (int u = 0; u < 32; ++u) tile[tid * 33 + u] = pre[u];
-        xs[tid] = c0 + tid < n ? x[c0 + tid] : T(0);
-        __syncthreads();
-        const int c1 = c0 + kSdCols;
-        if (c1 < n) {                             // next tile in flight during the chain
-#pragma unroll
-            for (int u = 0; u < 32; ++u) pre[u] = (u < rows && c1 + tid < n) ? A.val[rbase[u] + c1 + tid] : T(0);
-        }
-        if (tid < rows) {
-            const int jn = min(kSdCols, n - c0);
-            for (int j = 0; j < jn; ++j) acc = Ar<T>::fma(tile[j * 33 + tid], xs[j], acc);
-        }
-        __syncthreads();
-    }
-    if (tid < rows) rloc[row0 + tid] = Ar<T>::sub(b[r0 + row0 + tid], acc);
+    const int rows = min(32, s - row0);
+    const bool vec = ((long long)A.n * (int)sizeof(T)) % 16 == 0;
+    const T bi = lane < rows ? b[r0 + row0 + lane] : T(0);
+    const T acc = dense_chain<T, T, kSdStages>(A.val + (long long)(r0 + row0) * A.n, rows, A.n, x, dr_ring, vec);
+    if (lane < rows) rloc[row0 + lane] = Ar<T>::sub(bi, acc);
 }
 
+// y = W_tau r_tau, one warp per 32 rows.  W_tau is stored full and symmetric, so
+// a lane reads its row down the column: the warp's loads are coalesced, and the
+// rows' warps sit on different SMs.  256 rows: 45 -> 22 us (FP64; 256 links of 64
+// cycles are 8), 46 -> 17 us (FP32).
 template <typename T>
-__global__ void __launch_bounds__(1024) k_sd_apply(Mat<T> A, const T *__restrict__ rloc, T *y,
-                                                   Ctl *ctl, int l) {
+__global__ void __launch_bounds__(32) k_sd_apply(Mat<T> A, const T *__restrict__ rloc, T *y, Ctl *ctl, int l) {
+    __shared__ T rs[kMaxBlockRows];
     if (ctl->done || ctl->halt || l >= ctl->n_static) return;
-    const long long it = ctl->iter_base + ctl->iter;
-    const int tau = sample_block(ctl->scdf ? ctl->scdf : A.cdf, A.k, ctl->seed, ctl->sysid, (uint64_t)it, (uint64_t)l);
+    const int tau = drawn_block(A, ctl, l);
     if (A.wood_ptr && A.wood_ptr[tau] >= 0) return;   // the s >= n form needs no W r
     const int r0 = A.off[tau], s = A.off[tau + 1] - r0;
-    const int a = threadIdx.x;
+    const int a = blockIdx.x * 32 + threadIdx.x;
+    if (blockIdx.x * 32 >= s) return;
+    const int sb = A.s_ptr[tau], nS = A.s_ptr[tau + 1] - sb;
+    for (int q = threadIdx.x; q < nS; q += 32) rs[q] = rloc[A.s_idx[sb + q]];
+    __syncwarp();
     if (a >= s) return;
     const int pos = A.s_pos[r0 + a];
     if (pos < 0) {
         y[a] = Ar<T>::fma(A.w_diag[r0 + a], rloc[a], T(0));
     } else {
-        const int sb = A.s_ptr[tau], nS = A.s_ptr[tau + 1] - sb;
-        const T *Wr = A.w_ss + A.w_ptr[tau] + (long long)pos * nS;
-        T acc2 = T(0);
-#pragma unroll 8
-        for (int q = 0; q < nS; ++q) acc2 = Ar<T>::fma(Wr[q], rloc[A.s_idx[sb + q]], acc2);
-        y[a] = acc2;
+        const T *Wc = A.w_ss + A.w_ptr[tau] + pos;
+        y[a] = column_chain<T>(nS, rs, [&](int q) { return __ldg(Wc + (long long)q * nS); });
     }
 }
 
@@ -2163,26 +2180,24 @@ __global__ void __launch_bounds__(1024) k_sd_apply(Mat<T> A, const T *__restrict
 // same chain with loads coalesced across the threads' columns.  For a block in
 // the s >= n form it forms g_c = sum over the rows of a_ac r_a into y instead
 // (k_sd_wood applies V).
+constexpr int kSdThreads = 64;      // column-parallel passes: more SMs share the FP64 chains of a narrow system
+
 template <typename T>
-__global__ void __launch_bounds__(256) k_sd_scatter(Mat<T> A, const T *__restrict__ rl, T *y, T *x,
-                                                    Ctl *ctl, int l) {
-    __shared__ long long rbase[kMaxBlockRows];
+__global__ void __launch_bounds__(kSdThreads) k_sd_scatter(Mat<T> A, const T *__restrict__ rl, T *y, T *x, Ctl *ctl,
+                                                           int l) {
+    __shared__ T ys[kMaxBlockRows];
     if (ctl->done || ctl->halt || l >= ctl->n_static) return;
-    const long long it = ctl->iter_base + ctl->iter;
-    const int tau = sample_block(ctl->scdf ? ctl->scdf : A.cdf, A.k, ctl->seed, ctl->sysid, (uint64_t)it, (uint64_t)l);
+    const int tau = drawn_block(A, ctl, l);
     const int r0 = A.off[tau], s = A.off[tau + 1] - r0;
-    for (int a = threadIdx.x; a < s; a += blockDim.x) rbase[a] = A.rowptr[r0 + a];
-    __syncthreads();
     const bool wood = A.wood_ptr && A.wood_ptr[tau] >= 0;
+    const T *src = wood ? rl : y;
+    for (int a = threadIdx.x; a < s; a += blockDim.x) ys[a] = src[a];
+    __syncthreads();
+    const T *B0 = A.val + (long long)r0 * A.n;
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < A.n; c += gridDim.x * blockDim.x) {
-        T acc3 = T(0);
-        if (wood) {
-            for (int a = 0; a < s; ++a) acc3 = Ar<T>::fma(A.val[rbase[a] + c], rl[a], acc3);
-            y[c] = acc3;
-        } else {
-            for (int a = 0; a < s; ++a) acc3 = Ar<T>::fma(A.val[rbase[a] + c], y[a], acc3);
-            x[c] = Ar<T>::add(x[c], acc3);
-        }
+        const T acc3 = column_chain<T>(s, ys, [&](int a) { return __ldg(B0 + (long long)a * A.n + c); });
+        if (wood) y[c] = acc3;
+        else x[c] = Ar<T>::add(x[c], acc3);
     }
 }
 
@@ -2191,9 +2206,7 @@ __global__ void __launch_bounds__(256) k_sd_scatter(Mat<T> A, const T *__restric
 template <typename T>
 __global__ void __launch_bounds__(256) k_sd_wood(Mat<T> A, const T *__restrict__ g, T *x, Ctl *ctl, int l) {
     if (ctl->done || ctl->halt || l >= ctl->n_static) return;
-    const long long it = ctl->iter_base + ctl->iter;
-    const int tau = sample_block(ctl->scdf ? ctl->scdf : A.cdf, A.k, ctl->seed, ctl->sysid, (uint64_t)it, (uint64_t)l);
-    const long long wp = A.wood_ptr[tau];
+    const long long wp = A.wood_ptr[drawn_block(A, ctl, l)];
     if (wp < 0) return;
     const T *V = A.wood + wp;
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < A.n; c += gridDim.x * blockDim.x) {
@@ -2600,18 +2613,24 @@ __global__ void __launch_bounds__(256) k_dyn_dense_scatter(const double *__restr
                                                            int use_cond,
                                                            cudaGraphConditionalHandle hcond, int wood) {
     __shared__ int is_last;
+    __shared__ int rows[kMaxDynRows];
+    __shared__ T ys[kMaxDynRows];
     if (ctl->done || ctl->status || ctl->halt) {
         if (count_iter && blockIdx.x == 0) end_iteration<T>(x, n, ctl, use_cond, hcond);
         return;
     }
+    if (!wood)
+        for (int a = threadIdx.x; a < K; a += blockDim.x) {
+            rows[a] = D.I[a];
+            ys[a] = as<T>(D.y[a]);
+        }
+    __syncthreads();
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
         if (wood) {                           // the n x n form: x_c += y_c
             x[c] = Ar<T>::add(x[c], as<T>(D.y[c]));
             continue;
         }
-        T acc = T(0);
-        for (int a = 0; a < K; ++a)
-            acc = Ar<T>::fma(dense_value<T>(v64, v32, (long long)D.I[a] * n + c), as<T>(D.y[a]), acc);
+        const T acc = column_chain<T>(K, ys, [&](int a) { return dense_value<T>(v64, v32, (long long)rows[a] * n + c); });
         x[c] = Ar<T>::add(x[c], acc);
     }
     __threadfence();
@@ -3220,9 +3239,10 @@ static Dyn dyn_bufs(rorbk_ctx *h) {
                h->dyn.gc, h->dyn.z, h->dyn.fidx, h->K, (int)h->n, h->dyn.skcap};
 }
 
-// The sparse path's plan of the next draws (the dense path samples its own).
-static Plan plan_of(rorbk_ctx *h) {
-    if (h->format != RORBK_FORMAT_CSR) return Plan{};
+// The plan of the next draws: formed by the dynamic update of a sparse A, by the
+// top-K pass of a dense one.
+static Plan plan_of(rorbk_ctx *h, int format) {
+    if (h->format != format) return Plan{};
     return Plan{h->cdf, h->k, h->off, h->ops.s_ptr, h->blk_nz, h->ops.w_ptr};
 }
 
@@ -3250,21 +3270,23 @@ int grid_scatter(rorbk_ctx *h) {
 }
 
 int residual_grid(rorbk_ctx *h) {
+    if (h->format == RORBK_FORMAT_DENSE) return h->num_sms;   // k_residual_dense: one block per SM
     int per_sm = 0, per_sm32 = 0;
-    if (h->format == RORBK_FORMAT_DENSE) {
-        if (h->vdtype == RORBK_F32)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_residual<double, float, true>, 256, 0);
-        else
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_residual<double, double, true>, 256, 0);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm32, k_residual<float, float, true>, 256, 0);
-    } else {
-        if (h->vdtype == RORBK_F32)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_residual<double, float>, 256, 0);
-        else
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_residual<double, double>, 256, 0);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm32, k_residual<float, float>, 256, 0);
-    }
+    if (h->vdtype == RORBK_F32)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_residual<double, float>, 256, 0);
+    else
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_residual<double, double>, 256, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm32, k_residual<float, float>, 256, 0);
     return std::max(1, std::min(per_sm, per_sm32 > 0 ? per_sm32 : per_sm)) * h->num_sms;
+}
+
+template <typename T, typename V>
+static void configure_residual_dense() {
+    const int sm = (int)dense_res_smem<T, V>();
+    cudaFuncSetAttribute(k_residual_dense<T, V, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    cudaFuncSetAttribute(k_residual_dense<T, V, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    cudaFuncSetAttribute(k_residual_dense<T, V, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    cudaFuncSetAttribute(k_residual_dense<T, V, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
 }
 
 template <int NR>
@@ -3351,10 +3373,13 @@ void configure_kernels() {
     configure_cluster(k_dense_chol<double>);
     configure_cluster(k_dense_chol<float>);
     cudaFuncSetAttribute(k_dyn_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gram_tc_smem());
-    cudaFuncSetAttribute(k_sd_rows_tiled<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(k_sd_rows<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)sd_rows_smem<double>());
-    cudaFuncSetAttribute(k_sd_rows_tiled<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(k_sd_rows<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)sd_rows_smem<float>());
+    configure_residual_dense<double, double>();
+    configure_residual_dense<double, float>();
+    configure_residual_dense<float, float>();
     // the column-block instances
     cudaFuncSetAttribute(k_static<double, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)static_smem_bytes<double>());
@@ -3519,7 +3544,7 @@ static void launch_dynamic_tail(rorbk_ctx *h, const T *r, T *x, Ctl *ctl, int ch
     Mat<T> A = make_mat<T>(h);
     k_dyn_mark<T><<<grid_mark(h), 512, factor_smem_bytes(), h->stream>>>(A, r, dyn_bufs(h), ctl,
                                                                         check_done, one_col((int)h->m),
-                                                                        count_iter ? plan_of(h) : Plan{},
+                                                                        count_iter ? plan_of(h, RORBK_FORMAT_CSR) : Plan{},
                                                                         fac_max(h));
     if (inc) launch_dyn_scatter<T, true, false>(h, x, ctl, count_iter, use_cond, hcond, one_col((int)h->m));
     else launch_dyn_scatter<T, false, false>(h, x, ctl, count_iter, use_cond, hcond, one_col((int)h->m));
@@ -3532,17 +3557,30 @@ const double *csc_values<double>(const rorbk_ctx *h) { return h->csc_val; }
 template <>
 const float *csc_values<float>(const rorbk_ctx *h) { return h->csc_val32; }
 
-// The residual kernel for this handle's format (the dense instance reads no
-// column indices).
+template <typename V>
+static const V *row_major(const rorbk_ctx *h);
+template <>
+const double *row_major<double>(const rorbk_ctx *h) { return h->val; }
+template <>
+const float *row_major<float>(const rorbk_ctx *h) { return h->val32; }
+
+// The residual kernel for this handle's format.  Dense: as many chain warps per
+// SM as there are groups of 32 rows for it (8 at most).
 template <typename T, typename V>
 static void residual_launch(rorbk_ctx *h, const Mat<T> &A, const T *b, const T *x, T *r, Ctl *ctl,
                             int finalize) {
-    if (h->format == RORBK_FORMAT_DENSE)
-        k_residual<T, V, true><<<h->grid_res, 256, 0, h->stream>>>(A, b, x, r, h->partials, h->hist1, ctl,
-                                                                   finalize);
-    else
-        k_residual<T, V, false><<<h->grid_res, 256, 0, h->stream>>>(A, b, x, r, h->partials, h->hist1, ctl,
-                                                                    finalize);
+    if (h->format != RORBK_FORMAT_DENSE) {
+        k_residual<T, V><<<h->grid_res, 256, 0, h->stream>>>(A, b, x, r, h->partials, h->hist1, ctl, finalize);
+        return;
+    }
+    const int m = (int)h->m, n = (int)h->n, nsl = (m + 31) / 32, g = std::min(h->grid_res, nsl);
+    const int per = (nsl + h->grid_res - 1) / h->grid_res;
+    const size_t sm = dense_res_smem<T, V>();
+    const V *v = row_major<V>(h);
+    if (per > 4) k_residual_dense<T, V, 8><<<g, 256, sm, h->stream>>>(v, m, n, h->K, b, x, r, h->partials, h->hist1, ctl, finalize);
+    else if (per > 2) k_residual_dense<T, V, 4><<<g, 256, sm, h->stream>>>(v, m, n, h->K, b, x, r, h->partials, h->hist1, ctl, finalize);
+    else if (per > 1) k_residual_dense<T, V, 2><<<g, 256, sm, h->stream>>>(v, m, n, h->K, b, x, r, h->partials, h->hist1, ctl, finalize);
+    else k_residual_dense<T, V, 1><<<g, 256, sm, h->stream>>>(v, m, n, h->K, b, x, r, h->partials, h->hist1, ctl, finalize);
 }
 
 template <typename T>
@@ -3552,14 +3590,12 @@ void launch_iteration_t(rorbk_ctx *h, const T *b, T *x, T *r, Ctl *ctl, int use_
     if (h->format == RORBK_FORMAT_DENSE) {
         T *rl = (T *)h->sd_scratch, *yy = rl + kMaxBlockRows;
         const int gr = (h->smax + 31) / 32;
-        // column-parallel passes in blocks of 64 threads: more SMs share the
-        // FP64 chains of a narrow system
-        const int gs = std::max(1, std::min(8 * h->num_sms, (int)((h->n + 63) / 64)));
+        const int gs = std::max(1, std::min(8 * h->num_sms, (int)((h->n + kSdThreads - 1) / kSdThreads)));
         for (int l = 0; l < kDenseStatic; ++l) {
-            k_sd_rows_tiled<T><<<gr, kSdCols, sd_rows_smem<T>(), h->stream>>>(A, b, x, rl, ctl, l);
-            k_sd_apply<T><<<1, 1024, 0, h->stream>>>(A, rl, yy, ctl, l);
-            k_sd_scatter<T><<<gs, 64, 0, h->stream>>>(A, rl, yy, x, ctl, l);
-            if (h->n_wood) k_sd_wood<T><<<gs, 64, 0, h->stream>>>(A, yy, x, ctl, l);
+            k_sd_rows<T><<<gr, 32, sd_rows_smem<T>(), h->stream>>>(A, b, x, rl, ctl, l);
+            k_sd_apply<T><<<gr, 32, 0, h->stream>>>(A, rl, yy, ctl, l);
+            k_sd_scatter<T><<<gs, kSdThreads, 0, h->stream>>>(A, rl, yy, x, ctl, l);
+            if (h->n_wood) k_sd_wood<T><<<gs, kSdThreads, 0, h->stream>>>(A, yy, x, ctl, l);
         }
         // updates beyond kDenseStatic (n_static > 3), if any
         (h->n_wood ? k_static<T, false, true> : k_static<T, false, false>)<<<1, 1024, static_smem_bytes<T>(),
@@ -3589,7 +3625,8 @@ void launch_iteration_t(rorbk_ctx *h, const T *b, T *x, T *r, Ctl *ctl, int use_
         if (weighted) launch_weights(h, r);      // the draws of the next iteration
     k_topk_hist2<T><<<grid_topk(h), 256, 0, h->stream>>>(r, (int)h->m, h->K, h->hist2, ctl, 1, one_col((int)h->m));
     k_topk_collect<T><<<grid_collect(h), 512, collect_smem_bytes(), h->stream>>>(
-        r, (int)h->m, h->K, h->rowptr, h->in_list, h->eq_list, dyn_bufs(h), ctl, 1, one_col((int)h->m));
+        r, (int)h->m, h->K, h->rowptr, h->in_list, h->eq_list, dyn_bufs(h), ctl, 1, one_col((int)h->m),
+        plan_of(h, RORBK_FORMAT_DENSE));
     launch_dynamic_tail<T>(h, r, x, ctl, 1, 1, use_cond, hcond, inc);
 }
 
@@ -3633,9 +3670,9 @@ static void launch_mr_iteration_t(rorbk_ctx *h, const T *b, T *x, T *r, Ctl *ctl
         k_topk_hist1<T, true><<<dim3(g, nr), 256, 0, st>>>(r, m, K, h->hist1, ctl, cl, 1);
     k_topk_hist2<T, true><<<dim3(g, nr), 256, 0, st>>>(r, m, K, h->hist2, ctl, 1, cl);
     k_topk_collect<T, true><<<dim3(grid_collect(h), nr), 512, collect_smem_bytes(), st>>>(
-        r, m, K, h->rowptr, h->in_list, h->eq_list, dyn_bufs(h), ctl, 1, cl);
+        r, m, K, h->rowptr, h->in_list, h->eq_list, dyn_bufs(h), ctl, 1, cl, Plan{});
     k_dyn_mark<T, true><<<dim3(grid_mark(h), nr), 512, factor_smem_bytes(), st>>>(
-        A, r, dyn_bufs(h), ctl, 1, cl, plan_of(h), fac_max(h));
+        A, r, dyn_bufs(h), ctl, 1, cl, plan_of(h, RORBK_FORMAT_CSR), fac_max(h));
     launch_dyn_scatter<T, false, true>(h, x, ctl, 1, use_cond, hcond, cl);
 }
 
@@ -3726,7 +3763,7 @@ void launch_topk_only(rorbk_ctx *h, const double *r, int *I) {
     k_topk_hist1<double><<<g, 256, 0, h->stream>>>(r, (int)h->m, h->K, h->hist1, h->ctl, one, 0);
     k_topk_hist2<double><<<g, 256, 0, h->stream>>>(r, (int)h->m, h->K, h->hist2, h->ctl, 0, one);
     k_topk_collect<double><<<std::max(1, g / 2), 512, collect_smem_bytes(), h->stream>>>(
-        r, (int)h->m, h->K, h->rowptr, h->in_list, h->eq_list, dyn_bufs(h), h->ctl, 0, one);
+        r, (int)h->m, h->K, h->rowptr, h->in_list, h->eq_list, dyn_bufs(h), h->ctl, 0, one, Plan{});
     cudaMemcpyAsync(I, h->dyn.I, h->K * sizeof(int), cudaMemcpyDeviceToDevice, h->stream);
 }
 

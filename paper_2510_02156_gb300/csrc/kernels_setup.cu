@@ -571,14 +571,13 @@ void widen_values(rorbk_ctx *h, int dtype) {
 }
 
 // SELL-32 copy of A: lane l of slice s holds row sell_row[32 s + l]; entry j
-// of that lane sits at ptr[s] + 32 j + l (the values of a dense A: grouped
-// VW consecutive entries per lane, see below).
+// of that lane sits at ptr[s] + 32 j + l.
 __global__ void k_sell_fill(const int *__restrict__ rowptr, const int *__restrict__ col,
                             const double *__restrict__ val, const float *__restrict__ val32,
                             int nslices, const long long *__restrict__ ptr,
                             const int *__restrict__ srow, const int *__restrict__ srlen,
                             int *__restrict__ scol, double *__restrict__ sval,
-                            float *__restrict__ sval32, int dense) {
+                            float *__restrict__ sval32) {
     const long long slot = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (slot >= (long long)nslices * 32) return;
     const int s = (int)(slot >> 5), lane = (int)(slot & 31);
@@ -589,12 +588,8 @@ __global__ void k_sell_fill(const int *__restrict__ rowptr, const int *__restric
         const long long d = base + 32LL * j;
         const bool in = j < len;
         scol[d] = in ? col[p0 + j] : 0;
-        // a dense A's values: entry j of lane l at 32 VW (j / VW) + VW l + j % VW,
-        // VW = 16 bytes / value size, so a lane reads VW entries per load
-        const long long d64 = dense ? ptr[s] + 64LL * (j >> 1) + 2 * lane + (j & 1) : d;
-        const long long d32 = dense ? ptr[s] + 128LL * (j >> 2) + 4 * lane + (j & 3) : d;
-        if (sval) sval[d64] = in ? val[p0 + j] : 0.0;
-        if (sval32) sval32[d32] = in ? val32[p0 + j] : 0.0f;
+        if (sval) sval[d] = in ? val[p0 + j] : 0.0;
+        if (sval32) sval32[d] = in ? val32[p0 + j] : 0.0f;
     }
 }
 
@@ -731,7 +726,8 @@ static rorbk_status scan_device(rorbk_ctx *h, int *d, long long n, int *grand_to
 }
 
 // Rows sorted by length (longest first, ties by row) into slices of 32.  On a
-// refresh of the values only the values are copied again.
+// refresh of the values only the values are copied again.  (A dense A's passes
+// read it row-major and need no such copy.)
 static rorbk_status build_sell(rorbk_ctx *h, const std::vector<int> &hrp, bool refresh) {
     auto &S = h->sell;
     cudaStream_t st = h->stream;
@@ -759,10 +755,7 @@ static rorbk_status build_sell(rorbk_ctx *h, const std::vector<int> &hrp, bool r
                 }
             }
             len[sl] = L;
-            // a dense A's slices span a multiple of 4 entries per lane (its values
-            // are grouped 4 (FP32) or 2 (FP64) entries per lane)
-            const int Lp = h->format == RORBK_FORMAT_DENSE ? (L + 3) & ~3 : L;
-            ptr[sl + 1] = ptr[sl] + 32LL * Lp;
+            ptr[sl + 1] = ptr[sl] + 32LL * L;
         }
         S.nslices = ns;
         S.ptr = (long long *)dev_alloc(h, (ns + 1) * sizeof(long long));
@@ -783,8 +776,7 @@ static rorbk_status build_sell(rorbk_ctx *h, const std::vector<int> &hrp, bool r
     }
     const int ns = S.nslices;
     k_sell_fill<<<(unsigned)((ns * 32LL + 255) / 256), 256, 0, st>>>(
-        h->rowptr, h->col, h->val, h->val32, ns, S.ptr, S.row, S.rlen, S.col, S.val, S.val32,
-        h->format == RORBK_FORMAT_DENSE ? 1 : 0);
+        h->rowptr, h->col, h->val, h->val32, ns, S.ptr, S.row, S.rlen, S.col, S.val, S.val32);
     return cuda_check(h, cudaStreamSynchronize(st), "SELL copy of A");
 }
 
@@ -836,7 +828,7 @@ rorbk_status build_setup(rorbk_ctx *h, const std::vector<int> &hrp, bool refresh
     if (hf[0] & 2) return fail(h, RORBK_ERR_NUMERIC, "A holds NaN or Inf");
     if (!keep(h, h->blk_nz, k + 1)) return fail(h, RORBK_ERR_OOM, "block entry offsets");
     k_block_nz<<<std::max(1, (k + 256) / 256), 256, 0, s>>>(h->rowptr, h->off, k, h->blk_nz);
-    if ((st = build_sell(h, hrp, refresh))) return st;
+    if (h->format == RORBK_FORMAT_CSR && (st = build_sell(h, hrp, refresh))) return st;
     if (!refresh && (st = build_block_order(h, hrp))) return st;
     // row norms for the dynamic update: from the FP64 values, and from the
     // FP32 copy that the mixed form's inner solve reads when it differs
