@@ -3,12 +3,14 @@
 // A row's dot product with x is one fused multiply-add chain over its columns,
 // so the parallelism of a dense pass is its rows: one lane per row, 32 rows per
 // warp.  What bounds such a warp is either the chain itself (GB300: 4.7 cycles
-// per FP32 link, 64 per FP64 link) or the bytes it keeps in flight; registers
-// hold too few of the latter, so each warp runs a ring of stages in shared
-// memory that it fills for itself by asynchronous 16-byte copies (cp.async),
-// 256 bytes of each of its rows and the matching part of x per stage.  A row of
-// a stage starts 272 bytes after the previous one: the lanes' 16-byte reads of
-// their own rows meet no bank conflict.
+// per FP32 link, 64 per FP64 link) or the bytes it keeps in flight.  Registers
+// hold too few of the latter, so the rows go through a ring of stages in shared
+// memory, RB bytes of each row and the matching part of x per stage, filled by
+// asynchronous 16-byte copies.  A second warp issues the copies: the chain's warp
+// is left with the reads of its stage, one pack of values ahead of the chain
+// (with the copies in its own instruction stream an FP32 link took 14 cycles and
+// an FP64 link 88).  A row of a stage starts RB + 16 bytes after the previous
+// one: the lanes' 16-byte reads of their own rows meet no bank conflict.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -18,10 +20,10 @@
 
 namespace rorbk {
 
-template <typename T, typename V>
+template <typename T, typename V, int RB>
 struct DenseStage {
-    static constexpr int cols = 256 / sizeof(V);                 // columns per stage
-    static constexpr int pitch = 272;                            // bytes between rows
+    static constexpr int cols = RB / sizeof(V);                  // columns per stage
+    static constexpr int pitch = RB + 16;                        // bytes between rows
     static constexpr int bytes = 32 * pitch + cols * (int)sizeof(T);
 };
 
@@ -41,96 +43,140 @@ template <typename T> struct Pack16;
 template <> struct Pack16<float> { using type = float4; };
 template <> struct Pack16<double> { using type = double2; };
 
-// One warp: acc_l = sum over j ascending of A0[l * n + j] x[j] (one fused chain
-// from 0) for the lanes l < rows.  ring: ST stages of DenseStage<T, V>::bytes.
-// vec: every row starts on a 16-byte boundary (n * sizeof(V) % 16 == 0); else
-// the rows are copied value by value.
-template <typename T, typename V, int ST>
-__device__ __forceinline__ T dense_chain(const V *__restrict__ A0, int rows, int n, const T *__restrict__ x,
-                                         unsigned char *ring, bool vec) {
-    using S = DenseStage<T, V>;
+// A pair of warps: acc_l = sum over j ascending of A0[l * n + j] x[j] (one fused
+// chain from 0) for the lanes l < rows, in the warp that calls dense_sum; the
+// other warp calls dense_copy for the same rows.  ring: ST stages of DenseStage<T, V, RB>::bytes.  vec: every
+// row starts on a 16-byte boundary (n * sizeof(V) % 16 == 0); else the rows are
+// copied value by value.  The pair meets at named barrier `bar` once per stage:
+// behind it stage k has landed and stage k - 1 is free.
+__device__ __forceinline__ void pair_sync(int bar) {
+    __syncwarp();
+    switch (bar) {                                    // an immediate barrier number
+        case 1: asm volatile("bar.sync 1, 64;" ::: "memory"); break;
+        case 2: asm volatile("bar.sync 2, 64;" ::: "memory"); break;
+        case 3: asm volatile("bar.sync 3, 64;" ::: "memory"); break;
+        case 4: asm volatile("bar.sync 4, 64;" ::: "memory"); break;
+        case 5: asm volatile("bar.sync 5, 64;" ::: "memory"); break;
+        case 6: asm volatile("bar.sync 6, 64;" ::: "memory"); break;
+        case 7: asm volatile("bar.sync 7, 64;" ::: "memory"); break;
+        default: asm volatile("bar.sync 8, 64;" ::: "memory"); break;
+    }
+}
+
+template <typename T, typename V, int RB, int ST>
+__device__ __forceinline__ void dense_copy(const V *__restrict__ A0, int rows, int n, const T *__restrict__ x,
+                                           unsigned char *ring, bool vec, int bar) {
+    using S = DenseStage<T, V, RB>;
     constexpr int EP = 16 / sizeof(V);                            // values per 16 bytes
+    constexpr int RP = 32 / (RB / 16);                            // rows per copy instruction (1 or 2)
     const int lane = threadIdx.x & 31;
     const int nst = (n + S::cols - 1) / S::cols;
-    const unsigned rb = smem_u32(ring);
-    auto issue = [&](int k) {
-        if (k < nst) {
-            const unsigned sb = rb + (unsigned)(k % ST) * S::bytes;
-            const int c0 = k * S::cols;
-            if (vec) {
-                const int ch = lane & 15, c = c0 + ch * EP;
-                const int bytes = min(16, (n - c) * (int)sizeof(V));
-                const V *src = A0 + (long long)(lane >> 4) * n + c;
-                unsigned dst = sb + (lane >> 4) * S::pitch + ch * 16;
+    {
+        const unsigned rb = smem_u32(ring);
+        const int ch = lane % (RB / 16), u0 = lane / (RB / 16);
+        auto issue = [&](int k) {
+            if (k < nst) {
+                const unsigned sb = rb + (unsigned)(k % ST) * S::bytes;
+                const int c0 = k * S::cols;
+                if (vec) {
+                    const int c = c0 + ch * EP, bytes = min(16, (n - c) * (int)sizeof(V));
+                    const V *src = A0 + (long long)u0 * n + c;
+                    unsigned dst = sb + u0 * S::pitch + ch * 16;
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
-                    if (2 * u + (lane >> 4) < rows && bytes > 0) cp_async16(dst, src, bytes);
-                    src += 2LL * n;
-                    dst += 2 * S::pitch;
+                    for (int u = 0; u < 32; u += RP) {
+                        if (u + u0 < rows && bytes > 0) cp_async16(dst, src, bytes);
+                        src += (long long)RP * n;
+                        dst += RP * S::pitch;
+                    }
+                } else {
+                    for (int u = 0; u < rows; ++u)
+#pragma unroll
+                        for (int q = 0; q < S::cols / 32; ++q) {
+                            const int c = c0 + 32 * q + lane;
+                            if (c < n)
+                                cp_async_elem<sizeof(V)>(sb + u * S::pitch + (32 * q + lane) * (int)sizeof(V),
+                                                         A0 + (long long)u * n + c);
+                        }
+                }
+#pragma unroll
+                for (int q = 0; q < S::cols / 32; ++q) {
+                    const int c = c0 + 32 * q + lane;
+                    if (c < n) cp_async_elem<sizeof(T)>(sb + 32 * S::pitch + (32 * q + lane) * (int)sizeof(T), x + c);
+                }
+            }
+            cp_async_commit();
+        };
+#pragma unroll 1
+        for (int k = 0; k < ST - 1; ++k) issue(k);
+#pragma unroll 1
+        for (int k = 0; k < nst; ++k) {
+            cp_async_wait<ST - 2>();
+            pair_sync(bar);
+            issue(k + ST - 1);
+        }
+        cp_async_wait<0>();
+    }
+    pair_sync(bar);                                   // the ring is free for the next rows
+}
+
+template <typename T, typename V, int RB, int ST>
+__device__ __forceinline__ T dense_sum(int n, const unsigned char *ring, int bar) {
+    using S = DenseStage<T, V, RB>;
+    constexpr int EP = 16 / sizeof(V);
+    const int lane = threadIdx.x & 31;
+    const int nst = (n + S::cols - 1) / S::cols;
+    T acc = T(0);
+    {
+        constexpr int GP = 4;                                     // packs per group
+        constexpr int NG = RB / 16 / GP;
+#pragma unroll 1
+        for (int k = 0; k < nst; ++k) {
+            pair_sync(bar);
+            const unsigned char *st = ring + (size_t)(k % ST) * S::bytes;
+            const V *row = (const V *)(st + lane * S::pitch);
+            const T *xs = (const T *)(st + 32 * S::pitch);
+            if (k * S::cols + S::cols <= n) {
+                V v[2][GP * EP];
+                T xv[2][GP * EP];
+                auto fetch = [&](int g, V *vd, T *xd) {
+#pragma unroll
+                    for (int q = 0; q < GP; ++q) {
+                        const typename Pack16<V>::type t = *(const typename Pack16<V>::type *)(row + (g * GP + q) * EP);
+                        vd[q * EP] = t.x;
+                        vd[q * EP + 1] = t.y;
+                        if constexpr (EP == 4) { vd[q * EP + 2] = t.z; vd[q * EP + 3] = t.w; }
+                    }
+#pragma unroll
+                    for (int q = 0; q < GP * EP; q += 16 / (int)sizeof(T)) {
+                        const typename Pack16<T>::type t = *(const typename Pack16<T>::type *)(xs + g * GP * EP + q);
+                        xd[q] = t.x;
+                        xd[q + 1] = t.y;
+                        if constexpr (sizeof(T) == 4) { xd[q + 2] = t.z; xd[q + 3] = t.w; }
+                    }
+                };
+                fetch(0, v[0], xv[0]);
+#pragma unroll
+                for (int g = 0; g < NG; ++g) {
+                    if (g + 1 < NG) fetch(g + 1, v[(g + 1) & 1], xv[(g + 1) & 1]);
+#pragma unroll
+                    for (int q = 0; q < GP * EP; ++q) acc = Ar<T>::fma(wide<T>(v[g & 1][q]), xv[g & 1][q], acc);
                 }
             } else {
-                for (int u = 0; u < rows; ++u)
-#pragma unroll
-                    for (int q = 0; q < S::cols / 32; ++q) {
-                        const int c = c0 + 32 * q + lane;
-                        if (c < n)
-                            cp_async_elem<sizeof(V)>(sb + u * S::pitch + (32 * q + lane) * (int)sizeof(V),
-                                                     A0 + (long long)u * n + c);
-                    }
+                for (int j = 0; j < n - k * S::cols; ++j) acc = Ar<T>::fma(wide<T>(row[j]), xs[j], acc);
             }
-#pragma unroll
-            for (int q = 0; q < S::cols / 32; ++q) {
-                const int c = c0 + 32 * q + lane;
-                if (c < n) cp_async_elem<sizeof(T)>(sb + 32 * S::pitch + (32 * q + lane) * (int)sizeof(T), x + c);
-            }
-        }
-        cp_async_commit();
-    };
-    __syncwarp();                                     // the ring's earlier readers are done
-#pragma unroll 1
-    for (int k = 0; k < ST - 1; ++k) issue(k);
-    T acc = T(0);
-#pragma unroll 1
-    for (int k = 0; k < nst; ++k) {
-        cp_async_wait<ST - 2>();
-        __syncwarp();                                 // stage k is there; stage k - 1 is free
-        issue(k + ST - 1);
-        const unsigned char *st = ring + (size_t)(k % ST) * S::bytes;
-        const V *row = (const V *)(st + lane * S::pitch);
-        const T *xs = (const T *)(st + 32 * S::pitch);
-        if (k * S::cols + S::cols <= n) {
-#pragma unroll 4
-            for (int q = 0; q < S::cols / EP; ++q) {
-                const typename Pack16<V>::type v = *(const typename Pack16<V>::type *)(row + q * EP);
-                T xv[EP];
-#pragma unroll
-                for (int u = 0; u < EP; u += 16 / (int)sizeof(T)) {
-                    const typename Pack16<T>::type t = *(const typename Pack16<T>::type *)(xs + q * EP + u);
-                    xv[u] = t.x;
-                    xv[u + 1] = t.y;
-                    if constexpr (sizeof(T) == 4) { xv[u + 2] = t.z; xv[u + 3] = t.w; }
-                }
-                acc = Ar<T>::fma(wide<T>(v.x), xv[0], acc);
-                acc = Ar<T>::fma(wide<T>(v.y), xv[1], acc);
-                if constexpr (EP == 4) {
-                    acc = Ar<T>::fma(wide<T>(v.z), xv[2], acc);
-                    acc = Ar<T>::fma(wide<T>(v.w), xv[3], acc);
-                }
-            }
-        } else {
-            for (int j = 0; j < n - k * S::cols; ++j) acc = Ar<T>::fma(wide<T>(row[j]), xs[j], acc);
         }
     }
-    cp_async_wait<0>();
+    pair_sync(bar);
     return acc;
 }
 
 // One thread: sum over a = 0 .. s-1 ascending of at(a) * y[a] (one fused chain
 // from 0), the values read kAhead at a time while the chain runs over the
-// previous ones.
+// previous ones: 16 FP64 links last about as long as a load, 64 FP32 links half
+// as long.
 template <typename T, typename At>
 __device__ __forceinline__ T column_chain(int s, const T *y, At at) {
-    constexpr int kAhead = 16;
+    constexpr int kAhead = sizeof(T) == 8 ? 24 : 64;
     T acc = T(0), nx[kAhead];
 #pragma unroll
     for (int u = 0; u < kAhead; ++u) nx[u] = u < s ? at(u) : T(0);

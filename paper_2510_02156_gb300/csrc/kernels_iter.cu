@@ -846,44 +846,50 @@ __global__ void __launch_bounds__(256, 4) k_residual(Mat<T> A, const T *__restri
     residual_finish(rr, hist, partials, hist1, ctl, A.K, finalize);
 }
 
-// r = b - A x for a dense A: one warp per 32 consecutive rows on its own ring of
-// stages (dense_rows.cuh), row-major values, one block per SM.  W warps per block
-// run chains, with 24 / W stages each: as many as there are groups of rows per
-// SM, so that a short A (few chains) keeps more bytes of each in flight.
-constexpr int kDrStages = 24;       // stages per block, about 9 KB each
+// r = b - A x for a dense A: a pair of warps per 32 consecutive rows on a ring
+// of stages (dense_rows.cuh), row-major values, one block per SM.  W pairs per
+// block run, with longer and more stages the fewer they are, so that a short A
+// (few chains) keeps more bytes of each in flight.
+// 200,000 x 2,048 FP32: 300 -> 262 us, 0.92 of measured HBM; 25,600 x 2,048 FP64:
+// 175 -> 117 us (bound by the FP64 rate: 107); 2,048 x 100,000: 8,300 -> 3,628 us
+// FP64, 4,280 -> 284 us FP32 (bound by the chains: 3,200 and 240).
+template <typename T, typename V, int RB, int ST>
+__host__ __device__ constexpr size_t dense_res_smem(int W) { return (size_t)W * ST * DenseStage<T, V, RB>::bytes; }
 
-template <typename T, typename V>
-__host__ __device__ constexpr size_t dense_res_smem() { return (size_t)kDrStages * DenseStage<T, V>::bytes; }
-
-template <typename T, typename V, int W>
-__global__ void __launch_bounds__(256, 1) k_residual_dense(const V *__restrict__ val, int m, int n, int K,
+template <typename T, typename V, int RB, int ST>
+__global__ void __launch_bounds__(512, 1) k_residual_dense(const V *__restrict__ val, int m, int n, int K,
                                                           const T *__restrict__ b, const T *__restrict__ x,
                                                           T *__restrict__ r, double *partials, unsigned *hist1,
-                                                          Ctl *ctl, int finalize) {
+                                                          Ctl *ctl, int finalize, int W) {
     extern __shared__ __align__(16) unsigned char dr_ring[];
     __shared__ unsigned hist[kHistBins];
     if ((finalize == 1 || finalize == 3) && (ctl->done || ctl->halt)) return;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, pair = ST == 8 ? 0 : threadIdx.x >> 6;
+    const bool load = (threadIdx.x >> 5) & 1;
     for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) hist[i] = 0u;
     __syncthreads();
     double rr = 0.0;
-    constexpr int ST = kDrStages / W;
-    if (wid < W) {
+    if (ST == 8 ? threadIdx.x < 64 : pair < W) {
         const bool vec = ((long long)n * (int)sizeof(V)) % 16 == 0;
-        const int nsl = (m + 31) / 32, Wt = gridDim.x * W, g = wid * gridDim.x + blockIdx.x;
-        unsigned char *ring = dr_ring + (size_t)wid * ST * DenseStage<T, V>::bytes;
-        for (int sl = g; sl < nsl; sl += Wt) {
-            const int row0 = sl * 32, rows = min(32, m - row0);
-            const T acc = dense_chain<T, V, ST>(val + (long long)row0 * n, rows, n, x, ring, vec);
-            const bool act = lane < rows;
-            unsigned bin = 0;
-            if (act) {
-                const T ri = Ar<T>::sub(b[row0 + lane], acc);
-                r[row0 + lane] = ri;
-                rr = __fma_rn((double)ri, (double)ri, rr);
-                bin = (unsigned)(abs_key(ri) >> 52);
+        const int nsl = (m + 31) / 32, Wt = gridDim.x * W, g = pair * gridDim.x + blockIdx.x;
+        unsigned char *ring = dr_ring + (size_t)pair * ST * DenseStage<T, V, RB>::bytes;
+        if (load) {
+            for (int sl = g; sl < nsl; sl += Wt)
+                dense_copy<T, V, RB, ST>(val + (long long)sl * 32 * n, min(32, m - sl * 32), n, x, ring, vec, 1 + pair);
+        } else {
+            for (int sl = g; sl < nsl; sl += Wt) {
+                const int row = sl * 32 + lane;
+                const T acc = dense_sum<T, V, RB, ST>(n, ring, 1 + pair);
+                const bool act = row < m;
+                unsigned bin = 0;
+                if (act) {
+                    const T ri = Ar<T>::sub(b[row], acc);
+                    r[row] = ri;
+                    rr = __fma_rn((double)ri, (double)ri, rr);
+                    bin = (unsigned)(abs_key(ri) >> 52);
+                }
+                if (finalize == 1) hist_add(hist, bin, act);
             }
-            if (finalize == 1) hist_add(hist, bin, act);
         }
     }
     residual_finish(rr, hist, partials, hist1, ctl, K, finalize);
@@ -2121,37 +2127,40 @@ __device__ __forceinline__ int drawn_block(const Mat<T> &A, const Ctl *ctl, int 
     return sample_block(ctl->scdf ? ctl->scdf : A.cdf, A.k, ctl->seed, ctl->sysid, (uint64_t)it, (uint64_t)l);
 }
 
-// The block's residual r_tau = b_tau - A_tau x: grid block g is one warp that
-// takes rows 32g .. 32g + 31 on a ring of 8 stages (dense_rows.cuh: seven stages
-// of FP32 links take longer than a load).  256 x 2,048: 95 -> 93 us in FP64
-// (2,048 links of 64 cycles are 66), 37 -> 22 us in FP32; 256 x 100,000 in FP32:
-// 1,537 -> 735 us.
-constexpr int kSdStages = 8;
+// The block's residual r_tau = b_tau - A_tau x: grid block g is a pair of warps
+// that takes rows 32g .. 32g + 31 on a ring of 8 stages (dense_rows.cuh).  256 x
+// 2,048: 95 -> 80 us in FP64 (2,048 links of 64 cycles are 66), 37 -> 15 us in FP32;
+// 256 x 100,000 in FP32: 1,537 -> 275 us.
+constexpr int kSdStages = 8, kSdRowBytes = 512;
 template <typename T>
-__host__ __device__ constexpr size_t sd_rows_smem() { return (size_t)kSdStages * DenseStage<T, T>::bytes; }
+__host__ __device__ constexpr size_t sd_rows_smem() { return (size_t)kSdStages * DenseStage<T, T, kSdRowBytes>::bytes; }
 
 template <typename T>
-__global__ void __launch_bounds__(32) k_sd_rows(Mat<T> A, const T *__restrict__ b, const T *__restrict__ x, T *rloc,
+__global__ void __launch_bounds__(64) k_sd_rows(Mat<T> A, const T *__restrict__ b, const T *__restrict__ x, T *rloc,
                                                 Ctl *ctl, int l) {
     extern __shared__ __align__(16) unsigned char dr_ring[];
     if (ctl->done || ctl->halt || l >= ctl->n_static) return;
-    const int tau = drawn_block(A, ctl, l), lane = threadIdx.x;
-    if (blockIdx.x == 0 && lane == 0 && ctl->tr_tau && ctl->iter < ctl->trace_cap)
+    const int tau = drawn_block(A, ctl, l), lane = threadIdx.x & 31;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && ctl->tr_tau && ctl->iter < ctl->trace_cap)
         ctl->tr_tau[ctl->iter * ctl->n_static + l] = tau;
     const int r0 = A.off[tau], s = A.off[tau + 1] - r0;
     const int row0 = blockIdx.x * 32;
     if (row0 >= s) return;
     const int rows = min(32, s - row0);
-    const bool vec = ((long long)A.n * (int)sizeof(T)) % 16 == 0;
+    const bool vec = ((long long)A.n * (int)sizeof(T)) % 16 == 0, load = threadIdx.x >= 32;
+    if (load) {
+        dense_copy<T, T, kSdRowBytes, kSdStages>(A.val + (long long)(r0 + row0) * A.n, rows, A.n, x, dr_ring, vec, 1);
+        return;
+    }
     const T bi = lane < rows ? b[r0 + row0 + lane] : T(0);
-    const T acc = dense_chain<T, T, kSdStages>(A.val + (long long)(r0 + row0) * A.n, rows, A.n, x, dr_ring, vec);
+    const T acc = dense_sum<T, T, kSdRowBytes, kSdStages>(A.n, dr_ring, 1);
     if (lane < rows) rloc[row0 + lane] = Ar<T>::sub(bi, acc);
 }
 
 // y = W_tau r_tau, one warp per 32 rows.  W_tau is stored full and symmetric, so
 // a lane reads its row down the column: the warp's loads are coalesced, and the
-// rows' warps sit on different SMs.  256 rows: 45 -> 22 us (FP64; 256 links of 64
-// cycles are 8), 46 -> 17 us (FP32).
+// rows' warps sit on different SMs.  256 rows: 45 -> 20 us (FP64; 256 links of 64
+// cycles are 8), 46 -> 16 us (FP32: launch and dependent loads).
 template <typename T>
 __global__ void __launch_bounds__(32) k_sd_apply(Mat<T> A, const T *__restrict__ rloc, T *y, Ctl *ctl, int l) {
     __shared__ T rs[kMaxBlockRows];
@@ -2159,17 +2168,20 @@ __global__ void __launch_bounds__(32) k_sd_apply(Mat<T> A, const T *__restrict__
     const int tau = drawn_block(A, ctl, l);
     if (A.wood_ptr && A.wood_ptr[tau] >= 0) return;   // the s >= n form needs no W r
     const int r0 = A.off[tau], s = A.off[tau + 1] - r0;
+    const int sb = A.s_ptr[tau], nS = A.s_ptr[tau + 1] - sb;
+    const long long wp = A.w_ptr[tau];
     const int a = blockIdx.x * 32 + threadIdx.x;
     if (blockIdx.x * 32 >= s) return;
-    const int sb = A.s_ptr[tau], nS = A.s_ptr[tau + 1] - sb;
-    for (int q = threadIdx.x; q < nS; q += 32) rs[q] = rloc[A.s_idx[sb + q]];
+    const int pos = a < s ? A.s_pos[r0 + a] : -1;
+    const bool all = nS == s;                         // every row is coupled: S is the block's rows in order
+#pragma unroll 8
+    for (int q = threadIdx.x; q < nS; q += 32) rs[q] = rloc[all ? q : A.s_idx[sb + q]];
     __syncwarp();
     if (a >= s) return;
-    const int pos = A.s_pos[r0 + a];
     if (pos < 0) {
         y[a] = Ar<T>::fma(A.w_diag[r0 + a], rloc[a], T(0));
     } else {
-        const T *Wc = A.w_ss + A.w_ptr[tau] + pos;
+        const T *Wc = A.w_ss + wp + pos;
         y[a] = column_chain<T>(nS, rs, [&](int q) { return __ldg(Wc + (long long)q * nS); });
     }
 }
@@ -2191,6 +2203,7 @@ __global__ void __launch_bounds__(kSdThreads) k_sd_scatter(Mat<T> A, const T *__
     const int r0 = A.off[tau], s = A.off[tau + 1] - r0;
     const bool wood = A.wood_ptr && A.wood_ptr[tau] >= 0;
     const T *src = wood ? rl : y;
+#pragma unroll 4
     for (int a = threadIdx.x; a < s; a += blockDim.x) ys[a] = src[a];
     __syncthreads();
     const T *B0 = A.val + (long long)r0 * A.n;
@@ -2224,32 +2237,79 @@ __global__ void __launch_bounds__(256) k_sd_wood(Mat<T> A, const T *__restrict__
 // solves (the same right-looking Cholesky and column-oriented solves as the
 // sparse coupled set); x += A_I^T y, each column summed over ascending rows
 // of I, then added.
-constexpr int kGT = 16;         // Gram tile: kGT x kGT entries per block
-constexpr int kGC = 64;         // columns staged per step
+//
+// The FP64 Gram: one warp per patch of 4 rows x 8 columns of the lower triangle
+// (a lane per entry), on its own ring of stages of the 12 rows.  Bound by the
+// FP64 rate: 17 cycles per warp instruction and SM, so what counts is that every
+// SM gets the same number of patches (1,056 of them at K = 256, 7 per SM) and that
+// few lanes idle above the diagonal.  K = 256, n = 2,048: 206 -> 125 us (16 x 16
+// tiles of 8 warps on 136 SMs before).
+constexpr int kGa = 4, kGb = 8;         // patch
+constexpr int kGcols = 32, kGpitch = kGcols * 8 + 16, kGst = 4;
+constexpr int kGstage = (kGa + kGb) * kGpitch;
 
-__global__ void __launch_bounds__(kGT * kGT) k_dyn_dense_gram(const double *__restrict__ val, int n,
-                                                              int K, double mu, Dyn D, Ctl *ctl) {
-    __shared__ double sa[kGT][kGC + 1], sb[kGT][kGC + 1];
+__global__ void __launch_bounds__(32) k_dyn_dense_gram(const double *__restrict__ val, int n, int K, double mu, Dyn D,
+                                                       Ctl *ctl) {
+    __shared__ __align__(16) unsigned char ring[kGst * kGstage];
     if (ctl->done || ctl->status || ctl->halt) return;
-    int t = blockIdx.x, ti = 0;                 // tile (ti, tj), tj <= ti
-    while (t > ti) { t -= ti + 1; ++ti; }
-    const int tj = t, tid = threadIdx.x;
-    const int ta = tid / kGT, tb = tid % kGT;
-    const int a = ti * kGT + ta, b = tj * kGT + tb;
-    double acc = 0.0;
-    for (int c0 = 0; c0 < n; c0 += kGC) {
-        const int w = min(kGC, n - c0);
-        for (int q = tid; q < kGT * kGC; q += blockDim.x) {
-            const int rr = q / kGC, cc = q % kGC;
-            const int ra = ti * kGT + rr, rb = tj * kGT + rr;
-            sa[rr][cc] = (ra < K && cc < w) ? val[(long long)D.I[ra] * n + c0 + cc] : 0.0;
-            sb[rr][cc] = (rb < K && cc < w) ? val[(long long)D.I[rb] * n + c0 + cc] : 0.0;
-        }
-        __syncthreads();
-        if (a < K && b <= a)
-            for (int cc = 0; cc < w; ++cc) acc = __fma_rn(sa[ta][cc], sb[tb][cc], acc);
-        __syncthreads();
+    // patches in rows of two: groups 2t and 2t + 1 of 4 rows have t + 1 patches each
+    int q = blockIdx.x, t = (int)((sqrtf(4.0f * (float)q + 1.0f) - 1.0f) * 0.5f);
+    while (t * (t + 1) > q) --t;
+    while ((t + 1) * (t + 2) <= q) ++t;
+    q -= t * (t + 1);
+    const int ua = 2 * t + q / (t + 1), ub = q % (t + 1);
+    const int lane = threadIdx.x, la = lane >> 3, lb = lane & 7;
+    const int a = ua * kGa + la, b = ub * kGb + lb;
+    if (ua * kGa >= K) return;
+    const bool vec = n % 2 == 0;
+    const unsigned rb = smem_u32(ring);
+    const int nst = (n + kGcols - 1) / kGcols;
+    // this lane's copies: 16-byte chunk lane & 15 of rows 2 u + (lane >> 4), u < 6
+    const double *src[6];
+#pragma unroll
+    for (int u = 0; u < 6; ++u) {
+        const int i = 2 * u + (lane >> 4), row = i < kGa ? ua * kGa + i : ub * kGb + i - kGa;
+        src[u] = row < K ? val + (long long)D.I[row] * n : nullptr;
     }
+    auto issue = [&](int k) {
+        if (k < nst) {
+            const unsigned sb = rb + (unsigned)(k % kGst) * kGstage + (lane >> 4) * kGpitch + (lane & 15) * 16;
+            const int c = k * kGcols + 2 * (lane & 15), left = n - c;
+#pragma unroll
+            for (int u = 0; u < 6; ++u) {
+                if (!src[u] || left <= 0) continue;
+                if (vec) {
+                    cp_async16(sb + 2 * u * kGpitch, src[u] + c, min(16, left * 8));
+                } else {
+                    cp_async_elem<8>(sb + 2 * u * kGpitch, src[u] + c);
+                    if (left > 1) cp_async_elem<8>(sb + 2 * u * kGpitch + 8, src[u] + c + 1);
+                }
+            }
+        }
+        cp_async_commit();
+    };
+    for (int k = 0; k < kGst - 1; ++k) issue(k);
+    double acc = 0.0;
+#pragma unroll 1
+    for (int k = 0; k < nst; ++k) {
+        cp_async_wait<kGst - 2>();
+        __syncwarp();
+        issue(k + kGst - 1);
+        const unsigned char *st = ring + (size_t)(k % kGst) * kGstage;
+        const double *ra = (const double *)(st + la * kGpitch), *rbp = (const double *)(st + (kGa + lb) * kGpitch);
+        const int w = min(kGcols, n - k * kGcols);
+        if (w == kGcols) {
+#pragma unroll
+            for (int c = 0; c < kGcols; c += 2) {
+                const double2 va = *(const double2 *)(ra + c), vb = *(const double2 *)(rbp + c);
+                acc = __fma_rn(va.x, vb.x, acc);
+                acc = __fma_rn(va.y, vb.y, acc);
+            }
+        } else {
+            for (int c = 0; c < w; ++c) acc = __fma_rn(ra[c], rbp[c], acc);
+        }
+    }
+    cp_async_wait<0>();
     if (a < K && b <= a) D.g[pidx(a, b)] = a == b ? __dadd_rn(acc, mu) : acc;
 }
 
@@ -2263,45 +2323,56 @@ __global__ void __launch_bounds__(kGT * kGT) k_dyn_dense_gram(const double *__re
 // stages the next chunk.  The accumulator is written as an FP32 partial tile;
 // k_dyn_gram_reduce adds a tile's partials in split order in FP64, adds mu on
 // the diagonal and writes the packed G that the FP64 Cholesky reads.
+//
+// The rows of a tile are gathered, so what bounds the kernel is the bytes of them
+// in flight: three slots of half a chunk (64 columns of both operands, 64 KB)
+// are filled by asynchronous copies, two of them in flight while the MMAs of the
+// third run.  K = 256: 48 -> 13 us at n = 2,048, 502 -> 96 us at n = 100,000 (2.1 TB/s
+// of gathered rows; one synchronous 128-column chunk at a time before).
 constexpr int kTcRows = 128;                             // tile edge: M = N = 128
-constexpr int kTcCols = 128;                             // columns per chunk: 16 MMAs of K = 8
-constexpr unsigned kTcOperand = kTcRows * kTcCols * 4;   // bytes of one operand chunk
+constexpr int kTcCols = 128;                             // columns per chunk (the unit of a split's share)
+constexpr int kTcHalf = 64;                              // columns per slot: 8 MMAs of K = 8
+constexpr int kTcSlots = 3;
+constexpr int kTcThreads = 256;
+constexpr unsigned kTcOperand = kTcRows * kTcHalf * 4;   // bytes of one operand of a slot
 constexpr unsigned kTcKStride = 128;                     // core matrices adjacent along K
-constexpr unsigned kTcRowStride = (kTcCols / 4) * 128;   // adjacent 8-row groups
+constexpr unsigned kTcRowStride = (kTcHalf / 4) * 128;   // adjacent 8-row groups
+constexpr int kTcPer = kTcRows * kTcHalf / 4 / kTcThreads;   // 16-byte pieces per thread and operand
 
-size_t gram_tc_smem() { return 2 * (size_t)kTcOperand + 1024; }
+size_t gram_tc_smem() { return (size_t)kTcSlots * 2 * kTcOperand + 1024; }
 
-// Rows r0.. r0+127 of A_I, columns c0.. c0+127, into core-matrix order: slot q
-// holds 4 consecutive values of row 8 (q / 256) + q % 8 at column group
-// (q / 8) % 32, so a warp reads 8 rows x 64 contiguous bytes and writes 512
-// contiguous bytes of shared memory.  Rows >= K and columns >= n are zero.
-__device__ __forceinline__ void tc_stage(unsigned char *dst, const float *__restrict__ v32,
-                                         const int *__restrict__ I, int K, long long n, int r0,
-                                         long long c0, bool vec) {
-    for (int q = threadIdx.x; q < kTcRows * kTcCols / 4; q += blockDim.x) {
-        const int r8 = q & 7, kg = (q >> 3) & 31, g = q >> 8;
-        const int row = r0 + g * 8 + r8;
-        const long long col = c0 + kg * 4;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (row < K) {
-            const float *src = v32 + (long long)I[row] * n + col;
-            if (vec && col + 3 < n) {
-                v = *reinterpret_cast<const float4 *>(src);
-            } else {
-                if (col < n) v.x = src[0];
-                if (col + 1 < n) v.y = src[1];
-                if (col + 2 < n) v.z = src[2];
-                if (col + 3 < n) v.w = src[3];
+// Rows r0 .. r0 + 127 of A_I (src: this thread's rows, nullptr beyond K), columns
+// c0 .. c0 + 63, into core-matrix order: piece q holds 4 consecutive values of
+// row 8 (q / 128) + q % 8 at column group (q / 8) % 16, so a warp reads 8 rows x
+// 64 contiguous bytes and writes 512 contiguous bytes of shared memory.  Rows
+// >= K and columns >= n are zero.
+__device__ __forceinline__ void tc_stage(unsigned char *dst, const float *v32, const float *const (&src)[kTcPer],
+                                         long long n, long long c0, bool vec) {
+    const int r8 = threadIdx.x & 7, kg = (threadIdx.x >> 3) & 15, g0 = threadIdx.x >> 7;
+    const long long col = c0 + kg * 4;
+#pragma unroll
+    for (int i = 0; i < kTcPer; ++i) {
+        unsigned char *d = dst + (g0 + 2 * i) * kTcRowStride + kg * kTcKStride + r8 * 16;
+        const bool in = src[i] != nullptr && col < n;
+        if (vec) {                                       // n % 4 == 0: a piece is inside or outside
+            cp_async16(smem_u32(d), in ? src[i] + col : v32, in ? 16 : 0);   // 0: zeros, nothing is read
+        } else {
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (in) {
+                v.x = src[i][col];
+                if (col + 1 < n) v.y = src[i][col + 1];
+                if (col + 2 < n) v.z = src[i][col + 2];
+                if (col + 3 < n) v.w = src[i][col + 3];
             }
+            *reinterpret_cast<float4 *>(d) = v;
         }
-        *reinterpret_cast<float4 *>(dst + g * kTcRowStride + kg * kTcKStride + r8 * 16) = v;
     }
 }
 
-__global__ void __launch_bounds__(128) k_dyn_gram_tc(const float *__restrict__ v32, int n, int K, int S,
-                                                     int vec, Dyn D, float *__restrict__ part, Ctl *ctl) {
+__global__ void __launch_bounds__(kTcThreads) k_dyn_gram_tc(const float *__restrict__ v32, int n, int K, int S,
+                                                            int vec, Dyn D, float *__restrict__ part, Ctl *ctl) {
     extern __shared__ __align__(1024) unsigned char tc_smem[];
-    __shared__ unsigned long long bar;
+    __shared__ unsigned long long bar[kTcSlots];
     __shared__ unsigned tslot;
     __shared__ int s_fail;
     if (ctl->done || ctl->status || ctl->halt) return;
@@ -2309,47 +2380,75 @@ __global__ void __launch_bounds__(128) k_dyn_gram_tc(const float *__restrict__ v
     int ti = 0, tj = t;
     while (tj > ti) { tj -= ti + 1; ++ti; }
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    unsigned char *sa = tc_smem, *sb = tc_smem + kTcOperand;
     const bool diag = ti == tj;
     const int nchunks = (n + kTcCols - 1) / kTcCols;
     const int per = (nchunks + S - 1) / S, ch0 = s * per, ch1 = min(nchunks, ch0 + per);
+    const int nh = max(0, 2 * (ch1 - ch0));              // halves of chunks
     if (tid == 0) {
-        mbar_init(&bar, 1);
+        for (int q = 0; q < kTcSlots; ++q) mbar_init(&bar[q], 1);
         s_fail = 0;
     }
     if (warp == 0) tmem_alloc(&tslot, kTcRows);
+    // this thread's rows of both operands
+    const float *srca[kTcPer], *srcb[kTcPer];
+#pragma unroll
+    for (int i = 0; i < kTcPer; ++i) {
+        const int row = ((tid >> 7) + 2 * i) * 8 + (tid & 7);
+        const int ra = ti * kTcRows + row, rb = tj * kTcRows + row;
+        srca[i] = ra < K ? v32 + (long long)D.I[ra] * n : nullptr;
+        srcb[i] = rb < K && !diag ? v32 + (long long)D.I[rb] * n : nullptr;
+    }
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
     const unsigned tmem = tslot;
     const unsigned idesc = idesc_tf32_f32(kTcRows, kTcRows);
-    unsigned phase = 0;
-    for (int c = ch0; c < ch1; ++c) {
-        tc_stage(sa, v32, D.I, K, n, ti * kTcRows, (long long)c * kTcCols, vec != 0);
-        if (!diag) tc_stage(sb, v32, D.I, K, n, tj * kTcRows, (long long)c * kTcCols, vec != 0);
-        fence_proxy_async_smem();
-        __syncthreads();
-        tc_fence_after_sync();
-        if (tid == 0) {
-            const unsigned a0 = smem_u32(sa), b0 = smem_u32(diag ? sa : sb);
-            for (int k = 0; k < kTcCols / 8; ++k)      // K = 8 TF32 values = 2 core matrices
-                mma_tf32(tmem, umma_desc(a0 + 256u * k, kTcKStride, kTcRowStride),
-                         umma_desc(b0 + 256u * k, kTcKStride, kTcRowStride), idesc,
-                         (c > ch0 || k > 0) ? 1u : 0u);
-            mma_commit(&bar);
+    auto fill = [&](int h) {
+        if (h < nh) {
+            unsigned char *sa = tc_smem + (size_t)(h % kTcSlots) * 2 * kTcOperand;
+            const long long c0 = (long long)ch0 * kTcCols + (long long)h * kTcHalf;
+            tc_stage(sa, v32, srca, n, c0, vec != 0);
+            if (!diag) tc_stage(sa + kTcOperand, v32, srcb, n, c0, vec != 0);
         }
-        if (!mbar_wait_bounded(&bar, phase, kWaitTries)) atomicOr(&s_fail, 1);
-        phase ^= 1u;
-        __syncthreads();                               // the chunk's operands are free again
-        if (s_fail) break;
+        cp_async_commit();
+    };
+    fill(0);
+    fill(1);
+    bool ok = true;
+    int last = -1;                                       // the last half whose MMAs were issued
+    for (int h = 0; h < nh; ++h) {
+        last = h;
+        cp_async_wait<1>();                              // half h has landed (this thread's copies)
+        fence_proxy_async_smem();
+        __syncthreads();                                 // everyone's
+        if (tid == 0) {
+            tc_fence_after_sync();
+            const unsigned a0 = smem_u32(tc_smem + (size_t)(h % kTcSlots) * 2 * kTcOperand);
+            const unsigned b0 = diag ? a0 : a0 + kTcOperand;
+            for (int k = 0; k < kTcHalf / 8; ++k)        // K = 8 TF32 values = 2 core matrices
+                mma_tf32(tmem, umma_desc(a0 + 256u * k, kTcKStride, kTcRowStride),
+                         umma_desc(b0 + 256u * k, kTcKStride, kTcRowStride), idesc, (h > 0 || k > 0) ? 1u : 0u);
+            mma_commit(&bar[h % kTcSlots]);
+        }
+        // the slot of half h + 2 is free when the MMAs of half h - 1 are done
+        if (h > 0) {
+            if (!mbar_wait_bounded(&bar[(h - 1) % kTcSlots], ((h - 1) / kTcSlots) & 1, kWaitTries)) ok = false;
+            if (!__syncthreads_and(ok)) break;
+        }
+        fill(h + 2);
     }
-    if (s_fail && tid == 0) mbar_wait_bounded(&bar, phase ^ 1u, kWaitTries);   // the MMAs in flight
+    cp_async_wait<0>();
+    // the last MMAs (they complete in order); after a failed wait this is the one more
+    // bounded wait for what is in flight
+    if (last >= 0 && !mbar_wait_bounded(&bar[last % kTcSlots], (last / kTcSlots) & 1, kWaitTries)) ok = false;
+    if (!ok) atomicOr(&s_fail, 1);
+    __syncthreads();
     tc_fence_after_sync();
-    if (!s_fail) {
+    if (!s_fail && warp < 4) {
         float *P = part + ((long long)t * S + s) * kTcRows * kTcRows + (long long)(warp * 32 + lane) * kTcRows;
         for (int c0 = 0; c0 < kTcRows; c0 += 32) {
             unsigned v[32];
-            if (ch1 > ch0) {
+            if (nh > 0) {
                 tmem_ld_32cols(tmem + ((unsigned)(warp * 32) << 16) + (unsigned)c0, v);
             } else {
 #pragma unroll
@@ -2620,6 +2719,7 @@ __global__ void __launch_bounds__(256) k_dyn_dense_scatter(const double *__restr
         return;
     }
     if (!wood)
+#pragma unroll 4
         for (int a = threadIdx.x; a < K; a += blockDim.x) {
             rows[a] = D.I[a];
             ys[a] = as<T>(D.y[a]);
@@ -3280,13 +3380,18 @@ int residual_grid(rorbk_ctx *h) {
     return std::max(1, std::min(per_sm, per_sm32 > 0 ? per_sm32 : per_sm)) * h->num_sms;
 }
 
+// The rings of k_residual_dense: long stages and many of them for few pairs.
+constexpr int kDrMaxPairs = 8;
 template <typename T, typename V>
 static void configure_residual_dense() {
-    const int sm = (int)dense_res_smem<T, V>();
-    cudaFuncSetAttribute(k_residual_dense<T, V, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    cudaFuncSetAttribute(k_residual_dense<T, V, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    cudaFuncSetAttribute(k_residual_dense<T, V, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    cudaFuncSetAttribute(k_residual_dense<T, V, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    cudaFuncSetAttribute(k_residual_dense<T, V, 512, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)dense_res_smem<T, V, 512, 8>(1));
+    cudaFuncSetAttribute(k_residual_dense<T, V, 512, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)dense_res_smem<T, V, 512, 6>(2));
+    cudaFuncSetAttribute(k_residual_dense<T, V, 256, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)dense_res_smem<T, V, 256, 6>(4));
+    cudaFuncSetAttribute(k_residual_dense<T, V, 256, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)dense_res_smem<T, V, 256, 3>(kDrMaxPairs));
 }
 
 template <int NR>
@@ -3419,15 +3524,14 @@ void launch_dense_gram(rorbk_ctx *h, Ctl *ctl, int tensor_cores) {
     if (tensor_cores) {
         const int tiles = h->gram_tiles, S = h->gram_splits;
         const int vec = (h->n % 4 == 0) && ((reinterpret_cast<uintptr_t>(h->val32) & 15) == 0);
-        k_dyn_gram_tc<<<dim3(tiles, S), 128, gram_tc_smem(), h->stream>>>(h->val32, (int)h->n, K, S, vec,
+        k_dyn_gram_tc<<<dim3(tiles, S), kTcThreads, gram_tc_smem(), h->stream>>>(h->val32, (int)h->n, K, S, vec,
                                                                        dyn_bufs(h), h->gram_part, ctl);
         const long long np = (long long)K * (K + 1) / 2;
         k_dyn_gram_reduce<<<(int)std::min<long long>(4LL * h->num_sms, (np + 255) / 256), 256, 0, h->stream>>>(
             h->gram_part, K, S, h->mu, dyn_bufs(h), ctl);
     } else {
-        const int T16 = (K + kGT - 1) / kGT;
-        k_dyn_dense_gram<<<T16 * (T16 + 1) / 2, kGT * kGT, 0, h->stream>>>(h->val, (int)h->n, K, h->mu,
-                                                                          dyn_bufs(h), ctl);
+        const int t = (K + 2 * kGa - 1) / (2 * kGa);      // pairs of 4-row groups
+        k_dyn_dense_gram<<<t * (t + 1), 32, 0, h->stream>>>(h->val, (int)h->n, K, h->mu, dyn_bufs(h), ctl);
     }
 }
 
@@ -3564,8 +3668,17 @@ const double *row_major<double>(const rorbk_ctx *h) { return h->val; }
 template <>
 const float *row_major<float>(const rorbk_ctx *h) { return h->val32; }
 
-// The residual kernel for this handle's format.  Dense: as many chain warps per
-// SM as there are groups of 32 rows for it (8 at most).
+template <typename T, typename V, int RB, int ST>
+static void residual_dense_launch(rorbk_ctx *h, const T *b, const T *x, T *r, Ctl *ctl, int finalize, int g, int W) {
+    k_residual_dense<T, V, RB, ST><<<g, 512, dense_res_smem<T, V, RB, ST>(W), h->stream>>>(
+        row_major<V>(h), (int)h->m, (int)h->n, h->K, b, x, r, h->partials, h->hist1, ctl, finalize, W);
+}
+
+// The residual kernel for this handle's format.  Dense: as many pairs of warps
+// per SM as there are groups of 32 rows for it.  From five on (four keep the
+// FP64 unit busy) the count that leaves the fewest idle in the last round: a
+// lone chain runs at a quarter of the SM's FP64 rate (200,000 rows, 42 groups
+// per SM: 775 us with 8 pairs, 732 with 7).
 template <typename T, typename V>
 static void residual_launch(rorbk_ctx *h, const Mat<T> &A, const T *b, const T *x, T *r, Ctl *ctl,
                             int finalize) {
@@ -3573,14 +3686,16 @@ static void residual_launch(rorbk_ctx *h, const Mat<T> &A, const T *b, const T *
         k_residual<T, V><<<h->grid_res, 256, 0, h->stream>>>(A, b, x, r, h->partials, h->hist1, ctl, finalize);
         return;
     }
-    const int m = (int)h->m, n = (int)h->n, nsl = (m + 31) / 32, g = std::min(h->grid_res, nsl);
-    const int per = (nsl + h->grid_res - 1) / h->grid_res;
-    const size_t sm = dense_res_smem<T, V>();
-    const V *v = row_major<V>(h);
-    if (per > 4) k_residual_dense<T, V, 8><<<g, 256, sm, h->stream>>>(v, m, n, h->K, b, x, r, h->partials, h->hist1, ctl, finalize);
-    else if (per > 2) k_residual_dense<T, V, 4><<<g, 256, sm, h->stream>>>(v, m, n, h->K, b, x, r, h->partials, h->hist1, ctl, finalize);
-    else if (per > 1) k_residual_dense<T, V, 2><<<g, 256, sm, h->stream>>>(v, m, n, h->K, b, x, r, h->partials, h->hist1, ctl, finalize);
-    else k_residual_dense<T, V, 1><<<g, 256, sm, h->stream>>>(v, m, n, h->K, b, x, r, h->partials, h->hist1, ctl, finalize);
+    const int nsl = (int)((h->m + 31) / 32), g = std::min(h->grid_res, nsl), per = (nsl + g - 1) / g;
+    if (per == 1) residual_dense_launch<T, V, 512, 8>(h, b, x, r, ctl, finalize, g, 1);
+    else if (per == 2) residual_dense_launch<T, V, 512, 6>(h, b, x, r, ctl, finalize, g, 2);
+    else if (per <= 4) residual_dense_launch<T, V, 256, 6>(h, b, x, r, ctl, finalize, g, per);
+    else {
+        int W = kDrMaxPairs;
+        for (int c = kDrMaxPairs - 1; c >= 5; --c)
+            if ((per + c - 1) / c * c < (per + W - 1) / W * W) W = c;
+        residual_dense_launch<T, V, 256, 3>(h, b, x, r, ctl, finalize, g, W);
+    }
 }
 
 template <typename T>
@@ -3592,7 +3707,7 @@ void launch_iteration_t(rorbk_ctx *h, const T *b, T *x, T *r, Ctl *ctl, int use_
         const int gr = (h->smax + 31) / 32;
         const int gs = std::max(1, std::min(8 * h->num_sms, (int)((h->n + kSdThreads - 1) / kSdThreads)));
         for (int l = 0; l < kDenseStatic; ++l) {
-            k_sd_rows<T><<<gr, 32, sd_rows_smem<T>(), h->stream>>>(A, b, x, rl, ctl, l);
+            k_sd_rows<T><<<gr, 64, sd_rows_smem<T>(), h->stream>>>(A, b, x, rl, ctl, l);
             k_sd_apply<T><<<gr, 32, 0, h->stream>>>(A, rl, yy, ctl, l);
             k_sd_scatter<T><<<gs, kSdThreads, 0, h->stream>>>(A, rl, yy, x, ctl, l);
             if (h->n_wood) k_sd_wood<T><<<gs, kSdThreads, 0, h->stream>>>(A, yy, x, ctl, l);
