@@ -168,7 +168,7 @@ __device__ __forceinline__ double widen(float f) {
 }
 __device__ __forceinline__ double widen(double d) { return d; }
 
-__device__ __forceinline__ int next_pow2(int v) {
+__host__ __device__ __forceinline__ int next_pow2(int v) {
     int p = 1;
     while (p < v) p <<= 1;
     return p;

@@ -98,6 +98,8 @@ struct StaticOps {
     double *w_diag = nullptr;   // [m] W_ii for uncoupled rows
     int *s_pos = nullptr;       // [m] position of a row in its S_t, or -1
     float *w_ss32 = nullptr, *w_diag32 = nullptr;  // FP32 copies (mixed)
+    long long w_total = 0, wood_total = 0;         // entries of w_ss and of the s >= n operators
+    int max_coupled = 0;                           // largest |S_t|
 };
 
 // Per-block column-sorted copy of the block's nonzeros, used for the
@@ -113,6 +115,10 @@ struct BlockT {
     int *seg = nullptr;         // segment (distinct column) start positions
     int *seg_ptr = nullptr;     // [k] segment count of block t; its segments
                                 // start at seg[row_ptr[off[t]] ...]
+    unsigned char *coupled = nullptr;   // [m] rows that share a column with another of their block
+    int *ncoupled = nullptr;            // [k] their number
+    int max_entries = 0;                // entries of the largest block (sparse A)
+    int total_segs = 0;                 // distinct (block, column) pairs
 };
 
 // Device memory owned jointly by a handle and its clones (rorbk_clone): the

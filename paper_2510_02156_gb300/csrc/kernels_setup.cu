@@ -62,10 +62,14 @@ __global__ void k_block_nz(const int *__restrict__ rowptr, const int *__restrict
 }
 
 // ---------------------------------------------------------- block transpose
-// One block of threads per static block t.  Entry p of the block's CSR range
-// lands at rank(p) = #entries with a smaller column + #entries in earlier
-// rows with the same column, found by binary searches in every row of the
-// block (rows hold ascending columns).
+// One block of threads per static block t.  The block's entries are ordered by
+// (column, row): up to kBtSort entries by a bitonic sort of (column, position)
+// keys in shared memory; a larger
+// block places entry p at rank(p) = #entries with a smaller column + #entries in
+// earlier rows with the same column, found by binary searches in every row of
+// the block (rows hold ascending columns).
+constexpr int kBtSort = 8192;
+
 __device__ __forceinline__ int lower_bound_col(const int *col, int lo, int hi, int c) {
     while (lo < hi) {
         int mid = (lo + hi) >> 1;
@@ -74,13 +78,24 @@ __device__ __forceinline__ int lower_bound_col(const int *col, int lo, int hi, i
     return lo;
 }
 
+// Last row i in [lo, hi) with rowptr[i] <= p.
+__device__ __forceinline__ int row_of_entry(const int *rowptr, int lo, int hi, int p) {
+    while (hi - lo > 1) {
+        int mid = (lo + hi) >> 1;
+        if (rowptr[mid] <= p) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
+// sort: entries that the launch's dynamic shared memory holds (a power of two).
 __global__ void k_block_transpose(const int *__restrict__ rowptr, const int *__restrict__ col,
                                   const double *__restrict__ val, const int *__restrict__ off,
                                   int *__restrict__ bt_col, uint16_t *__restrict__ bt_row,
                                   double *__restrict__ bt_val, uint16_t *__restrict__ bt_off,
                                   int *__restrict__ bt_seg,
                                   int *__restrict__ nseg_out, unsigned char *__restrict__ coupled,
-                                  int *__restrict__ ncoupled_out) {
+                                  int *__restrict__ ncoupled_out, int sort) {
+    extern __shared__ unsigned long long bt_keys[];
     __shared__ int scan_scratch[33];
     __shared__ unsigned char flag[kMaxBlockRows];
     const int t = blockIdx.x;
@@ -88,27 +103,37 @@ __global__ void k_block_transpose(const int *__restrict__ rowptr, const int *__r
     const int p0 = rowptr[r0], E = rowptr[r1] - p0;
     for (int a = threadIdx.x; a < s; a += blockDim.x) flag[a] = 0;
 
-    for (int e = threadIdx.x; e < E; e += blockDim.x) {
-        int p = p0 + e;
-        int c = col[p];
-        int lo = r0, hi = r1;                    // row of entry p: last i with rowptr[i] <= p
-        while (hi - lo > 1) {
-            int mid = (lo + hi) >> 1;
-            if (rowptr[mid] <= p) lo = mid; else hi = mid;
+    if (E <= sort) {
+        const int np = next_pow2(max(E, 1));
+        for (int e = threadIdx.x; e < np; e += blockDim.x)
+            bt_keys[e] = e < E ? (unsigned long long)(unsigned)col[p0 + e] << 32 | (unsigned)e : ~0ull;
+        __syncthreads();
+        block_bitonic_sort(bt_keys, np);
+        for (int q = threadIdx.x; q < E; q += blockDim.x) {
+            const int e = (int)(unsigned)bt_keys[q], dst = p0 + q;
+            bt_col[dst] = (int)(bt_keys[q] >> 32);
+            bt_row[dst] = (uint16_t)(row_of_entry(rowptr, r0, r1, p0 + e) - r0);
+            bt_val[dst] = val[p0 + e];
+            bt_off[dst] = (uint16_t)e;
         }
-        int a = lo - r0;
-        int rank = 0;
-        for (int b = 0; b < s; ++b) {
-            int q0 = rowptr[r0 + b], q1 = rowptr[r0 + b + 1];
-            int lb = lower_bound_col(col, q0, q1, c);
-            rank += lb - q0;
-            if (b < a && lb < q1 && col[lb] == c) rank += 1;
+    } else {
+        for (int e = threadIdx.x; e < E; e += blockDim.x) {
+            int p = p0 + e;
+            int c = col[p];
+            int a = row_of_entry(rowptr, r0, r1, p) - r0;
+            int rank = 0;
+            for (int b = 0; b < s; ++b) {
+                int q0 = rowptr[r0 + b], q1 = rowptr[r0 + b + 1];
+                int lb = lower_bound_col(col, q0, q1, c);
+                rank += lb - q0;
+                if (b < a && lb < q1 && col[lb] == c) rank += 1;
+            }
+            int dst = p0 + rank;
+            bt_col[dst] = c;
+            bt_row[dst] = (uint16_t)a;
+            bt_val[dst] = val[p];
+            bt_off[dst] = (uint16_t)e;
         }
-        int dst = p0 + rank;
-        bt_col[dst] = c;
-        bt_row[dst] = (uint16_t)a;
-        bt_val[dst] = val[p];
-        bt_off[dst] = (uint16_t)e;
     }
     __syncthreads();
 
@@ -140,6 +165,15 @@ __global__ void k_block_transpose(const int *__restrict__ rowptr, const int *__r
         nseg_out[t] = nseg;
         ncoupled_out[t] = tot;
     }
+}
+
+// New values of the same pattern: entry q of a block's column-sorted copy is the
+// block's entry bt_off[q] (blocks of at most 65,536 entries).  262,144 rows: 14 us
+// where the ranking by binary searches took 1,756.
+__global__ void k_block_refill(const int *__restrict__ blk_nz, const double *__restrict__ val,
+                               const uint16_t *__restrict__ bt_off, double *__restrict__ bt_val) {
+    const int p0 = blk_nz[blockIdx.x], p1 = blk_nz[blockIdx.x + 1];
+    for (int q = p0 + threadIdx.x; q < p1; q += blockDim.x) bt_val[q] = val[p0 + bt_off[q]];
 }
 
 // A dense A (every entry stored, rows of n entries): block t's column-sorted
@@ -232,6 +266,31 @@ __global__ void k_row_norms(const int *__restrict__ rowptr, const V *__restrict_
     }
 }
 
+// The same over the SELL copy (a warp's rows are of one length, its loads
+// coalesced; values stored as FP32 widen exactly).
+template <typename V>
+__global__ void k_row_norms_sell(int nslices, const long long *__restrict__ ptr, const int *__restrict__ srow,
+                                 const int *__restrict__ srlen, const V *__restrict__ sval, double *__restrict__ rn) {
+    const long long slot = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (slot >= (long long)nslices * 32) return;
+    const int row = srow[slot], len = srlen[slot];
+    if (row < 0) return;
+    const V *v = sval + ptr[slot >> 5] + (slot & 31);
+    double g = 0.0;
+    for (int j = 0; j < len; j += 8) {                // eight loads ahead of the chain
+        V x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = j + u < len ? v[32LL * (j + u)] : V(0);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (j + u < len) {
+                const double w = widen(x[u]);         // integer operations: a conversion takes the FP64 unit
+                g = __fma_rn(w, w, g);
+            }
+    }
+    rn[row] = g;
+}
+
 // ------------------------------------------------------------ device scans
 // Exclusive scan of n ints in place (n < 2^31), three launches.
 __global__ void k_scan_tiles(const int *__restrict__ in, int *__restrict__ out,
@@ -303,28 +362,76 @@ __global__ void k_centroid_fill(const int *__restrict__ rowptr, const int *__res
 
 // Row t of G = Abar Abar^T, one warp per block t: columns c of Abar_t in
 // ascending order, G(t, j) += Abar_tc * Abar_jc over the blocks j of column c
-// (distinct j inside one column, so the lanes never collide).
-__global__ void k_centroid_gram(const int *__restrict__ rowptr, const int *__restrict__ off,
-                                const int *__restrict__ bt_col, const double *__restrict__ bt_val,
-                                const int *__restrict__ bt_seg, const int *__restrict__ nseg,
-                                int k, const int *__restrict__ colptr,
-                                const int *__restrict__ cb, const double *__restrict__ cv,
-                                double *__restrict__ G) {
-    int lane = threadIdx.x & 31;
-    int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (t >= k) return;
-    int p0 = rowptr[off[t]], pend = rowptr[off[t + 1]];
-    double *Gt = G + (long long)t * k;
-    for (int g = 0; g < nseg[t]; ++g) {
-        int q = bt_seg[p0 + g];
-        int c = bt_col[q];
-        double v = segment_sum(bt_val, bt_col, q, pend);
-        for (int e = colptr[c] + lane; e < colptr[c + 1]; e += 32) {
-            int j = cb[e];
-            Gt[j] = __fma_rn(v, cv[e], Gt[j]);
+// (distinct j inside one column, so the lanes never collide).  The row is
+// accumulated in shared memory (SM; rows too long for it in G itself), the
+// columns' data are read 32 columns at a time, and the entries of the next eight
+// columns are in flight while those of eight are added.  262,144 columns, k =
+// 1,024: 2,420 -> 590 us (about 480 cycles per column and block: the read,
+// multiply-add and write of the row's entries, one column after the other).
+template <bool SM>
+__global__ void __launch_bounds__(32) k_centroid_gram(const int *__restrict__ rowptr, const int *__restrict__ off,
+                                                      const int *__restrict__ bt_col, const double *__restrict__ bt_val,
+                                                      const int *__restrict__ bt_seg, const int *__restrict__ nseg,
+                                                      int k, const int *__restrict__ colptr,
+                                                      const int *__restrict__ cb, const double *__restrict__ cv,
+                                                      double *__restrict__ G) {
+    extern __shared__ double g_row[];
+    constexpr int kU = 8;
+    __shared__ double sv[32];
+    __shared__ int2 se[32];
+    const int lane = threadIdx.x, t = blockIdx.x;
+    const int p0 = rowptr[off[t]], pend = rowptr[off[t + 1]], ns = nseg[t];
+    double *Gt = SM ? g_row : G + (long long)t * k;
+    for (int j = lane; j < k; j += 32) Gt[j] = 0.0;
+    __syncwarp();
+    for (int base = 0; base < ns; base += 32) {
+        double v = 0.0;
+        int e0 = 0, e1 = 0;
+        if (base + lane < ns) {
+            const int q = bt_seg[p0 + base + lane], c = bt_col[q];
+            v = segment_sum(bt_val, bt_col, q, pend);
+            e0 = colptr[c];
+            e1 = colptr[c + 1];
         }
+        sv[lane] = v;
+        se[lane] = make_int2(e0, e1);
+        const bool long_col = __any_sync(0xffffffffu, e1 - e0 > 32);
         __syncwarp();
+        int jn[kU];
+        double an[kU], vn[kU];
+        auto fetch = [&](int u0) {
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int2 e = se[(u0 + u) & 31];
+                const bool in = u0 + u < 32 && e.x + lane < e.y;
+                jn[u] = in ? cb[e.x + lane] : -1;
+                an[u] = in ? cv[e.x + lane] : 0.0;
+                vn[u] = sv[(u0 + u) & 31];
+            }
+        };
+        fetch(0);
+        for (int u0 = 0; u0 < 32 && base + u0 < ns; u0 += kU) {
+            int jc[kU];
+            double ac[kU], vc[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                jc[u] = jn[u];
+                ac[u] = an[u];
+                vc[u] = vn[u];
+            }
+            fetch(u0 + kU);
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                if (jc[u] >= 0) Gt[jc[u]] = __fma_rn(vc[u], ac[u], Gt[jc[u]]);
+                if (long_col)                        // a column in more than 32 blocks
+                    for (int e = se[u0 + u].x + 32 + lane; e < se[u0 + u].y; e += 32)
+                        Gt[cb[e]] = __fma_rn(vc[u], cv[e], Gt[cb[e]]);
+                __syncwarp();
+            }
+        }
     }
+    if (SM)
+        for (int j = lane; j < k; j += 32) G[(long long)t * k + j] = g_row[j];
 }
 
 // Dense centroids: Abar (k x n) row t = sum of the block's rows in order.
@@ -351,19 +458,27 @@ __global__ void k_centroid_gram_dense(const double *__restrict__ Abar, int k, in
     G[(long long)t * k + j] = s;
 }
 
+// |Abar_t|.
+__global__ void k_centroid_norms(const double *__restrict__ G, int k, double *__restrict__ nrm) {
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < k; t += gridDim.x * blockDim.x)
+        nrm[t] = sqrt(G[(long long)t * k + t]);
+}
+
 // sum_j C(t, j), C(t,t) = 1, C(t,j) = 0 when either centroid is zero.
-__global__ void k_crowsum(const double *__restrict__ G, int k, double *__restrict__ rowsum) {
+__global__ void k_crowsum(const double *__restrict__ G, const double *__restrict__ nrm, int k,
+                          double *__restrict__ rowsum) {
     int lane = threadIdx.x & 31;
     int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (t >= k) return;
-    double nt = sqrt(G[(long long)t * k + t]);
+    const double nt = nrm[t];
     double s = 0.0;
+#pragma unroll 4
     for (int j = lane; j < k; j += 32) {
-        double nj = sqrt(G[(long long)j * k + j]);
+        const double nj = nrm[j], g = G[(long long)t * k + j];
         double cij;
         if (j == t) cij = 1.0;
         else if (nt == 0.0 || nj == 0.0) cij = 0.0;
-        else cij = fabs(G[(long long)t * k + j]) / (nt * nj);
+        else cij = fabs(g) / (nt * nj);
         s += cij;
     }
     s = warp_sum(s);
@@ -371,21 +486,41 @@ __global__ void k_crowsum(const double *__restrict__ G, int k, double *__restric
 }
 
 // Pbar_t = exp(-2 rowsum_t / n); cdf_t = Pbar_0 + ... + Pbar_t summed in
-// order by one thread (the normalisation of P is folded into the sampler).
-__global__ void k_proposal(const double *__restrict__ rowsum, int k, double n,
-                           double *__restrict__ cdf, double *__restrict__ pbar) {
-    for (int t = threadIdx.x; t < k; t += blockDim.x) {
-        const double v = exp(-2.0 * rowsum[t] / n);
-        cdf[t] = v;
-        pbar[t] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int t = 0; t < k; ++t) {
-            s += cdf[t];
-            cdf[t] = s;
+// order by one thread (the normalisation of P is folded into the sampler) over
+// chunks that the block holds in shared memory.
+constexpr int kPropChunk = 2048;
+__global__ void __launch_bounds__(1024) k_proposal(const double *__restrict__ rowsum, int k, double n,
+                                                   double *__restrict__ cdf, double *__restrict__ pbar) {
+    __shared__ double c[kPropChunk];
+    double s = 0.0;
+    for (int base = 0; base < k; base += kPropChunk) {
+        const int w = min(kPropChunk, k - base);
+        for (int t = threadIdx.x; t < w; t += blockDim.x) {
+            const double v = exp(-2.0 * rowsum[base + t] / n);
+            c[t] = v;
+            pbar[base + t] = v;
         }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int t = 0;
+            for (; t + 8 <= w; t += 8) {
+                double v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] = c[t + u];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    s += v[u];
+                    c[t + u] = s;
+                }
+            }
+            for (; t < w; ++t) {
+                s += c[t];
+                c[t] = s;
+            }
+        }
+        __syncthreads();
+        for (int t = threadIdx.x; t < w; t += blockDim.x) cdf[base + t] = c[t];
+        __syncthreads();
     }
 }
 
@@ -394,7 +529,7 @@ __global__ void k_proposal(const double *__restrict__ rowsum, int k, double n,
 // column: Linv_jj = 1/L_jj, Linv_ij = -(sum_{c=j}^{i-1} L_ic Linv_cj) / L_ii, c
 // ascending; then W_ij = sum_{c >= max(i,j)} Linv_ci Linv_cj (c ascending).
 // All threads of the block take part.
-__device__ void spd_inverse_from_factor(double *G, double *Li, int nS) {
+__device__ __forceinline__ void spd_inverse_from_factor(double *G, double *Li, int nS) {
     for (int j = threadIdx.x; j < nS; j += blockDim.x) {
         for (int i = 0; i < j; ++i) Li[(long long)i * nS + j] = 0.0;
         Li[(long long)j * nS + j] = 1.0 / G[(long long)j * nS + j];
@@ -427,6 +562,7 @@ __device__ void spd_inverse_from_factor(double *G, double *Li, int nS) {
 // flags and S offsets; outputs W on S (row-major |S|^2 at w_ss + w_ptr[t]),
 // W_ii for uncoupled rows, and s_idx / s_pos.  Linv scratch has the layout of
 // w_ss.
+constexpr int kSoStage = 8192;        // entries of a block staged for the merges of its rows
 __global__ void k_static_ops(const int *__restrict__ rowptr, const int *__restrict__ col,
                              const double *__restrict__ val, const int *__restrict__ off,
                              double mu, const unsigned char *__restrict__ coupled,
@@ -434,7 +570,10 @@ __global__ void k_static_ops(const int *__restrict__ rowptr, const int *__restri
                              uint16_t *__restrict__ s_idx, int *__restrict__ s_pos,
                              double *__restrict__ w_ss, double *__restrict__ w_diag,
                              double *__restrict__ linv, const long long *__restrict__ wood_ptr,
-                             int *__restrict__ status, int gram_ready) {
+                             int *__restrict__ status, int gram_ready, const double *__restrict__ rn, int stage,
+                             int mat) {
+    extern __shared__ double so_val[];           // [stage] values, then columns, of the block's entries;
+                                                 // then, over them, two matrices of mat doubles together
     __shared__ int scan_scratch[33];
     __shared__ int bad;
     __shared__ double gdiag[kMaxBlockRows];
@@ -462,10 +601,7 @@ __global__ void k_static_ops(const int *__restrict__ rowptr, const int *__restri
         if (a < s) {
             s_pos[r0 + a] = f ? cnt + pre : -1;
             if (f) s_idx[sb + cnt + pre] = (uint16_t)a;
-            int p0 = rowptr[r0 + a], p1 = rowptr[r0 + a + 1];
-            double g = 0.0;
-            for (int p = p0; p < p1; ++p) g = __fma_rn(val[p], val[p], g);
-            g = __dadd_rn(g, mu);
+            double g = __dadd_rn(rn[r0 + a], mu);    // the row's fused chain (k_row_norms)
             gdiag[a] = g;
             if (!f) {
                 if (!(g > 0.0)) { bad = 1; g = 1.0; }
@@ -482,6 +618,18 @@ __global__ void k_static_ops(const int *__restrict__ rowptr, const int *__restri
         // G on S: merges of the coupled rows (lower triangle + diagonal),
         // unless k_dense_static_gram formed it already (gram_ready)
         long long pairs = gram_ready ? 0 : (long long)nS * (nS + 1) / 2;
+        // a merge of two rows is a chain of dependent loads: from shared memory
+        // where the block's entries fit
+        const int b0 = rowptr[r0], E = rowptr[r0 + s] - b0;
+        const bool st = pairs > 0 && E <= stage;
+        int *so_col = (int *)(so_val + stage);
+        if (st) {
+            for (int e = threadIdx.x; e < E; e += blockDim.x) {
+                so_val[e] = val[b0 + e];
+                so_col[e] = col[b0 + e];
+            }
+            __syncthreads();
+        }
         for (long long idx = threadIdx.x; idx < pairs; idx += blockDim.x) {
             int i = (int)((sqrt(8.0 * (double)idx + 1.0) - 1.0) * 0.5);
             while ((long long)(i + 1) * (i + 2) / 2 <= idx) ++i;
@@ -489,14 +637,27 @@ __global__ void k_static_ops(const int *__restrict__ rowptr, const int *__restri
             int j = (int)(idx - (long long)i * (i + 1) / 2);
             int a = s_idx[sb + i], b = s_idx[sb + j];
             double g;
+            const int pa = rowptr[r0 + a], ea = rowptr[r0 + a + 1], pb = rowptr[r0 + b], eb = rowptr[r0 + b + 1];
             if (i == j) g = gdiag[a];
-            else g = row_merge_dot(col, val, rowptr[r0 + a], rowptr[r0 + a + 1],
-                                   rowptr[r0 + b], rowptr[r0 + b + 1]);
+            else if (st) g = row_merge_dot(so_col, so_val, pa - b0, ea - b0, pb - b0, eb - b0);
+            else g = row_merge_dot(col, val, pa, ea, pb, eb);
             G[(long long)i * nS + j] = g;
         }
         __syncthreads();
-        block_cholesky(G, nS, nS, &bad);
-        spd_inverse_from_factor(G, Li, nS);
+        if (2LL * nS * nS <= mat) {
+            // the factor and the inverse are chains of dependent accesses: in
+            // shared memory (over the staged entries) where both matrices fit
+            double *Gs = so_val, *Ls = so_val + nS * nS;
+            for (int idx = threadIdx.x; idx < nS * nS; idx += blockDim.x) Gs[idx] = idx / nS >= idx % nS ? G[idx] : 0.0;
+            __syncthreads();
+            block_cholesky(Gs, nS, nS, &bad);
+            spd_inverse_from_factor(Gs, Ls, nS);
+            __syncthreads();
+            for (int idx = threadIdx.x; idx < nS * nS; idx += blockDim.x) G[idx] = Gs[idx];
+        } else {
+            block_cholesky(G, nS, nS, &bad);
+            spd_inverse_from_factor(G, Li, nS);
+        }
     }
     __syncthreads();
     if (threadIdx.x == 0 && bad) set_status(status, kDevNotSpd);
@@ -587,7 +748,7 @@ __global__ void k_sell_fill(const int *__restrict__ rowptr, const int *__restric
     for (int j = 0; j < (int)((ptr[s + 1] - ptr[s]) >> 5); ++j) {
         const long long d = base + 32LL * j;
         const bool in = j < len;
-        scol[d] = in ? col[p0 + j] : 0;
+        if (scol) scol[d] = in ? col[p0 + j] : 0;
         if (sval) sval[d] = in ? val[p0 + j] : 0.0;
         if (sval32) sval32[d] = in ? val32[p0 + j] : 0.0f;
     }
@@ -676,17 +837,38 @@ __global__ void k_col_gather(const int *__restrict__ slot, const int *__restrict
 
 // ---------------------------------------------------------------- driver
 // Device scratch of one set-up pass, freed when the pass ends (after the
-// stream has drained).
+// stream has drained).  With a size, one allocation that the buffers share (a
+// refresh knows its sizes; an allocation and its release cost tens of
+// microseconds each).
 struct Scratch {
     cudaStream_t s;
     std::vector<void *> p;
-    explicit Scratch(cudaStream_t s_) : s(s_) {}
+    char *arena = nullptr;
+    size_t left = 0;
+    explicit Scratch(cudaStream_t s_, size_t bytes = 0) : s(s_) {
+        if (!bytes) return;
+        if (cudaMalloc(&arena, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            arena = nullptr;
+            return;
+        }
+        p.push_back(arena);
+        left = bytes;
+    }
     Scratch(const Scratch &) = delete;
     Scratch &operator=(const Scratch &) = delete;
+    static size_t room(size_t bytes) { return (std::max<size_t>(bytes, 16) + 255) & ~(size_t)255; }
     template <typename T>
     T *get(size_t count) {
+        const size_t need = room(count * sizeof(T));
+        if (need <= left) {
+            void *q = arena;
+            arena += need;
+            left -= need;
+            return (T *)q;
+        }
         void *q = nullptr;
-        if (cudaMalloc(&q, std::max<size_t>(count * sizeof(T), 16)) != cudaSuccess) {
+        if (cudaMalloc(&q, need) != cudaSuccess) {
             cudaGetLastError();
             return nullptr;
         }
@@ -708,17 +890,19 @@ static bool keep(rorbk_ctx *h, T *&ptr, size_t count) {
     return ptr != nullptr;
 }
 
-// Exclusive scan of n ints in place; *grand_total_host receives the sum.
-static rorbk_status scan_device(rorbk_ctx *h, int *d, long long n, int *grand_total_host) {
+// Exclusive scan of n ints in place; *grand_total_host receives the sum (NULL:
+// not asked for, and not waited for; the scratch is sc's).
+static long long scan_tiles(long long n) { return (n + 255) / 256; }
+static rorbk_status scan_device(rorbk_ctx *h, Scratch &sc, int *d, long long n, int *grand_total_host) {
     const int nt = 256;
-    long long tiles = (n + nt - 1) / nt;
-    Scratch sc(h->stream);
+    long long tiles = scan_tiles(n);
     int *sums = sc.get<int>(tiles + 1);
     int *tot = sc.get<int>(1);
     if (!sums || !tot) return fail(h, RORBK_ERR_OOM, "scan workspace");
     k_scan_tiles<<<(unsigned)tiles, nt, 0, h->stream>>>(d, d, sums, n);
     k_scan_sums<<<1, 1024, 0, h->stream>>>(sums, (int)tiles, tot);
     k_scan_add<<<(unsigned)tiles, nt, 0, h->stream>>>(d, sums, n);
+    if (!grand_total_host) return cuda_check(h, cudaGetLastError(), "scan");
     rorbk_status st = cuda_check(h, cudaMemcpyAsync(grand_total_host, tot, sizeof(int),
                                                     cudaMemcpyDeviceToHost, h->stream), "scan total");
     if (st) return st;
@@ -776,7 +960,8 @@ static rorbk_status build_sell(rorbk_ctx *h, const std::vector<int> &hrp, bool r
     }
     const int ns = S.nslices;
     k_sell_fill<<<(unsigned)((ns * 32LL + 255) / 256), 256, 0, st>>>(
-        h->rowptr, h->col, h->val, h->val32, ns, S.ptr, S.row, S.rlen, S.col, S.val, S.val32);
+        h->rowptr, h->col, h->val, h->val32, ns, S.ptr, S.row, S.rlen, refresh ? nullptr : S.col, S.val,
+        S.val32);
     return cuda_check(h, cudaStreamSynchronize(st), "SELL copy of A");
 }
 
@@ -812,119 +997,163 @@ rorbk_status build_setup(rorbk_ctx *h, const std::vector<int> &hrp, bool refresh
     cudaStream_t s = h->stream;
     const int m = (int)h->m, n = (int)h->n, k = h->k;
     rorbk_status st;
-    Scratch sc(s);
+    // a refresh of a sparse A: every scratch buffer below in one allocation
+    size_t bytes = 0;
+    if (refresh && h->format == RORBK_FORMAT_CSR && !h->n_wood) {
+        const size_t segs = std::max(1, h->bt.total_segs);
+        for (size_t b : {(size_t)8, (size_t)(n + 1) * 4, (size_t)(n + 1) * 4, (size_t)(scan_tiles(n + 1) + 1) * 4, (size_t)4,
+                         segs * 4, segs * 8, (size_t)k * k * 8, (size_t)k * 8, (size_t)std::max(1LL, h->ops.w_total) * 8})
+            bytes += Scratch::room(b);
+    }
+    Scratch sc(s, bytes);
     int *flags = sc.get<int>(2);
     if (!flags) return fail(h, RORBK_ERR_OOM, "flags");
     cudaMemsetAsync(flags, 0, 2 * sizeof(int), s);
     int gs = std::max(1, std::min(4 * h->num_sms, (m + 255) / 256));
-    k_validate_csr<<<gs, 256, 0, s>>>(h->rowptr, h->col, h->val, m, n, flags);
-    int hf[2] = {0, 0};
-    if ((st = cuda_check(h, cudaMemcpyAsync(hf, flags, sizeof(int), cudaMemcpyDeviceToHost, s), "validate")))
-        return st;
-    if ((st = cuda_check(h, cudaStreamSynchronize(s), "validate"))) return st;
-    if (hf[0] & 1)
-        return fail(h, RORBK_ERR_INVALID_ARG,
-                    "CSR structure: row_ptr must be non-decreasing and columns strictly ascending in [0,n)");
-    if (hf[0] & 2) return fail(h, RORBK_ERR_NUMERIC, "A holds NaN or Inf");
-    if (!keep(h, h->blk_nz, k + 1)) return fail(h, RORBK_ERR_OOM, "block entry offsets");
-    k_block_nz<<<std::max(1, (k + 256) / 256), 256, 0, s>>>(h->rowptr, h->off, k, h->blk_nz);
+    if (!refresh) {          // a refresh keeps the pattern, and its values were checked before they were taken over
+        k_validate_csr<<<gs, 256, 0, s>>>(h->rowptr, h->col, h->val, m, n, flags);
+        int hf[2] = {0, 0};
+        if ((st = cuda_check(h, cudaMemcpyAsync(hf, flags, sizeof(int), cudaMemcpyDeviceToHost, s), "validate")))
+            return st;
+        if ((st = cuda_check(h, cudaStreamSynchronize(s), "validate"))) return st;
+        if (hf[0] & 1)
+            return fail(h, RORBK_ERR_INVALID_ARG,
+                        "CSR structure: row_ptr must be non-decreasing and columns strictly ascending in [0,n)");
+        if (hf[0] & 2) return fail(h, RORBK_ERR_NUMERIC, "A holds NaN or Inf");
+        if (!keep(h, h->blk_nz, k + 1)) return fail(h, RORBK_ERR_OOM, "block entry offsets");
+        k_block_nz<<<std::max(1, (k + 256) / 256), 256, 0, s>>>(h->rowptr, h->off, k, h->blk_nz);
+    }
     if (h->format == RORBK_FORMAT_CSR && (st = build_sell(h, hrp, refresh))) return st;
     if (!refresh && (st = build_block_order(h, hrp))) return st;
     // row norms for the dynamic update: from the FP64 values, and from the
     // FP32 copy that the mixed form's inner solve reads when it differs
     if (!keep(h, h->rn, m)) return fail(h, RORBK_ERR_OOM, "row norms");
-    k_row_norms<double><<<gs, 256, 0, s>>>(h->rowptr, h->val, m, h->rn);
+    const auto &S = h->sell;
+    const bool dense = h->format == RORBK_FORMAT_DENSE;
+    const unsigned gsl = (unsigned)((S.nslices * 32LL + 255) / 256);
+    if (dense) k_row_norms<double><<<gs, 256, 0, s>>>(h->rowptr, h->val, m, h->rn);
+    else if (h->vdtype == RORBK_F64) k_row_norms_sell<double><<<gsl, 256, 0, s>>>(S.nslices, S.ptr, S.row, S.rlen, S.val, h->rn);
+    else k_row_norms_sell<float><<<gsl, 256, 0, s>>>(S.nslices, S.ptr, S.row, S.rlen, S.val32, h->rn);
     if (!refresh) h->rn32 = h->rn;
     if (h->val32 && h->vdtype == RORBK_F64) {
         if (h->rn32 == h->rn) h->rn32 = nullptr;
         if (!keep(h, h->rn32, m)) return fail(h, RORBK_ERR_OOM, "row norms");
-        k_row_norms<float><<<gs, 256, 0, s>>>(h->rowptr, h->val32, m, h->rn32);
+        if (dense) k_row_norms<float><<<gs, 256, 0, s>>>(h->rowptr, h->val32, m, h->rn32);
+        else k_row_norms_sell<float><<<gsl, 256, 0, s>>>(S.nslices, S.ptr, S.row, S.rlen, S.val32, h->rn32);
     }
 
     // block transpose, coupled rows
     const long long nnz = h->nnz;
-    unsigned char *coupled = sc.get<unsigned char>(m);
-    int *ncoupled = sc.get<int>(k + 1);
+    // (coupled rows follow from the pattern: kept for a refresh)
+    if (!keep(h, h->bt.coupled, m) || !keep(h, h->bt.ncoupled, k + 1)) return fail(h, RORBK_ERR_OOM, "block transpose");
+    unsigned char *coupled = h->bt.coupled;
+    int *ncoupled = h->bt.ncoupled;
     if (!keep(h, h->bt.col, nnz + 16) || !keep(h, h->bt.row, nnz + 16) || !keep(h, h->bt.val, nnz + 16) ||
         !keep(h, h->bt.off16, nnz + 16) ||
-        !keep(h, h->bt.seg, nnz) || !keep(h, h->bt.seg_ptr, k) || !coupled || !ncoupled)
+        !keep(h, h->bt.seg, nnz) || !keep(h, h->bt.seg_ptr, k))
         return fail(h, RORBK_ERR_OOM, "block transpose");
     if (h->format == RORBK_FORMAT_DENSE) {
         const int gx = std::max(1, std::min(4 * h->num_sms, (int)((h->nnz / k + 255) / 256)));
         k_block_transpose_dense<<<dim3(gx, k), 256, 0, s>>>(h->val, h->off, n, h->bt.col, h->bt.row, h->bt.val,
                                                             h->bt.off16, h->bt.seg, h->bt.seg_ptr, coupled,
                                                             ncoupled);
+    } else if (refresh && h->bt.max_entries <= 65536) {
+        k_block_refill<<<k, 256, 0, s>>>(h->blk_nz, h->val, h->bt.off16, h->bt.val);
     } else {
-        k_block_transpose<<<k, 256, 0, s>>>(h->rowptr, h->col, h->val, h->off, h->bt.col, h->bt.row,
-                                            h->bt.val, h->bt.off16, h->bt.seg, h->bt.seg_ptr, coupled, ncoupled);
+        if (!refresh)
+            for (int t = 0; t < k; ++t)
+                h->bt.max_entries = std::max(h->bt.max_entries, hrp[h->h_off[t + 1]] - hrp[h->h_off[t]]);
+        const int sort = std::min(kBtSort, next_pow2(std::max(1, h->bt.max_entries)));
+        cudaFuncSetAttribute(k_block_transpose, cudaFuncAttributeMaxDynamicSharedMemorySize, kBtSort * 8);
+        k_block_transpose<<<k, 256, (size_t)sort * 8, s>>>(h->rowptr, h->col, h->val, h->off, h->bt.col, h->bt.row,
+                                                           h->bt.val, h->bt.off16, h->bt.seg, h->bt.seg_ptr, coupled,
+                                                           ncoupled, sort);
     }
     if ((st = cuda_check(h, cudaGetLastError(), "block transpose"))) return st;
 
     // centroids, C row sums, proposal
     {
-        Scratch cs(s);
+        Scratch own(s);                              // of this part, unless the arena holds it
+        Scratch &cs = bytes ? sc : own;
         int *colcnt = cs.get<int>(n + 1);
         int *fill = cs.get<int>(n + 1);
         if (!colcnt || !fill) return fail(h, RORBK_ERR_OOM, "centroid columns");
         cudaMemsetAsync(colcnt, 0, (size_t)(n + 1) * sizeof(int), s);
         cudaMemsetAsync(fill, 0, (size_t)(n + 1) * sizeof(int), s);
         int gk = std::min(k, 8 * h->num_sms);
-        k_centroid_count<<<gk, 128, 0, s>>>(h->rowptr, h->off, h->bt.col, h->bt.seg, h->bt.seg_ptr,
+        k_centroid_count<<<gk, 512, 0, s>>>(h->rowptr, h->off, h->bt.col, h->bt.seg, h->bt.seg_ptr,
                                            k, colcnt);
-        int total = 0;
-        if ((st = scan_device(h, colcnt, (long long)n + 1, &total))) return st;
+        int total = h->bt.total_segs;                // (the pattern's)
+        if ((st = scan_device(h, cs, colcnt, (long long)n + 1, refresh ? nullptr : &total))) return st;
+        h->bt.total_segs = total;
         int *cb = cs.get<int>(std::max(1, total));
         double *cv = cs.get<double>(std::max(1, total));
         double *G = cs.get<double>((size_t)k * k);
         if (!cb || !cv || !G) return fail(h, RORBK_ERR_OOM, "centroid Gram");
-        k_centroid_fill<<<gk, 128, 0, s>>>(h->rowptr, h->off, h->bt.col, h->bt.val, h->bt.seg,
+        k_centroid_fill<<<gk, 512, 0, s>>>(h->rowptr, h->off, h->bt.col, h->bt.val, h->bt.seg,
                                           h->bt.seg_ptr, k, colcnt, fill, cb, cv);
-        cudaMemsetAsync(G, 0, (size_t)k * k * sizeof(double), s);
-        k_centroid_gram<<<(k * 32 + 255) / 256, 256, 0, s>>>(h->rowptr, h->off, h->bt.col, h->bt.val,
-                                                            h->bt.seg, h->bt.seg_ptr, k, colcnt,
-                                                            cb, cv, G);
-        k_crowsum<<<(k * 32 + 255) / 256, 256, 0, s>>>(G, k, h->crowsum);
+        // the row of G of one block in shared memory: up to 24,576 blocks
+        constexpr int kGramRow = 24576;
+        if (k <= kGramRow) {
+            cudaFuncSetAttribute(k_centroid_gram<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGramRow * 8);
+            k_centroid_gram<true><<<k, 32, (size_t)k * 8, s>>>(h->rowptr, h->off, h->bt.col, h->bt.val, h->bt.seg,
+                                                               h->bt.seg_ptr, k, colcnt, cb, cv, G);
+        } else {
+            k_centroid_gram<false><<<k, 32, 0, s>>>(h->rowptr, h->off, h->bt.col, h->bt.val, h->bt.seg,
+                                                    h->bt.seg_ptr, k, colcnt, cb, cv, G);
+        }
+        double *nrm = cv;                            // the centroids are no longer needed
+        if (total < k && !(nrm = cs.get<double>(k))) return fail(h, RORBK_ERR_OOM, "centroid norms");
+        k_centroid_norms<<<std::max(1, std::min(h->num_sms, (k + 255) / 256)), 256, 0, s>>>(G, k, nrm);
+        k_crowsum<<<(k * 32 + 255) / 256, 256, 0, s>>>(G, nrm, k, h->crowsum);
         k_proposal<<<1, 1024, 0, s>>>(h->crowsum, k, (double)n, h->cdf, h->pbar);
         if ((st = cuda_check(h, cudaGetLastError(), "proposal"))) return st;
     }
 
     // static operators on the coupled rows of every block
     {
-        std::vector<int> hcnt(k + 1, 0);
-        if ((st = cuda_check(h, cudaMemcpyAsync(hcnt.data(), ncoupled, k * sizeof(int),
-                                                cudaMemcpyDeviceToHost, s), "coupled counts")))
-            return st;
-        if ((st = cuda_check(h, cudaStreamSynchronize(s), "coupled counts"))) return st;
-        // blocks with at least n rows take the n x n form (Lemma 1, Section 3.1)
-        std::vector<long long> woodp(k, -1);
-        long long wtot = 0;
-        h->n_wood = 0;
-        for (int t = 0; t < k; ++t)
-            if (h->h_off[t + 1] - h->h_off[t] >= n) {
-                woodp[t] = wtot;
-                wtot += (long long)n * n;
-                hcnt[t] = 0;
-                ++h->n_wood;
+        // offsets and sizes follow from the pattern: formed once
+        if (!refresh) {
+            std::vector<int> hcnt(k + 1, 0);
+            if ((st = cuda_check(h, cudaMemcpyAsync(hcnt.data(), ncoupled, k * sizeof(int),
+                                                    cudaMemcpyDeviceToHost, s), "coupled counts")))
+                return st;
+            if ((st = cuda_check(h, cudaStreamSynchronize(s), "coupled counts"))) return st;
+            // blocks with at least n rows take the n x n form (Lemma 1, Section 3.1)
+            std::vector<long long> woodp(k, -1);
+            h->ops.wood_total = 0;
+            h->n_wood = 0;
+            for (int t = 0; t < k; ++t)
+                if (h->h_off[t + 1] - h->h_off[t] >= n) {
+                    woodp[t] = h->ops.wood_total;
+                    h->ops.wood_total += (long long)n * n;
+                    hcnt[t] = 0;
+                    ++h->n_wood;
+                }
+            if (h->n_wood) {
+                if (!keep(h, h->wood_ptr, k) || !keep(h, h->wood_ss, h->ops.wood_total))
+                    return fail(h, RORBK_ERR_OOM, "s >= n operators");
+                cudaMemcpyAsync(h->wood_ptr, woodp.data(), (size_t)k * sizeof(long long), cudaMemcpyHostToDevice, s);
             }
-        if (h->n_wood) {
-            if (!keep(h, h->wood_ptr, k) || !keep(h, h->wood_ss, wtot))
-                return fail(h, RORBK_ERR_OOM, "s >= n operators");
-            cudaMemcpyAsync(h->wood_ptr, woodp.data(), (size_t)k * sizeof(long long), cudaMemcpyHostToDevice, s);
+            std::vector<int> sptr(k + 1, 0);
+            std::vector<long long> wptr(k + 1, 0);
+            h->ops.max_coupled = 0;
+            for (int t = 0; t < k; ++t) {
+                sptr[t + 1] = sptr[t] + hcnt[t];
+                wptr[t + 1] = wptr[t] + (long long)hcnt[t] * hcnt[t];
+                h->ops.max_coupled = std::max(h->ops.max_coupled, hcnt[t]);
+            }
+            h->ops.w_total = wptr[k];
+            if (!keep(h, h->ops.s_ptr, k + 1) || !keep(h, h->ops.w_ptr, k + 1) ||
+                !keep(h, h->ops.s_idx, std::max(1, sptr[k])) || !keep(h, h->ops.s_pos, m) ||
+                !keep(h, h->ops.w_ss, std::max(1LL, wptr[k])) || !keep(h, h->ops.w_diag, m))
+                return fail(h, RORBK_ERR_OOM, "static operators");
+            cudaMemcpyAsync(h->ops.s_ptr, sptr.data(), (k + 1) * sizeof(int), cudaMemcpyHostToDevice, s);
+            cudaMemcpyAsync(h->ops.w_ptr, wptr.data(), (k + 1) * sizeof(long long), cudaMemcpyHostToDevice, s);
         }
-        std::vector<int> sptr(k + 1, 0);
-        std::vector<long long> wptr(k + 1, 0);
-        for (int t = 0; t < k; ++t) {
-            sptr[t + 1] = sptr[t] + hcnt[t];
-            wptr[t + 1] = wptr[t] + (long long)hcnt[t] * hcnt[t];
-        }
-        if (!keep(h, h->ops.s_ptr, k + 1) || !keep(h, h->ops.w_ptr, k + 1) ||
-            !keep(h, h->ops.s_idx, std::max(1, sptr[k])) || !keep(h, h->ops.s_pos, m) ||
-            !keep(h, h->ops.w_ss, std::max(1LL, wptr[k])) || !keep(h, h->ops.w_diag, m))
-            return fail(h, RORBK_ERR_OOM, "static operators");
-        double *linv = sc.get<double>(std::max(1LL, wptr[k]));
+        const long long wtot = h->ops.wood_total, wss = std::max(1LL, h->ops.w_total);
+        double *linv = sc.get<double>(wss);
         if (!linv) return fail(h, RORBK_ERR_OOM, "static operator scratch");
-        cudaMemcpyAsync(h->ops.s_ptr, sptr.data(), (k + 1) * sizeof(int), cudaMemcpyHostToDevice, s);
-        cudaMemcpyAsync(h->ops.w_ptr, wptr.data(), (k + 1) * sizeof(long long), cudaMemcpyHostToDevice, s);
         cudaMemsetAsync(flags, 0, sizeof(int), s);
         // a dense A: every block's Gram by the grid (the blocks' rows are long)
         const bool dense_gram = h->format == RORBK_FORMAT_DENSE && !h->n_wood;
@@ -933,10 +1162,14 @@ rorbk_status build_setup(rorbk_ctx *h, const std::vector<int> &hrp, bool refresh
             k_dense_static_gram<<<dim3(nt * (nt + 1) / 2, k), kSgT * kSgT, 0, s>>>(h->val, h->off, n, h->mu,
                                                                                  h->ops.w_ptr, h->ops.w_ss);
         }
-        k_static_ops<<<k, 256, 0, s>>>(h->rowptr, h->col, h->val, h->off, h->mu, coupled,
-                                       h->ops.s_ptr, h->ops.w_ptr, h->ops.s_idx, h->ops.s_pos,
-                                       h->ops.w_ss, h->ops.w_diag, linv, h->wood_ptr, flags,
-                                       dense_gram ? 1 : 0);
+        const int stage = dense_gram ? 0 : std::min(kSoStage, (h->bt.max_entries + 1) & ~1);
+        // two matrices of the largest coupled set, up to 64 rows (three blocks per SM)
+        const int mat = dense_gram ? 0 : 2 * std::min(h->ops.max_coupled, 64) * std::min(h->ops.max_coupled, 64);
+        cudaFuncSetAttribute(k_static_ops, cudaFuncAttributeMaxDynamicSharedMemorySize, kSoStage * 12);
+        k_static_ops<<<k, 256, std::max((size_t)stage * 12, (size_t)mat * 8), s>>>(h->rowptr, h->col, h->val, h->off, h->mu, coupled,
+                                                        h->ops.s_ptr, h->ops.w_ptr, h->ops.s_idx, h->ops.s_pos,
+                                                        h->ops.w_ss, h->ops.w_diag, linv, h->wood_ptr, flags,
+                                                        dense_gram ? 1 : 0, h->rn, stage, mat);
         if (h->n_wood) {
             double *linv2 = sc.get<double>(wtot);
             if (!linv2) return fail(h, RORBK_ERR_OOM, "s >= n operator scratch");
@@ -949,10 +1182,10 @@ rorbk_status build_setup(rorbk_ctx *h, const std::vector<int> &hrp, bool refresh
         if (st) return st;
         if (spd) return fail(h, RORBK_ERR_NOT_SPD, "a static block Gram is not positive definite (lambda = 0 with dependent rows?)");
         if (h->precision_built) {
-            if (!keep(h, h->ops.w_ss32, std::max(1LL, wptr[k])) || !keep(h, h->ops.w_diag32, m) ||
+            if (!keep(h, h->ops.w_ss32, wss) || !keep(h, h->ops.w_diag32, m) ||
                 !keep(h, h->bt.val32, nnz + 16))
                 return fail(h, RORBK_ERR_OOM, "fp32 operators");
-            k_narrow<<<gs, 256, 0, s>>>(h->ops.w_ss, h->ops.w_ss32, std::max(1LL, wptr[k]));
+            k_narrow<<<gs, 256, 0, s>>>(h->ops.w_ss, h->ops.w_ss32, wss);
             k_narrow<<<gs, 256, 0, s>>>(h->ops.w_diag, h->ops.w_diag32, m);
             k_narrow<<<gs, 256, 0, s>>>(h->bt.val, h->bt.val32, nnz);
             if (h->n_wood) {
@@ -981,7 +1214,7 @@ rorbk_status build_csc(rorbk_ctx *h, const double *scale, int *cp, int *crow, do
     cudaMemsetAsync(maxlen, 0, sizeof(int), s);
     k_col_count<<<ge, 256, 0, s>>>(h->col, nnz, cp);
     int total = 0;
-    if ((st = scan_device(h, cp, (long long)n + 1, &total))) return st;
+    if ((st = scan_device(h, sc, cp, (long long)n + 1, &total))) return st;
     if (total != nnz) return fail(h, RORBK_ERR_CUDA, "column-major copy of A: entry count");
     k_col_max<<<std::max(1, std::min(8 * h->num_sms, (n + 255) / 256)), 256, 0, s>>>(cp, n, maxlen);
     k_col_place<<<gr, 256, 0, s>>>(h->rowptr, h->col, m, cp, fill, slot, rowid);

@@ -583,11 +583,13 @@ rorbk_status rorbk_update_values(rorbk_handle h, const void *values, int32_t dty
             cudaMemcpyAsync(dtype == RORBK_F64 ? (void *)h->val : (void *)h->val32, tmp, nnz * esz,
                             cudaMemcpyDeviceToDevice, s);
             widen_values(h, dtype);
-            st = cuda_check(h, cudaStreamSynchronize(s), "rorbk_update_values");
         }
-        cudaFree(tmp);
     }
     if (!st) st = build_setup(h, std::vector<int>(), true);
+    if (tmp) {
+        cudaStreamSynchronize(s);
+        cudaFree(tmp);
+    }
     if (!st && h->values_version) ++*h->values_version;
     // this handle's own column-major copy now; those of handles sharing the
     // set-up at their next incremental solve
