@@ -19,20 +19,22 @@
 //     FP64 operations, no call to sqrt or to a division), while six warps apply
 //     the previous column to the columns after the next, from registers;
 //   - the trailing update of a panel runs over all warps of the cluster (a lane
-//     per column, four rows per warp) from a copy of the panel in shared memory;
+//     per column, a few rows per warp) from a copy of the panel in shared memory;
+//     only its part in the next panel's columns is awaited, the rest runs beside
+//     those columns in the block's second half;
 //   - the right-hand side is carried as one more row of the matrix, so the
 //     forward solve costs nothing extra; the backward solve runs in the
 //     cluster's first block, one warp on the 32-row diagonal chain while the
 //     others apply the finished rows of the solution further up.
 // Two cluster barriers per panel order the traffic through L2.
 //
-// Measured (16 blocks, one launch): order 256 344 us (mixed form's factor
-// 260 us), order 100 127 us, order 40 53 us, order 500 982 us.  At order 256 about
-// 356 kcycles are the 256 columns, 134 the trailing updates (FP64 rate of 16
-// SMs), 100 the backward solve, 78 loads, stores and barriers.  Before: 15
-// grid-wide launches and a one-block backward solve, 1,003 us at order 256 (dense
-// A); the sparse dynamic block, factored by one block of threads, 2,230 us at
-// about 230 coupled rows.
+// Measured (16 blocks, one launch): order 256 321 us (mixed form's factor
+// 237 us), order 100 121 us, order 40 51 us, order 500 866 us; with the whole
+// trailing update awaited 348, 128, 54 and 995 us.  At order 256 about 356 kcycles of
+// 622 are the 256 columns and 100 the backward solve.  Before: 15 grid-wide launches
+// and a one-block backward solve, 1,003 us at order 256 (dense A); the sparse
+// dynamic block, factored by one block of threads, 2,230 us at about 230 coupled
+// rows.
 //
 // Order of operations.  Every entry receives g = fma(-L_aj, L_bj, g) over
 // ascending j, then the correctly rounded quotient by
@@ -49,7 +51,7 @@ namespace rorbk {
 
 constexpr int kCw = 32;                 // panel width
 constexpr int kCwp = kCw + 1;           // row stride of panels in shared memory
-constexpr int kCcThreads = 256;
+constexpr int kCcThreads = 512;          // one system at a time (256 for a block of columns)
 constexpr int kCcMaxCluster = 16;       // blocks per cluster
 constexpr int kCcMaxRows = 32;          // rows below the diagonal block per block: one per lane
 
@@ -156,6 +158,8 @@ __host__ __device__ constexpr int cc_rows(int K, int C) { return K + 1 <= kCw ? 
 __host__ __device__ constexpr int cc_max_order(int C) {
     return C * kCcMaxRows + kCw - 1;
 }
+template <int N>
+struct IntC { static constexpr int value = N; };
 constexpr int kCcStage = 2 * kCw * kCwp;          // backward solve: one stage (two 32 x 32 tiles)
 // Dynamic shared memory for orders up to K: diagonal block, own rows, the
 // panel (or the three stages of the backward solve), z, reciprocals.
@@ -177,10 +181,17 @@ __host__ __device__ constexpr size_t cc_smem_bytes(int K, int C) {
 // so one barrier per column is enough.  Their entries are listed by descending
 // column: those still to be updated are always the first ones, and a step issues
 // as few FP64 instructions as the entries fill.
-constexpr int kCcBulk = kCcThreads - 64;
+constexpr int kCcBulk = 256 - 64;
 constexpr int kCcTri = kCw * (kCw - 1) / 2;          // entries of columns 1 .. kCw - 1 of the diagonal block
 constexpr int kCcGd = (kCcTri + kCcBulk - 1) / kCcBulk;
 constexpr int kCcGr = ((kCw - 1) * kCcMaxRows + kCcBulk - 1) / kCcBulk;
+
+// (The panel's 256 threads meet at named barrier 1: in a block of 512 the other
+// half works on the previous panel's trailing update meanwhile.)
+__device__ __forceinline__ void panel_sync() {
+    __syncwarp();
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+}
 
 template <bool RC>
 __device__ __forceinline__ void cc_panel(double *Ld, double *R, int w, int nr, double *rlp, int *bad) {
@@ -253,10 +264,10 @@ __device__ __forceinline__ void cc_panel(double *Ld, double *R, int w, int nr, d
                 if (c == j + 1) R[u * kCwp + c] = gr[k];
             }
         }
-        __syncthreads();
+        panel_sync();
     }
     if (threadIdx.x < w) Ld[threadIdx.x * kCwp + threadIdx.x] = rlp[kCw + threadIdx.x];
-    __syncthreads();
+    panel_sync();
 }
 
 // The matrix, packed lower row-major in g (order K), and its right-hand side:
@@ -264,9 +275,16 @@ __device__ __forceinline__ void cc_panel(double *Ld, double *R, int w, int nr, d
 // return out(i, x_i) has been called for every i of the solution (by the
 // cluster's first block), and *bad is set there if a pivot was not positive.
 // Every thread of the cluster calls it with the same K.
-template <bool RC, typename First, typename Out>
+//
+// OV (blocks of 512 threads): of a panel's trailing update only the next panel's
+// 32 columns are awaited; the rest is left to the second half of the block, beside
+// the next panel's columns, whose chain leaves half of the FP64 unit free.
+// A block of columns keeps blocks of 256, two per SM: its clusters fill the
+// device, and two chains on an SM overlap each other.
+template <bool RC, bool OV, typename First, typename Out>
 __device__ __forceinline__ void cluster_chol_solve(double *g, double *zbuf, int K, double *sm, int *bad,
                                                    First first, Out out) {
+    constexpr int NT = OV ? 512 : 256, NW = NT / 32;
     __shared__ double rlp[2 * kCw];               // the panel's 1 / L_jj, and its diagonal
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int rank = (int)cluster_rank(), C = (int)cluster_blocks();
@@ -275,21 +293,63 @@ __device__ __forceinline__ void cluster_chol_solve(double *g, double *zbuf, int 
     const size_t panel = (size_t)(K + 1) * kCwp > 3u * kCcStage ? (size_t)(K + 1) * kCwp : 3u * kCcStage;
     double *z = P + panel, *rlv = z + K + kCw;    // first block: solution, reciprocals of the pivots
     auto at = [](int i, int j) { return (long long)i * (i + 1) / 2 + j; };
+    // The trailing update by the panel before column j1 (P: its rows j1 .. K, row K
+    // the right-hand side) of the columns from j1 + bfrom up to j1 + bto, in units of
+    // RU rows x 32 columns dealt over the warps of the cluster.
+    auto trail = [&](auto ru, int j1, int bfrom, int bto, int wid, int nw) {
+        constexpr int RU = decltype(ru)::value;
+        const int nb = K + 1 - j1;
+        int unit = wid * C + rank;
+        for (int b0 = bfrom; b0 < min(bto, K - j1); b0 += kCw) {
+            const int groups = (nb - b0 + RU - 1) / RU;
+            for (; unit < groups; unit += C * nw) {
+                const int a0 = b0 + RU * unit, b = b0 + lane;     // rows and column, from j1
+                const bool bin = b < K - j1;
+                double acc[RU];
+#pragma unroll
+                for (int q = 0; q < RU; ++q) {
+                    const int a = a0 + q;
+                    acc[q] = 0.0;
+                    if (bin && a < nb - 1 && b <= a) acc[q] = __ldcg(&g[at(j1 + a, j1 + b)]);
+                    if (bin && a == nb - 1) acc[q] = j1 == kCw ? first(j1 + b) : __ldcg(&zbuf[j1 + b]);
+                }
+                const double *pb = P + (size_t)min(b, nb - 1) * kCwp;
+                const double *pa[RU];
+#pragma unroll
+                for (int q = 0; q < RU; ++q) pa[q] = P + (size_t)min(a0 + q, nb - 1) * kCwp;
+#pragma unroll 8
+                for (int j = 0; j < kCw; ++j) {
+                    const double lb = pb[j];
+#pragma unroll
+                    for (int q = 0; q < RU; ++q) acc[q] = sub_prod(acc[q], pa[q][j], lb);
+                }
+#pragma unroll
+                for (int q = 0; q < RU; ++q) {
+                    const int a = a0 + q;
+                    if (bin && a < nb - 1 && b <= a) g[at(j1 + a, j1 + b)] = acc[q];
+                    if (bin && a == nb - 1) zbuf[j1 + b] = acc[q];
+                }
+            }
+            unit -= groups;
+        }
+    };
     for (int j0 = 0; j0 < K; j0 += kCw) {
         const int w = min(kCw, K - j0), j1 = j0 + w;
         const int nr = max(0, (K + 1 - j1 - rank + C - 1) / C);     // rows j1 + rank + C u
-        for (int e = tid; e < w * kCw; e += kCcThreads) {
+        for (int e = tid; e < w * kCw; e += NT) {
             const int i = e >> 5, j = e & 31;
             if (j <= i) Ld[i * kCwp + j] = __ldcg(&g[at(j0 + i, j0 + j)]);
         }
-        for (int e = tid; e < nr * kCw; e += kCcThreads) {
+        for (int e = tid; e < nr * kCw; e += NT) {
             const int u = e >> 5, j = e & 31, i = j1 + rank + C * u;
             if (j < w)
                 R[u * kCwp + j] = i < K ? __ldcg(&g[at(i, j0 + j)]) : j0 == 0 ? first(j) : __ldcg(&zbuf[j0 + j]);
         }
         __syncthreads();
-        cc_panel<RC>(Ld, R, w, nr, rlp, bad);
-        for (int e = tid; e < nr * kCw; e += kCcThreads) {
+        if (tid < 256) cc_panel<RC>(Ld, R, w, nr, rlp, bad);
+        else if (OV && j0 > 0) trail(IntC<4>(), j0, kCw, K, warp - 8, 8);
+        if constexpr (OV) __syncthreads();
+        for (int e = tid; e < nr * kCw; e += NT) {
             const int u = e >> 5, j = e & 31, i = j1 + rank + C * u;
             if (j < w) {
                 if (i < K) g[at(i, j0 + j)] = R[u * kCwp + j];
@@ -300,58 +360,26 @@ __device__ __forceinline__ void cluster_chol_solve(double *g, double *zbuf, int 
         cluster_sync_all();
         // every block has its copy of the diagonal block: it can be replaced
         if (rank == 0)
-            for (int e = tid; e < w * kCw; e += kCcThreads) {
+            for (int e = tid; e < w * kCw; e += NT) {
                 const int i = e >> 5, j = e & 31;
                 if (j <= i) g[at(j0 + i, j0 + j)] = Ld[i * kCwp + j];
             }
         if (j1 >= K) break;
-        // trailing update: rows j1 .. K (row K: the right-hand side) of columns j1 ..
         const int nb = K + 1 - j1;
-        for (int u0 = warp; u0 < nb; u0 += 64) {      // a warp per row, eight rows in flight
+        for (int u0 = warp; u0 < nb; u0 += 8 * NW) {      // a warp per row, eight rows in flight
             double t[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                const int i = j1 + u0 + 8 * q;
+                const int i = j1 + u0 + NW * q;
                 t[q] = i < K ? __ldcg(&g[at(i, j0 + lane)]) : i == K ? __ldcg(&zbuf[j0 + lane]) : 0.0;
             }
 #pragma unroll
             for (int q = 0; q < 8; ++q)
-                if (u0 + 8 * q < nb) P[(u0 + 8 * q) * kCwp + lane] = t[q];
+                if (u0 + NW * q < nb) P[(u0 + NW * q) * kCwp + lane] = t[q];
         }
         __syncthreads();
-        int unit = warp * C + rank;               // units of 4 rows x 32 columns, dealt over the cluster
-        for (int b0 = 0; b0 < K - j1; b0 += kCw) {
-            const int groups = (nb - b0 + 3) >> 2;
-            for (; unit < groups; unit += C * (kCcThreads / 32)) {
-                const int a0 = b0 + 4 * unit, b = b0 + lane;      // rows and column, from j1
-                const bool bin = b < K - j1;
-                double acc[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int a = a0 + q;
-                    acc[q] = 0.0;
-                    if (bin && a < nb - 1 && b <= a) acc[q] = __ldcg(&g[at(j1 + a, j1 + b)]);
-                    if (bin && a == nb - 1) acc[q] = j0 == 0 ? first(j1 + b) : __ldcg(&zbuf[j1 + b]);
-                }
-                const double *pb = P + (size_t)min(b, nb - 1) * kCwp;
-                const double *pa[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) pa[q] = P + (size_t)min(a0 + q, nb - 1) * kCwp;
-#pragma unroll 8
-                for (int j = 0; j < kCw; ++j) {
-                    const double lb = pb[j];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) acc[q] = sub_prod(acc[q], pa[q][j], lb);
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int a = a0 + q;
-                    if (bin && a < nb - 1 && b <= a) g[at(j1 + a, j1 + b)] = acc[q];
-                    if (bin && a == nb - 1) zbuf[j1 + b] = acc[q];
-                }
-            }
-            unit -= groups;
-        }
+        if constexpr (OV) trail(IntC<2>(), j1, 0, kCw, warp, NW);
+        else trail(IntC<4>(), j1, 0, K, warp, NW);
         cluster_sync_all();
     }
     if (rank != 0) return;
@@ -371,9 +399,9 @@ __device__ __forceinline__ void cluster_chol_solve(double *g, double *zbuf, int 
             if (q > 0) U[j * kCwp + i] = __ldcg(&g[at(j0 + j, j0 - kCw + i)]);
         }
     };
-    for (int i = tid; i < K; i += kCcThreads) z[i] = __ldcg(&zbuf[i]);
-    stage(nblk - 1, tid, kCcThreads);
-    stage(nblk - 2, tid, kCcThreads);
+    for (int i = tid; i < K; i += NT) z[i] = __ldcg(&zbuf[i]);
+    stage(nblk - 1, tid, NT);
+    stage(nblk - 2, tid, NT);
     __syncthreads();
     for (int q = nblk - 1; q >= 0; --q) {
         const int j0 = q * kCw, w = min(kCw, K - j0);
@@ -408,8 +436,8 @@ __device__ __forceinline__ void cluster_chol_solve(double *g, double *zbuf, int 
             z[j0 - kCw + lane] = zi;
             __syncwarp();
         } else {
-            stage(q - 2, tid - 32, kCcThreads - 32);
-            for (int i = tid - 32; i < j0 - kCw; i += kCcThreads - 32) {
+            stage(q - 2, tid - 32, NT - 32);
+            for (int i = tid - 32; i < j0 - kCw; i += NT - 32) {
                 double zi = z[i];
 #pragma unroll 8
                 for (int j = w - 1; j >= 0; --j) {
@@ -420,7 +448,7 @@ __device__ __forceinline__ void cluster_chol_solve(double *g, double *zbuf, int 
             }
         }
     }
-    for (int i = tid; i < K; i += kCcThreads) out(i, z[i]);
+    for (int i = tid; i < K; i += NT) out(i, z[i]);
 }
 
 }  // namespace rorbk

@@ -172,7 +172,8 @@ struct Cols {
     const int *iperm;     // row -> SELL position
     unsigned *grp;        // [0] column ticket of the group, [1] 1 while any column runs
 };
-static inline Cols one_col(int m) { return Cols{1, 0, m, nullptr, nullptr, nullptr}; }
+__host__ __device__ inline Cols one_column(int m) { return Cols{1, 0, m, nullptr, nullptr, nullptr}; }
+static inline Cols one_col(int m) { return one_column(m); }
 // MC (several columns) is a template flag of every kernel that takes Cols, so
 // the one-column instances compile without the column arithmetic.
 template <bool MC>
@@ -1434,6 +1435,70 @@ __global__ void __launch_bounds__(512) k_topk_collect(const T *__restrict__ r, i
     if (threadIdx.x == 0) ctl->ticket = 0;
 }
 
+// Levels 2 and 3 and the exact set in one block, for residuals that it holds in
+// registers (m <= kTopkSmall: 16 values per thread): one launch instead of two
+// grids whose last blocks do most of the work (2,025 rows: 7.8 + 9.4 -> 12 us).
+// The first level (ctl->sel1, above1) comes from the residual pass; the sets are
+// those of k_topk_hist2 and k_topk_collect.
+constexpr int kTopkSmallU = 16;
+constexpr int kTopkSmall = 1024 * kTopkSmallU;
+
+template <typename T>
+__global__ void __launch_bounds__(1024, 1) k_topk_small(const T *__restrict__ r, int m, int K,
+                                                        const int *rowptr, int *in_list, int *eq_list, Dyn D,
+                                                        Ctl *ctl) {
+    extern __shared__ unsigned long long dsm_u64[];
+    __shared__ unsigned hist[kHistBins];
+    __shared__ int s_in, s_eq;
+    if (ctl->done || ctl->halt) return;
+    T v[kTopkSmallU];
+#pragma unroll
+    for (int u = 0; u < kTopkSmallU; ++u) {
+        const int i = u * 1024 + threadIdx.x;
+        v[u] = i < m ? r[i] : T(0);
+    }
+    const unsigned sel1 = (unsigned)ctl->sel1;
+    const int above1 = ctl->above1;
+    for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) hist[i] = 0u;
+    if (threadIdx.x == 0) s_in = s_eq = 0;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kTopkSmallU; ++u) {
+        const unsigned long long key = topk_key(v[u]);
+        if (u * 1024 + (int)threadIdx.x < m && (unsigned)(key >> 52) == sel1)
+            atomicAdd(&hist[(unsigned)(key >> 41) & 2047u], 1u);
+    }
+    __syncthreads();
+    int bin, above;
+    select_bin(hist, K - above1, &bin, &above);
+    const unsigned long long P = (unsigned long long)sel1 << 11 | (unsigned)bin;
+#pragma unroll
+    for (int u = 0; u < kTopkSmallU; ++u) {
+        const int i = u * 1024 + threadIdx.x;
+        if (i >= m) continue;
+        const unsigned long long pre = topk_key(v[u]) >> 41;
+        if (pre > P) {
+            in_list[atomicAdd(&s_in, 1)] = i;
+        } else if (pre == P) {
+            const int pos = atomicAdd(&s_eq, 1);
+            if (pos < kEqCap) eq_list[pos] = i;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        ctl->prefix = (int)P;
+        ctl->above = above1 + above;
+        ctl->n_in = s_in;
+        ctl->n_eq = s_eq;
+    }
+    __syncthreads();
+    unsigned long long *skey = dsm_u64;
+    int *sidx = (int *)(skey + kEqCap);
+    int *sI = sidx + kEqCap;
+    finalize_topk<T, false>(r, m, K, in_list, eq_list, ctl, sI, skey, sidx, one_column(m));
+    publish_rows(rowptr, sI, K, D, ctl, 1);
+}
+
 // Single-step API: a given ascending I, checked before any row is read (an
 // entry outside [0, m) or a set that is not strictly ascending records
 // kDevBounds, and the kernels after this one do nothing).
@@ -1951,13 +2016,13 @@ __global__ void __launch_bounds__(512, 1) k_dyn_mark(Mat<T> A, const T *__restri
 // Factor and solves of the Gram of a dense A's rows of I (order K, right-hand
 // side r_I), or of the n x n form (order n, right-hand side z0), by one cluster.
 template <typename T>
-__global__ void __launch_bounds__(kCcThreads, 2) k_dense_chol(const T *__restrict__ r, int K, Dyn D, Ctl *ctl,
+__global__ void __launch_bounds__(kCcThreads, 1) k_dense_chol(const T *__restrict__ r, int K, Dyn D, Ctl *ctl,
                                                               const double *__restrict__ z0) {
     extern __shared__ unsigned long long dsm_u64[];
     __shared__ int s_bad;
     if (ctl->done || ctl->status || ctl->halt) return;
     if (threadIdx.x == 0) s_bad = 0;
-    cluster_chol_solve<false>(
+    cluster_chol_solve<false, true>(
         D.g, D.z, K, (double *)dsm_u64, &s_bad, [&](int c) { return z0 ? z0[c] : (double)r[D.I[c]]; },
         [&](int i, double v) { D.y[i] = v; });
     if (threadIdx.x == 0 && cluster_rank() == 0 && s_bad) set_status(&ctl->status, kDevNotSpd);
@@ -1995,7 +2060,7 @@ __device__ void end_iteration(const T *x, int n, Ctl *ctl, int use_cond,
 // iteration that needs none (2 us of 140 in the steady state of the 2^20
 // power-law system); a scatter by 16 blocks instead of all costs nothing visible.
 template <typename T, bool LOG = false, bool MC = false>
-__global__ void __launch_bounds__(kCcThreads, 2) k_dyn_scatter(T *x, int n, Dyn D, Ctl *ctl, int count_iter,
+__global__ void __launch_bounds__(MC ? 256 : kCcThreads, MC ? 2 : 1) k_dyn_scatter(T *x, int n, Dyn D, Ctl *ctl, int count_iter,
                                                                int use_cond,
                                                                cudaGraphConditionalHandle hcond, Cols cl) {
     extern __shared__ unsigned long long dsm_u64[];
@@ -2018,7 +2083,7 @@ __global__ void __launch_bounds__(kCcThreads, 2) k_dyn_scatter(T *x, int n, Dyn 
         if (bid >= C) return;
         nblk = C;
         if (threadIdx.x == 0) s_bad = 0;
-        cluster_chol_solve<sizeof(T) == sizeof(float)>(
+        cluster_chol_solve<sizeof(T) == sizeof(float), !MC>(
             D.gc, D.z, nF, (double *)dsm_u64, &s_bad, [&](int c) { return __ldcg(&D.z[c]); },
             [&](int i, double v) { D.y[D.fidx[i]] = v; });
         if (threadIdx.x == 0 && bid == 0 && s_bad) set_status(&ctl->status, kDevNotSpd);
@@ -3362,11 +3427,18 @@ int grid_topk(rorbk_ctx *h) {
     return tuned(h->tune.topk, std::min<long long>(4 * h->num_sms / nr, (mp + 255) / 256));
 }
 int grid_collect(rorbk_ctx *h) { return tuned(h->tune.collect, grid_topk(h) / 2); }
-int grid_mark(rorbk_ctx *h) { return tuned(h->tune.mark, h->num_sms / std::max(1, h->nr)); }
+// (at most as many blocks as A_I's entries can fill; two at least: one plans the
+// next draws while the other factors)
+int grid_mark(rorbk_ctx *h) {
+    const long long need = std::max<long long>(2, (h->dyn.ecap + 255) / 256);
+    return tuned(h->tune.mark, (int)std::min<long long>(h->num_sms / std::max(1, h->nr), need));
+}
 // (about one block per SM, in whole clusters)
 int grid_scatter(rorbk_ctx *h) {
     const int C = std::max(1, h->dyn.cluster);
-    return tuned(h->tune.scatter, std::max(1, h->num_sms / std::max(1, h->nr) / C) * C);
+    const long long need = std::max<long long>(1, (h->dyn.ecap + kCcThreads - 1) / kCcThreads);
+    const int g = (int)std::min<long long>(h->num_sms / std::max(1, h->nr), need);
+    return tuned(h->tune.scatter, std::max(1, g / C) * C);
 }
 
 int residual_grid(rorbk_ctx *h) {
@@ -3465,6 +3537,10 @@ void configure_kernels() {
                          (int)collect_smem_bytes());
     cudaFuncSetAttribute(k_topk_collect<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)collect_smem_bytes());
+    cudaFuncSetAttribute(k_topk_small<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)collect_smem_bytes());
+    cudaFuncSetAttribute(k_topk_small<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)collect_smem_bytes());
     cudaFuncSetAttribute(k_dyn_mark<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)factor_smem_bytes());
     cudaFuncSetAttribute(k_dyn_mark<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -3537,10 +3613,11 @@ void launch_dense_gram(rorbk_ctx *h, Ctl *ctl, int tensor_cores) {
 
 // A launch in clusters of C blocks.
 template <typename... A, typename... B>
-static cudaError_t cluster_launch(cudaStream_t st, void (*kernel)(A...), dim3 grid, int C, size_t smem, B... args) {
+static cudaError_t cluster_launch(cudaStream_t st, void (*kernel)(A...), dim3 grid, int threads, int C, size_t smem,
+                                  B... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
-    cfg.blockDim = dim3(kCcThreads);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
@@ -3553,8 +3630,8 @@ static cudaError_t cluster_launch(cudaStream_t st, void (*kernel)(A...), dim3 gr
 }
 
 // Blocks of the cluster that factors a Gram of order up to K (0: none is
-// needed or none can be resident).  Measured at order 256: 344 us with 16
-// blocks, 393 us with 8 (the trailing updates); at order 100 both take 127 us,
+// needed or none can be resident).  Measured at order 256: 321 us with 16
+// blocks, 361 us with 8 (the trailing updates); at order 100 both take 121 us,
 // so 8 serve orders up to 128 and a block of columns, whose clusters run side
 // by side.  Orders up to 64 have one small trailing update: 4 blocks.
 int chol_cluster_blocks(rorbk_ctx *h) {
@@ -3565,7 +3642,7 @@ int chol_cluster_blocks(rorbk_ctx *h) {
     for (int C = K <= 64 ? 4 : half ? 8 : kCcMaxCluster; C >= 1; C /= 2) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(C);
-        cfg.blockDim = dim3(kCcThreads);
+        cfg.blockDim = dim3(h->nr ? 256 : kCcThreads);
         cfg.dynamicSmemBytes = cc_smem_bytes(std::min(K, cc_max_order(C)), C);
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -3574,7 +3651,8 @@ int chol_cluster_blocks(rorbk_ctx *h) {
         cfg.attrs = at;
         cfg.numAttrs = 1;
         int n = 0;
-        const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, k_dyn_scatter<double, false, true>, &cfg);
+        const cudaError_t e = h->nr ? cudaOccupancyMaxActiveClusters(&n, k_dyn_scatter<double, false, true>, &cfg)
+                                    : cudaOccupancyMaxActiveClusters(&n, k_dyn_scatter<double, false, false>, &cfg);
         if (e == cudaSuccess && n > 0) return C;
         cudaGetLastError();
     }
@@ -3590,7 +3668,7 @@ template <typename T>
 static void launch_dense_chol(rorbk_ctx *h, const T *r, int K, const double *z0, Ctl *ctl) {
     if (K <= fac_max(h)) {
         const int C = h->dyn.cluster;
-        cluster_launch(h->stream, k_dense_chol<T>, dim3(C), C, cc_smem_bytes(K, C), r, K, dyn_bufs(h), ctl, z0);
+        cluster_launch(h->stream, k_dense_chol<T>, dim3(C), kCcThreads, C, cc_smem_bytes(K, C), r, K, dyn_bufs(h), ctl, z0);
         return;
     }
     for (int j0 = 0; j0 < K; j0 += kPW) {
@@ -3609,7 +3687,8 @@ static void launch_dyn_scatter(rorbk_ctx *h, T *x, Ctl *ctl, int count_iter, int
                                const Cols &cl) {
     const int C = std::max(1, h->dyn.cluster), g = (grid_scatter(h) + C - 1) / C * C;
     const size_t smem = h->dyn.cluster ? cc_smem_bytes(std::min(h->K, cc_max_order(C)), C) : 0;
-    cluster_launch(h->stream, k_dyn_scatter<T, LOG, MC>, dim3(g, std::max(1, h->nr)), C, smem, x, (int)h->n,
+    cluster_launch(h->stream, k_dyn_scatter<T, LOG, MC>, dim3(g, std::max(1, h->nr)), MC ? 256 : kCcThreads, C, smem, x,
+                   (int)h->n,
                    dyn_bufs(h), ctl, count_iter, use_cond, (cudaGraphConditionalHandle)hcond, cl);
 }
 
@@ -3683,7 +3762,9 @@ template <typename T, typename V>
 static void residual_launch(rorbk_ctx *h, const Mat<T> &A, const T *b, const T *x, T *r, Ctl *ctl,
                             int finalize) {
     if (h->format != RORBK_FORMAT_DENSE) {
-        k_residual<T, V><<<h->grid_res, 256, 0, h->stream>>>(A, b, x, r, h->partials, h->hist1, ctl, finalize);
+        // blocks without a slice would only zero and flush a histogram
+        const int g = std::max(1, std::min(h->grid_res, h->sell.nslices));
+        k_residual<T, V><<<g, 256, 0, h->stream>>>(A, b, x, r, h->partials, h->hist1, ctl, finalize);
         return;
     }
     const int nsl = (int)((h->m + 31) / 32), g = std::min(h->grid_res, nsl), per = (nsl + g - 1) / g;
@@ -3738,10 +3819,17 @@ void launch_iteration_t(rorbk_ctx *h, const T *b, T *x, T *r, Ctl *ctl, int use_
     }
     if constexpr (sizeof(T) == sizeof(double))
         if (weighted) launch_weights(h, r);      // the draws of the next iteration
-    k_topk_hist2<T><<<grid_topk(h), 256, 0, h->stream>>>(r, (int)h->m, h->K, h->hist2, ctl, 1, one_col((int)h->m));
-    k_topk_collect<T><<<grid_collect(h), 512, collect_smem_bytes(), h->stream>>>(
-        r, (int)h->m, h->K, h->rowptr, h->in_list, h->eq_list, dyn_bufs(h), ctl, 1, one_col((int)h->m),
-        plan_of(h, RORBK_FORMAT_DENSE));
+    // one block takes a short residual of a sparse A (the dense passes plan their
+    // draws in k_topk_collect)
+    if (h->m <= kTopkSmall && h->format == RORBK_FORMAT_CSR) {
+        k_topk_small<T><<<1, 1024, collect_smem_bytes(), h->stream>>>(r, (int)h->m, h->K, h->rowptr, h->in_list,
+                                                                      h->eq_list, dyn_bufs(h), ctl);
+    } else {
+        k_topk_hist2<T><<<grid_topk(h), 256, 0, h->stream>>>(r, (int)h->m, h->K, h->hist2, ctl, 1, one_col((int)h->m));
+        k_topk_collect<T><<<grid_collect(h), 512, collect_smem_bytes(), h->stream>>>(
+            r, (int)h->m, h->K, h->rowptr, h->in_list, h->eq_list, dyn_bufs(h), ctl, 1, one_col((int)h->m),
+            plan_of(h, RORBK_FORMAT_DENSE));
+    }
     launch_dynamic_tail<T>(h, r, x, ctl, 1, 1, use_cond, hcond, inc);
 }
 
