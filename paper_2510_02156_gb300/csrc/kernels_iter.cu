@@ -452,7 +452,9 @@ __global__ void __launch_bounds__(1024, 1) k_static(Mat<T> A, const T *__restric
                                                  Ctl *ctl, int force_tau, int use_stages,
                                                  int l_begin, int ld_) {
     extern __shared__ unsigned long long dsm_u64[];
+    constexpr int kWAhead = sizeof(T) == 8 ? 8 : 16;  // entries of a row of W read ahead of its chain
     __shared__ T rloc[kMaxBlockRows];
+    __shared__ T rs[kMaxBlockRows];
     __shared__ T y[kMaxBlockRows];
     __shared__ int taus[64];
     __shared__ int s_r0[64], s_s[64], s_p0[64], s_pend[64], s_sb[64], s_nS[64];
@@ -569,6 +571,13 @@ __global__ void __launch_bounds__(1024, 1) k_static(Mat<T> A, const T *__restric
             return;
         }
         const int la = cur.la;
+        // the coupled rows' list and the first entries of this thread's row of W:
+        // in flight during the gather and the dot products
+        const int si = a < nS ? A.s_idx[sb + a] : 0;
+        const T *Wr = A.w_ss + wb + (long long)max(cur.pos, 0) * nS;
+        T wn[kWAhead];
+#pragma unroll
+        for (int u = 0; u < kWAhead; ++u) wn[u] = a < s && cur.pos >= 0 && u < nS ? __ldg(Wr + u) : T(0);
         T acc = T(0);
         if (staged) {
             const Stage<T> st = stage_at<T>(sbase + sidx * static_stage_bytes<T>());
@@ -615,16 +624,29 @@ __global__ void __launch_bounds__(1024, 1) k_static(Mat<T> A, const T *__restric
             cur = nxt;
             continue;
         }
+        if (nS > 0) {                                 // r_tau on the coupled rows, in their order
+            if (a < nS) rs[a] = rloc[si];
+            __syncthreads();
+        }
         if (a < s) {
             if (cur.pos < 0) {
                 y[la] = Ar<T>::fma(cur.wd, rloc[la], T(0));
             } else {
-                // the loads of W's row and of the row indices do not depend on
-                // the chain: unrolled, they are in flight ahead of it
-                const T *Wr = A.w_ss + wb + (long long)cur.pos * nS;
+                // the next entries of W's row are in flight during the chain over
+                // these: a load takes longer than their links
                 T acc2 = T(0);
-#pragma unroll 8
-                for (int q = 0; q < nS; ++q) acc2 = Ar<T>::fma(Wr[q], rloc[A.s_idx[sb + q]], acc2);
+#pragma unroll 1
+                for (int q = 0; q < nS; q += kWAhead) {
+                    T w[kWAhead];
+#pragma unroll
+                    for (int u = 0; u < kWAhead; ++u) {
+                        w[u] = wn[u];
+                        wn[u] = q + kWAhead + u < nS ? __ldg(Wr + q + kWAhead + u) : T(0);
+                    }
+#pragma unroll
+                    for (int u = 0; u < kWAhead; ++u)
+                        if (q + u < nS) acc2 = Ar<T>::fma(w[u], rs[q + u], acc2);
+                }
                 y[la] = acc2;
             }
         }
