@@ -50,6 +50,8 @@ struct Ctl {
     unsigned ticket;       // last-block election of grid-wide kernels
     // radix select of the top-K keys
     int sel1, above1, prefix, above, n_in, n_eq;
+    int lvl2;              // the residual pass selected the second level too (prefix, above)
+    int pad2_;
     // trace (device pointers, FP64 mode)
     long long trace_cap;
     long long *tr_tau;
@@ -250,6 +252,7 @@ struct rorbk_ctx {
         int topk = 0, collect = 0, mark = 0, scatter = 0, residual = 0;
         int unroll = 0;   // iterations per WHILE-body execution of the graphs
     } tune;
+    double *pin_rr = nullptr;           // pinned host value: ||r||^2 of the single-step residuals
     rorbk::Ctl *ctl = nullptr;
     rorbk::Ctl *ctl_in = nullptr;       // inner (FP32) loop state of the mixed form
     // graphs

@@ -742,15 +742,23 @@ __device__ __forceinline__ void hist_add(unsigned *hist, unsigned bin, bool acti
 
 // The end of a residual pass, by the whole block: its share of the first radix
 // histogram and of ||r||^2; the last block adds the shares in block order, runs
-// the convergence test and selects the first radix bin.
+// the convergence test and selects the first radix bin.  h2 != nullptr: the block
+// also counted the second digit of the keys in bin `guess` (the bin of the
+// iteration before, which holds the K-th largest again in most iterations); if
+// the first level selects that bin, the second level is selected here too and
+// k_topk_hist2 has nothing to do.
 __device__ __forceinline__ void residual_finish(double rr, unsigned *hist, double *partials, unsigned *hist1, Ctl *ctl,
-                                                int K, int finalize) {
+                                                int K, int finalize, unsigned *h2 = nullptr, unsigned *hist2 = nullptr,
+                                                int guess = -1) {
     __shared__ double red[32];
     __shared__ int is_last;
     __syncthreads();
     if (finalize == 1)
         for (int i = threadIdx.x; i < kHistBins; i += blockDim.x)
             if (hist[i]) atomicAdd(&hist1[i], hist[i]);
+    if (h2)
+        for (int i = threadIdx.x; i < kHistBins; i += blockDim.x)
+            if (h2[i]) atomicAdd(&hist2[i], h2[i]);
     rr = block_sum(rr, red);
     if (threadIdx.x == 0) {
         partials[blockIdx.x] = rr;
@@ -795,21 +803,43 @@ __device__ __forceinline__ void residual_finish(double rr, unsigned *hist, doubl
         } else {
             for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) hist1[i] = 0u;
         }
+        if (h2) {
+            const bool hit = !stop && bin == guess;
+            int bin2 = 0, above2 = 0;
+            __syncthreads();                       // select_bin's shared results are free again
+            if (hit) select_bin(hist2, K - above, &bin2, &above2);
+            else
+                for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) hist2[i] = 0u;
+            if (threadIdx.x == 0) {
+                ctl->lvl2 = hit;
+                if (hit) {
+                    ctl->prefix = (int)((unsigned)bin << 11 | (unsigned)bin2);
+                    ctl->above = above + above2;
+                }
+            }
+        }
     }
 }
 
-template <typename T, typename V>
+// L2ND: count the second radix digit of the bin the iteration before selected
+// (residual_finish); the iteration of a sparse A that runs the grid-wide top-K.
+template <typename T, typename V, bool L2ND>
 __global__ void __launch_bounds__(256, 4) k_residual(Mat<T> A, const T *__restrict__ b,
                                                   const T *__restrict__ x, T *__restrict__ r,
-                                                  double *partials, unsigned *hist1, Ctl *ctl,
+                                                  double *partials, unsigned *hist1, unsigned *hist2, Ctl *ctl,
                                                   int finalize) {
     __shared__ unsigned hist[kHistBins];
+    __shared__ unsigned h2[L2ND ? kHistBins : 1];
     if ((finalize == 1 || finalize == 3) && (ctl->done || ctl->halt)) return;
     if (finalize == 1 && ctl->inc && !ctl->inc_full) return;   // r came from the change log
     const V *__restrict__ val = sell_values<V, T>(A);
     const int lane = threadIdx.x & 31;
     const int nwb = blockDim.x >> 5;
-    for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) hist[i] = 0u;
+    const int guess = L2ND ? ctl->sel1 : -1;
+    for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) {
+        hist[i] = 0u;
+        if (L2ND) h2[i] = 0u;
+    }
     double rr = 0.0;
     __syncthreads();
     // One resident wave of blocks; slices (longest first) are dealt to the
@@ -862,11 +892,13 @@ __global__ void __launch_bounds__(256, 4) k_residual(Mat<T> A, const T *__restri
             const T ri = Ar<T>::sub(b[row], acc);
             r[row] = ri;
             rr = __fma_rn((double)ri, (double)ri, rr);
-            bin = (unsigned)(abs_key(ri) >> 52);
+            const unsigned long long key = topk_key(ri);
+            bin = (unsigned)(key >> 52);
+            if (L2ND && (int)bin == guess) atomicAdd(&h2[(unsigned)(key >> 41) & 2047u], 1u);
         }
         if (finalize == 1) hist_add(hist, bin, act);
     }
-    residual_finish(rr, hist, partials, hist1, ctl, A.K, finalize);
+    residual_finish(rr, hist, partials, hist1, ctl, A.K, finalize, L2ND ? h2 : nullptr, hist2, guess);
 }
 
 // r = b - A x for a dense A: a pair of warps per 32 consecutive rows on a ring
@@ -1000,7 +1032,7 @@ __global__ void __launch_bounds__(256) k_inc_finish(const T *__restrict__ r, int
     if (!stop) {
         int bin, above;
         select_bin(hist1, K, &bin, &above);
-        if (threadIdx.x == 0) { ctl->sel1 = bin; ctl->above1 = above; }
+        if (threadIdx.x == 0) { ctl->sel1 = bin; ctl->above1 = above; ctl->lvl2 = 0; }
     } else {
         for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) hist1[i] = 0u;
     }
@@ -1072,7 +1104,7 @@ __global__ void __launch_bounds__(256) k_topk_hist2(const T *__restrict__ r, int
         r += blockIdx.y * cl.rs;
         hist2 += blockIdx.y * kHistBins;
     }
-    if (check_done && (ctl->done || ctl->halt)) return;
+    if (check_done && (ctl->done || ctl->halt || ctl->lvl2)) return;   // lvl2: the residual pass did this
 
     const unsigned sel1 = (unsigned)ctl->sel1;
     const int mp = MC ? cl.mpos : m;
@@ -3467,10 +3499,10 @@ int residual_grid(rorbk_ctx *h) {
     if (h->format == RORBK_FORMAT_DENSE) return h->num_sms;   // k_residual_dense: one block per SM
     int per_sm = 0, per_sm32 = 0;
     if (h->vdtype == RORBK_F32)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_residual<double, float>, 256, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_residual<double, float, true>, 256, 0);
     else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_residual<double, double>, 256, 0);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm32, k_residual<float, float>, 256, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_residual<double, double, true>, 256, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm32, k_residual<float, float, true>, 256, 0);
     return std::max(1, std::min(per_sm, per_sm32 > 0 ? per_sm32 : per_sm)) * h->num_sms;
 }
 
@@ -3786,7 +3818,10 @@ static void residual_launch(rorbk_ctx *h, const Mat<T> &A, const T *b, const T *
     if (h->format != RORBK_FORMAT_DENSE) {
         // blocks without a slice would only zero and flush a histogram
         const int g = std::max(1, std::min(h->grid_res, h->sell.nslices));
-        k_residual<T, V><<<g, 256, 0, h->stream>>>(A, b, x, r, h->partials, h->hist1, ctl, finalize);
+        if (finalize == 1 && h->m > kTopkSmall)
+            k_residual<T, V, true><<<g, 256, 0, h->stream>>>(A, b, x, r, h->partials, h->hist1, h->hist2, ctl, finalize);
+        else
+            k_residual<T, V, false><<<g, 256, 0, h->stream>>>(A, b, x, r, h->partials, h->hist1, h->hist2, ctl, finalize);
         return;
     }
     const int nsl = (int)((h->m + 31) / 32), g = std::min(h->grid_res, nsl), per = (nsl + g - 1) / g;

@@ -331,6 +331,11 @@ static rorbk_status alloc_workspace(rorbk_ctx *h) {
         !h->hist1 || !h->hist2 || !h->in_list ||
         !h->eq_list || !h->ctl || !h->ctl_in)
         return fail(h, RORBK_ERR_OOM, "workspace");
+    if (cudaMallocHost(&h->pin_rr, sizeof(double)) != cudaSuccess) {
+        cudaGetLastError();
+        h->pin_rr = nullptr;
+        return fail(h, RORBK_ERR_OOM, "pinned result");
+    }
     cudaMemsetAsync(h->hist1, 0, nr * kHistBins * sizeof(unsigned), s);
     cudaMemsetAsync(h->hist2, 0, nr * kHistBins * sizeof(unsigned), s);
     cudaMemsetAsync(h->ctl, 0, nr * sizeof(Ctl), s);
@@ -400,6 +405,7 @@ void rorbk_free(rorbk_handle h) {
     if (h->cap_stream2) cudaStreamDestroy(h->cap_stream2);
     if (h->cap_stream3) cudaStreamDestroy(h->cap_stream3);
     for (void *p : h->allocs) cudaFree(p);
+    if (h->pin_rr) cudaFreeHost(h->pin_rr);
     cudaSetDevice(cur);
     delete h;
 }
@@ -1065,6 +1071,7 @@ static rorbk_status clone_impl(rorbk_handle src, int nr, rorbk_handle *out) {
     c->err.clear();
     c->allocs.clear();
     c->tmp.clear();
+    c->pin_rr = nullptr;        // each handle its own
     c->bytes = 0;
     c->nr = 0;                  // one right-hand side (rorbk_multi_create makes blocks)
     c->mr = decltype(c->mr)();
@@ -1404,6 +1411,16 @@ rorbk_status rorbk_static_update(rorbk_handle h, int64_t tau, const double *b, d
     return st;
 }
 
+// ||r||^2 of the residual just enqueued: eight bytes into the handle's pinned
+// value (a copy into pageable memory goes through a staging buffer: 5 us more).
+static rorbk_status read_rr(rorbk_handle h, double *rr_host, const char *what) {
+    rorbk_status st = cuda_check(h, cudaMemcpyAsync(h->pin_rr, &h->ctl->rr, sizeof(double),
+                                                    cudaMemcpyDeviceToHost, h->stream), what);
+    if (!st) st = cuda_check(h, cudaStreamSynchronize(h->stream), what);
+    if (!st) *rr_host = *h->pin_rr;
+    return st;
+}
+
 rorbk_status rorbk_residual(rorbk_handle h, const double *b, const double *x, double *r,
                             double *rr_host) {
     if (!h || !b || !x || !r) return RORBK_ERR_INVALID_ARG;
@@ -1411,11 +1428,7 @@ rorbk_status rorbk_residual(rorbk_handle h, const double *b, const double *x, do
     launch_residual_only(h, b, x, r);
     rorbk_status st = cuda_check(h, cudaGetLastError(), "residual");
     if (!rr_host) return st;            // enqueue only
-    Ctl c;
-    if (!st) st = cuda_check(h, cudaMemcpyAsync(&c, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, h->stream), "residual");
-    if (!st) st = cuda_check(h, cudaStreamSynchronize(h->stream), "residual");
-    if (!st && rr_host) *rr_host = c.rr;
-    return st;
+    return st ? st : read_rr(h, rr_host, "residual");
 }
 
 rorbk_status rorbk_residual32(rorbk_handle h, const float *b, const float *x, float *r,
@@ -1427,11 +1440,7 @@ rorbk_status rorbk_residual32(rorbk_handle h, const float *b, const float *x, fl
     launch_residual32_only(h, b, x, r);
     rorbk_status st = cuda_check(h, cudaGetLastError(), "residual32");
     if (!rr_host) return st;
-    Ctl c;
-    if (!st) st = cuda_check(h, cudaMemcpyAsync(&c, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, h->stream), "residual32");
-    if (!st) st = cuda_check(h, cudaStreamSynchronize(h->stream), "residual32");
-    if (!st) *rr_host = c.rr;
-    return st;
+    return st ? st : read_rr(h, rr_host, "residual32");
 }
 
 rorbk_status rorbk_topk(rorbk_handle h, const double *r, int32_t *I) {
