@@ -252,7 +252,6 @@ struct rorbk_ctx {
         int topk = 0, collect = 0, mark = 0, scatter = 0, residual = 0;
         int unroll = 0;   // iterations per WHILE-body execution of the graphs
     } tune;
-    double *pin_rr = nullptr;           // pinned host value: ||r||^2 of the single-step residuals
     rorbk::Ctl *ctl = nullptr;
     rorbk::Ctl *ctl_in = nullptr;       // inner (FP32) loop state of the mixed form
     // graphs

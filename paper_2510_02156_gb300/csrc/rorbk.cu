@@ -331,11 +331,6 @@ static rorbk_status alloc_workspace(rorbk_ctx *h) {
         !h->hist1 || !h->hist2 || !h->in_list ||
         !h->eq_list || !h->ctl || !h->ctl_in)
         return fail(h, RORBK_ERR_OOM, "workspace");
-    if (cudaMallocHost(&h->pin_rr, sizeof(double)) != cudaSuccess) {
-        cudaGetLastError();
-        h->pin_rr = nullptr;
-        return fail(h, RORBK_ERR_OOM, "pinned result");
-    }
     cudaMemsetAsync(h->hist1, 0, nr * kHistBins * sizeof(unsigned), s);
     cudaMemsetAsync(h->hist2, 0, nr * kHistBins * sizeof(unsigned), s);
     cudaMemsetAsync(h->ctl, 0, nr * sizeof(Ctl), s);
@@ -405,7 +400,6 @@ void rorbk_free(rorbk_handle h) {
     if (h->cap_stream2) cudaStreamDestroy(h->cap_stream2);
     if (h->cap_stream3) cudaStreamDestroy(h->cap_stream3);
     for (void *p : h->allocs) cudaFree(p);
-    if (h->pin_rr) cudaFreeHost(h->pin_rr);
     cudaSetDevice(cur);
     delete h;
 }
@@ -1071,7 +1065,6 @@ static rorbk_status clone_impl(rorbk_handle src, int nr, rorbk_handle *out) {
     c->err.clear();
     c->allocs.clear();
     c->tmp.clear();
-    c->pin_rr = nullptr;        // each handle its own
     c->bytes = 0;
     c->nr = 0;                  // one right-hand side (rorbk_multi_create makes blocks)
     c->mr = decltype(c->mr)();
@@ -1411,13 +1404,15 @@ rorbk_status rorbk_static_update(rorbk_handle h, int64_t tau, const double *b, d
     return st;
 }
 
-// ||r||^2 of the residual just enqueued: eight bytes into the handle's pinned
-// value (a copy into pageable memory goes through a staging buffer: 5 us more).
+// ||r||^2 of the residual just enqueued: its eight bytes, not the whole state.  (A
+// pinned value per handle saved up to 5 us a call, but cost every handle 200 us
+// when it was closed.)
 static rorbk_status read_rr(rorbk_handle h, double *rr_host, const char *what) {
-    rorbk_status st = cuda_check(h, cudaMemcpyAsync(h->pin_rr, &h->ctl->rr, sizeof(double),
-                                                    cudaMemcpyDeviceToHost, h->stream), what);
+    double rr = 0.0;
+    rorbk_status st = cuda_check(h, cudaMemcpyAsync(&rr, &h->ctl->rr, sizeof(double), cudaMemcpyDeviceToHost,
+                                                    h->stream), what);
     if (!st) st = cuda_check(h, cudaStreamSynchronize(h->stream), what);
-    if (!st) *rr_host = *h->pin_rr;
+    if (!st) *rr_host = rr;
     return st;
 }
 
