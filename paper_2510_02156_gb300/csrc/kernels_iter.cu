@@ -1748,6 +1748,7 @@ __device__ int component_factor(double *G, int nS, const unsigned long long *pke
             const int mj = M[j];
             double d = G[pidx(mj, mj)];
             const double v = lane == j ? zi : lane > j && lane < n ? G[pidx(mi, mj)] : 0.0;
+            __syncwarp();                                     // lane j replaces the pivot below
             if (!positive(d)) {
                 if (lane == 0) *bad = 1;
                 d = 1.0;
