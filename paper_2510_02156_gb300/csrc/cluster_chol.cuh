@@ -137,8 +137,11 @@ __device__ __forceinline__ double pivot_div(double v, const Pivot &p) {      // 
     return quotient_rn(v, __dmul_rn(v, p.rl), p.l, p.rl, p.ok);
 }
 
+// (.aligned: a warp's lanes arrive together, also where the code before left them
+// apart)
 __device__ __forceinline__ void cluster_sync_all() {
     __threadfence();
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ unsigned cluster_rank() {

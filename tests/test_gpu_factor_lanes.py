@@ -53,3 +53,37 @@ def _check(s):
 @pytest.mark.parametrize("seed", [1, 2])
 def test_small_components_with_lanes_apart(cuda_ok, sizes, seed):
     _check(_groups(sizes, seed))
+
+
+@pytest.mark.parametrize("sizes", [(33,), (64, 40), (150, 5, 1), (300,)])
+def test_cluster_with_lanes_apart(cuda_ok, sizes):
+    """Components above 32 rows: the same in the cluster (4, 8 and 16 blocks)."""
+    _check(_groups(sizes, 3))
+
+
+@pytest.mark.parametrize("half", [17, 40, 150])
+def test_singular_component_is_reported(cuda_ok, half):
+    """Rows i and half + i are equal, in different sampled blocks (each regular
+    with lambda = 0) but in one dynamic set and one component: a pivot of exactly
+    0 ends the update with NOT_SPD, x as it was, and the handle goes on."""
+    m = 2 * half
+    rng = np.random.default_rng(half)
+    # 1 in the pair's own column, 2 in one that all rows share
+    cols = np.array([[i % half, half] for i in range(m)], dtype=np.int32)
+    vals = np.array([[1.0, 2.0]] * m)
+    s = W.System("pairs", m, m + 3, row_ptr=2 * np.arange(m + 1), col_idx=cols.ravel(), values=vals.ravel(),
+                 b=np.ones(m), num_blocks=2, lam=0.0)
+    # K = half rows: with num_blocks = 2 the dynamic set holds both of some pairs
+    I = np.sort(np.concatenate([np.arange(half // 2), half + np.arange(half - half // 2)])).astype(np.int32)
+    x0 = rng.standard_normal(s.n)
+    r = torch.as_tensor(rng.standard_normal(m), device="cuda")
+    with B.Handle.from_system(s) as h:
+        x = torch.as_tensor(x0.copy(), device="cuda")
+        with pytest.raises(B.RorbkError) as e:
+            h.dynamic_update(torch.as_tensor(I, device="cuda"), r, x)
+        assert e.value.status == -4
+        np.testing.assert_array_equal(x.cpu().numpy(), x0)
+        I2 = np.arange(half, dtype=np.int32)
+        h.dynamic_update(torch.as_tensor(I2, device="cuda"), r, x)
+    xo = oracle.update_with_cholesky(s, I2, s.lam, r.cpu().numpy()[:half], x0)
+    np.testing.assert_array_equal(x.cpu().numpy(), xo)
