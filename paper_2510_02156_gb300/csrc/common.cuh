@@ -297,13 +297,16 @@ __device__ __forceinline__ unsigned long long umma_desc(unsigned saddr, unsigned
 __host__ __device__ constexpr unsigned idesc_tf32_f32(int M, int N) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24);
 }
+// (.sync.aligned: the whole warp, its lanes together)
 __device__ __forceinline__ void tmem_alloc(unsigned *slot, unsigned ncols) {   // one full warp
+    __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
                  "r"(ncols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void tmem_dealloc(unsigned taddr, unsigned ncols) {  // the allocating warp
+    __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before_sync() {
@@ -329,6 +332,7 @@ __device__ __forceinline__ void mma_commit(unsigned long long *bar) {
 }
 // 32 consecutive 32-bit columns of this warp's 32 TMEM lanes (lane = thread).
 __device__ __forceinline__ void tmem_ld_32cols(unsigned taddr, unsigned (&v)[32]) {
+    __syncwarp();
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
         "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
