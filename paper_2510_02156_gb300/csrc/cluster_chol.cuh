@@ -15,8 +15,9 @@
 //     dealt over the cluster, every block factors the diagonal block itself
 //     (identical operations), so a panel needs no communication;
 //   - inside a column two warps form the pivot and divide, with 1 / sqrt(d) taken
-//     first and root and quotients from it by fused remainders (15 dependent
-//     FP64 operations, no call to sqrt or to a division), while six warps apply
+//     first and root and quotients from it by fused remainders (pivot.cuh: 13
+//     dependent FP64 operations, the column's last update included, and no call to
+//     sqrt or to a division), while six warps apply
 //     the previous column to the columns after the next, from registers;
 //   - the trailing update of a panel runs over all warps of the cluster (a lane
 //     per column, a few rows per warp) from a copy of the panel in shared memory;
@@ -46,6 +47,7 @@
 #include <stdint.h>
 
 #include "common.cuh"
+#include "pivot.cuh"
 
 namespace rorbk {
 
@@ -54,88 +56,6 @@ constexpr int kCwp = kCw + 1;           // row stride of panels in shared memory
 constexpr int kCcThreads = 512;          // one system at a time (256 for a block of columns)
 constexpr int kCcMaxCluster = 16;       // blocks per cluster
 constexpr int kCcMaxRows = 32;          // rows below the diagonal block per block: one per lane
-
-// Comparisons with zero on the integer side: an FP64 comparison occupies the
-// FP64 unit for as long as a multiply-add.  (The halves are taken apart in PTX:
-// the compiler turns a 64-bit test of the bit pattern back into an FP64
-// comparison, which tripled the time of the trailing update.)
-__device__ __forceinline__ int2 halves(double v) {
-    int2 h;
-    asm("mov.b64 {%0, %1}, %2;" : "=r"(h.x), "=r"(h.y) : "d"(v));
-    return h;
-}
-__device__ __forceinline__ bool nonzero(double v) {
-    const int2 h = halves(v);
-    return ((h.y & 0x7fffffff) | h.x) != 0;
-}
-__device__ __forceinline__ bool positive(double v) {     // v > 0 (false for NaN)
-    const int2 h = halves(v);
-    return h.y >= 0 && (h.y | h.x) != 0 && (h.y < 0x7ff00000 || (h.y == 0x7ff00000 && h.x == 0));
-}
-// g - la lb.  The definition skips a zero factor; adding its zero product
-// changes nothing but the sign of a zero.  (A factor that is not finite makes
-// its own row's pivot not positive either way.)
-__device__ __forceinline__ double sub_prod(double g, double la, double lb) { return __fma_rn(-la, lb, g); }
-
-// Square root and quotients by fused remainders (P. W. Markstein, IBM J. Res.
-// Dev. 34, 1990), built so that the reciprocal is there before the root.
-//   pivot_recip(d): y = 1 / sqrt(d) to about half a unit in the last place: the
-//     hardware's approximation y0 and one third-order step, the first terms of
-//     (1 - e)^(-1/2) = 1 + e / 2 + 3 e^2 / 8 + ... for e = 1 - d y0^2;
-//   pivot_root(d, y): l = RN(sqrt(d)): s = d y, its remainder d - s^2 is exact,
-//     and s + (d - s^2) y / 2 rounds to the root;
-//   reciprocal_rn(l, y): one Newton step takes y to the rounded 1 / l;
-//   quotient_rn(v, q0, l, rl): q0 = v y, the remainder v - q0 l is exact, and
-//     q0 + (v - q0 l) rl rounds to v / l.
-// Three dependent operations per quotient instead of the nine of a division.
-// root_ok and quotient_rn's test keep every intermediate normal, and a mantissa
-// of all ones (whose rounded reciprocal is not guaranteed) out; other operands
-// take sqrt and the division themselves.
-__device__ __forceinline__ unsigned exponent(double v) { return ((unsigned)halves(v).y >> 20) & 0x7ffu; }
-__device__ __forceinline__ bool root_ok(double d) { return exponent(d) - 423u <= 1200u; }
-__device__ __forceinline__ double pivot_recip(double d) {
-    double y0;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(d));
-    const double e = __fma_rn(-__dmul_rn(d, y0), y0, 1.0);
-    return __fma_rn(__fma_rn(0.375, e, 0.5), __dmul_rn(e, y0), y0);
-}
-__device__ __forceinline__ double pivot_root(double d, double y) {
-    const double s = __dmul_rn(d, y);
-    const double h = __hiloint2double(halves(y).y - (1 << 20), halves(y).x);   // y / 2 (y is normal)
-    return __fma_rn(__fma_rn(-s, s, d), h, s);
-}
-__device__ __noinline__ double slow_root(double d) { return sqrt(d); }
-__device__ __noinline__ double slow_div(double v, double l) { return v / l; }
-__device__ __forceinline__ double reciprocal_rn(double l, double y) {
-    return __fma_rn(y, __fma_rn(-l, y, 1.0), y);
-}
-__device__ __forceinline__ bool divisor_ok(double l) {      // |exponent| <= 300, mantissa not all ones
-    const int2 h = halves(l);
-    return exponent(l) - 723u <= 600u && ((h.y & 0xfffff) != 0xfffff || h.x != -1);
-}
-__device__ __forceinline__ double quotient_rn(double v, double q0, double l, double rl, bool ok) {
-    double q = __fma_rn(__fma_rn(-q0, l, v), rl, q0);
-    if (!(ok & (exponent(v) - 423u <= 1200u || !nonzero(v)))) q = slow_div(v, l);
-    return q;
-}
-
-// A pivot d > 0: l = RN(sqrt(d)), rl = RN(1 / l), and y ~ 1 / sqrt(d).
-struct Pivot {
-    double l, rl, y;
-    bool ok;
-};
-__device__ __forceinline__ Pivot pivot(double d) {
-    Pivot p;
-    const bool in = root_ok(d);
-    p.y = in ? pivot_recip(d) : 1.0 / slow_root(d);
-    p.l = in ? pivot_root(d, p.y) : slow_root(d);
-    p.rl = reciprocal_rn(p.l, p.y);
-    p.ok = divisor_ok(p.l);
-    return p;
-}
-__device__ __forceinline__ double pivot_div(double v, const Pivot &p) {      // RN(v / l)
-    return quotient_rn(v, __dmul_rn(v, p.rl), p.l, p.rl, p.ok);
-}
 
 // (.aligned: a warp's lanes arrive together, also where the code before left them
 // apart)
@@ -242,7 +162,7 @@ __device__ __forceinline__ void cc_panel(double *Ld, double *R, int w, int nr, d
                 q = v * rl;
             } else {
                 const Pivot pv = pivot(d);
-                q = quotient_rn(v, __dmul_rn(v, pv.y), pv.l, pv.rl, pv.ok);   // v y: not behind l and rl
+                q = pivot_div_early(v, pv);
                 rl = pv.rl;
                 dg = pv.l;
             }
