@@ -51,7 +51,7 @@ struct Ctl {
     // radix select of the top-K keys
     int sel1, above1, prefix, above, n_in, n_eq;
     int lvl2;              // the residual pass selected the second level too (prefix, above)
-    int pad2_;
+    int pre_ok;            // pre_* hold the draws of Philox counter pre_it
     // trace (device pointers, FP64 mode)
     long long trace_cap;
     long long *tr_tau;
@@ -80,7 +80,8 @@ struct Ctl {
     const double *scdf;    // the running sum the static draws use (P's, or the weighted one)
     int fault;             // RORBK_FAULT_* injected by the host (tests of the failure paths)
     // the next iteration's draws and their blocks' ranges, formed ahead by the
-    // top-K pass (pre_it = that iteration's Philox counter + 1; 0: none)
+    // top-K pass or the dynamic update, and that iteration's Philox counter (any
+    // value is one: pre_ok says whether they are there)
     long long pre_it;
     int pre_tau[8], pre_r0[8], pre_s[8], pre_p0[8], pre_pend[8], pre_sb[8], pre_nS[8];
     long long pre_wb[8];

@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(1024, 1) k_static(Mat<T> A, const T *__restric
     T *sx = (T *)(sbase + 2 * static_stage_bytes<T>());
     const long long cnt = ctl->iter_base + ctl->iter;
     // the draws and ranges formed ahead by the previous iteration's top-K pass
-    const bool planned = force_tau < 0 && nst <= kPreDraws && ctl->pre_it == cnt + 1;
+    const bool planned = force_tau < 0 && nst <= kPreDraws && ctl->pre_ok && ctl->pre_it == cnt;
     if (force_tau >= 0) {
         if (a == 0) taus[0] = force_tau;
         __syncthreads();
@@ -1421,7 +1421,8 @@ __device__ void plan_next(const Plan &pl, Ctl *ctl) {
     __syncthreads();
     if (a == 0) {
         __threadfence();
-        ctl->pre_it = next + 1;
+        ctl->pre_it = next;
+        ctl->pre_ok = 1;
     }
 }
 
@@ -2243,7 +2244,7 @@ constexpr int kDenseStatic = 3;
 template <typename T>
 __device__ __forceinline__ int drawn_block(const Mat<T> &A, const Ctl *ctl, int l) {
     const long long it = ctl->iter_base + ctl->iter;
-    if (ctl->pre_it == it + 1 && ctl->n_static <= kPreDraws) return ctl->pre_tau[l];
+    if (ctl->pre_ok && ctl->pre_it == it && ctl->n_static <= kPreDraws) return ctl->pre_tau[l];
     return sample_block(ctl->scdf ? ctl->scdf : A.cdf, A.k, ctl->seed, ctl->sysid, (uint64_t)it, (uint64_t)l);
 }
 
@@ -2928,7 +2929,7 @@ __global__ void __launch_bounds__(256) k_inner_prep(const double *__restrict__ r
         in->halt = !(bn > 0.0 && in->maxit > 0);
         in->status = 0;
         in->ticket = 0;
-        in->pre_it = 0;
+        in->pre_ok = 0;
         in->n_in = 0;
         in->n_eq = 0;
         in->trace_cap = 0;
@@ -3399,7 +3400,7 @@ __global__ void __launch_bounds__(256) k_mr_inner_prep(const double *__restrict_
             in->halt = 1;
         }
         in->ticket = 0;
-        in->pre_it = 0;
+        in->pre_ok = 0;
         in->n_in = 0;
         in->n_eq = 0;
         in->trace_cap = 0;
