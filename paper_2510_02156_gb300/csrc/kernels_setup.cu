@@ -839,7 +839,8 @@ __global__ void k_col_gather(const int *__restrict__ slot, const int *__restrict
 // Device scratch of one set-up pass, freed when the pass ends (after the
 // stream has drained).  With a size, one allocation that the buffers share (a
 // refresh knows its sizes; an allocation and its release cost tens of
-// microseconds each).
+// microseconds each); back_to gives what was taken from it since a mark to the
+// stream's later kernels.
 struct Scratch {
     cudaStream_t s;
     std::vector<void *> p;
@@ -857,6 +858,11 @@ struct Scratch {
     }
     Scratch(const Scratch &) = delete;
     Scratch &operator=(const Scratch &) = delete;
+    char *mark() const { return arena; }
+    void back_to(char *m) {
+        left += (size_t)(arena - m);
+        arena = m;
+    }
     static size_t room(size_t bytes) { return (std::max<size_t>(bytes, 16) + 255) & ~(size_t)255; }
     template <typename T>
     T *get(size_t count) {
@@ -997,13 +1003,15 @@ rorbk_status build_setup(rorbk_ctx *h, const std::vector<int> &hrp, bool refresh
     cudaStream_t s = h->stream;
     const int m = (int)h->m, n = (int)h->n, k = h->k;
     rorbk_status st;
-    // a refresh of a sparse A: every scratch buffer below in one allocation
+    // a refresh of a sparse A: every scratch buffer below in one allocation, the
+    // operators' over the centroids', which are done with by then
     size_t bytes = 0;
     if (refresh && h->format == RORBK_FORMAT_CSR && !h->n_wood) {
         const size_t segs = std::max(1, h->bt.total_segs);
-        for (size_t b : {(size_t)8, (size_t)(n + 1) * 4, (size_t)(n + 1) * 4, (size_t)(scan_tiles(n + 1) + 1) * 4, (size_t)4,
-                         segs * 4, segs * 8, (size_t)k * k * 8, (size_t)k * 8, (size_t)std::max(1LL, h->ops.w_total) * 8})
+        for (size_t b : {(size_t)(n + 1) * 4, (size_t)(n + 1) * 4, (size_t)(scan_tiles(n + 1) + 1) * 4, (size_t)4,
+                         segs * 4, segs * 8, (size_t)k * k * 8, (size_t)k * 8})
             bytes += Scratch::room(b);
+        bytes = std::max(bytes, Scratch::room((size_t)std::max(1LL, h->ops.w_total) * 8)) + Scratch::room(8);
     }
     Scratch sc(s, bytes);
     int *flags = sc.get<int>(2);
@@ -1073,8 +1081,9 @@ rorbk_status build_setup(rorbk_ctx *h, const std::vector<int> &hrp, bool refresh
 
     // centroids, C row sums, proposal
     {
-        Scratch own(s);                              // of this part, unless the arena holds it
-        Scratch &cs = bytes ? sc : own;
+        Scratch own(s);                              // of this part, unless the one allocation holds it
+        Scratch &cs = sc.arena ? sc : own;
+        char *const part = sc.mark();
         int *colcnt = cs.get<int>(n + 1);
         int *fill = cs.get<int>(n + 1);
         if (!colcnt || !fill) return fail(h, RORBK_ERR_OOM, "centroid columns");
@@ -1108,6 +1117,7 @@ rorbk_status build_setup(rorbk_ctx *h, const std::vector<int> &hrp, bool refresh
         k_crowsum<<<(k * 32 + 255) / 256, 256, 0, s>>>(G, nrm, k, h->crowsum);
         k_proposal<<<1, 1024, 0, s>>>(h->crowsum, k, (double)n, h->cdf, h->pbar);
         if ((st = cuda_check(h, cudaGetLastError(), "proposal"))) return st;
+        sc.back_to(part);
     }
 
     // static operators on the coupled rows of every block

@@ -559,37 +559,43 @@ rorbk_status rorbk_update_values(rorbk_handle h, const void *values, int32_t dty
     const size_t esz = dtype == RORBK_F64 ? sizeof(double) : sizeof(float);
     const long long nnz = h->nnz;
     rorbk_status st = cuda_check(h, cudaStreamSynchronize(s), "rorbk_update_values");
-    // the new values in scratch first, checked before the handle is touched
-    void *tmp = nullptr;
-    int *bad = nullptr;
+    // the new values are checked before the handle is touched: where they are, if
+    // that is this device's memory, else in scratch that is given back before the
+    // set-up is re-formed (a copy of A kept through it would raise the refresh's peak
+    // by as much as A's values take)
     if (!st && nnz) {
-        cudaError_t e = cudaMalloc(&tmp, nnz * esz + sizeof(int));
-        if (e != cudaSuccess) {
+        cudaPointerAttributes at = {};
+        const bool here = on_device && cudaPointerGetAttributes(&at, values) == cudaSuccess &&
+                          at.type == cudaMemoryTypeDevice && at.device == h->device;
+        cudaGetLastError();
+        const size_t copy = here ? 0 : nnz * esz;
+        void *tmp = nullptr;
+        if (cudaMalloc(&tmp, copy + sizeof(int)) != cudaSuccess) {
             cudaGetLastError();
             cudaSetDevice(cur);
             return fail(h, RORBK_ERR_OOM, "rorbk_update_values: scratch");
         }
-        bad = (int *)((char *)tmp + nnz * esz);
+        int *bad = (int *)((char *)tmp + copy);
+        const void *src = here ? values : tmp;
         cudaMemsetAsync(bad, 0, sizeof(int), s);
-        cudaMemcpyAsync(tmp, values, nnz * esz, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s);
+        if (!here)
+            cudaMemcpyAsync(tmp, values, copy, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s);
         const int g = (int)std::max(1LL, std::min<long long>(8LL * h->num_sms, (nnz + 255) / 256));
-        if (dtype == RORBK_F64) k_count_nonfinite_f64<<<g, 256, 0, s>>>((const double *)tmp, nnz, bad);
-        else k_count_nonfinite_f32<<<g, 256, 0, s>>>((const float *)tmp, nnz, bad);
+        if (dtype == RORBK_F64) k_count_nonfinite_f64<<<g, 256, 0, s>>>((const double *)src, nnz, bad);
+        else k_count_nonfinite_f32<<<g, 256, 0, s>>>((const float *)src, nnz, bad);
         int hb = 0;
         st = cuda_check(h, cudaMemcpyAsync(&hb, bad, sizeof(int), cudaMemcpyDeviceToHost, s), "rorbk_update_values");
         if (!st) st = cuda_check(h, cudaStreamSynchronize(s), "rorbk_update_values");
         if (!st && hb) st = fail(h, RORBK_ERR_NUMERIC, "rorbk_update_values: the values hold NaN or Inf");
         if (!st) {
-            cudaMemcpyAsync(dtype == RORBK_F64 ? (void *)h->val : (void *)h->val32, tmp, nnz * esz,
+            cudaMemcpyAsync(dtype == RORBK_F64 ? (void *)h->val : (void *)h->val32, src, nnz * esz,
                             cudaMemcpyDeviceToDevice, s);
             widen_values(h, dtype);
+            if (!here) st = cuda_check(h, cudaStreamSynchronize(s), "rorbk_update_values");
         }
-    }
-    if (!st) st = build_setup(h, std::vector<int>(), true);
-    if (tmp) {
-        cudaStreamSynchronize(s);
         cudaFree(tmp);
     }
+    if (!st) st = build_setup(h, std::vector<int>(), true);
     if (!st && h->values_version) ++*h->values_version;
     // this handle's own column-major copy now; those of handles sharing the
     // set-up at their next incremental solve
