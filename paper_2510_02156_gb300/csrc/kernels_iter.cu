@@ -904,10 +904,19 @@ __global__ void __launch_bounds__(256, 4) k_residual(Mat<T> A, const T *__restri
 // r = b - A x for a dense A: a pair of warps per 32 consecutive rows on a ring
 // of stages (dense_rows.cuh), row-major values, one block per SM.  W pairs per
 // block run, with longer and more stages the fewer they are, so that a short A
-// (few chains) keeps more bytes of each in flight.
+// (few chains) keeps more bytes of each in flight.  A warp's number decides which
+// quarter of the SM issues it: from five pairs on, and where FP32 values are widened
+// from two on, the summing warps are the first eight and the copying warps the others, one
+// quarter further on, so that every quarter has its share of both.  (With the two kinds
+// taking turns the sums ran in two quarters.  Whole calls at 200,000 x 2,048: 760 us
+// in FP64 against 724, 1,233 against 822 over FP32 values, whose widening is integer
+// work; 15,000 rows of those 164 against 141.  Four chains of FP64 values, 15,000 rows, are
+// better off in turns: 117 us against 125.)
 // 200,000 x 2,048 FP32: 300 -> 262 us, 0.92 of measured HBM; 25,600 x 2,048 FP64:
 // 175 -> 117 us (bound by the FP64 rate: 107); 2,048 x 100,000: 8,300 -> 3,628 us
 // FP64, 4,280 -> 284 us FP32 (bound by the chains: 3,200 and 240).
+constexpr int kDrMaxPairs = 8;
+
 template <typename T, typename V, int RB, int ST>
 __host__ __device__ constexpr size_t dense_res_smem(int W) { return (size_t)W * ST * DenseStage<T, V, RB>::bytes; }
 
@@ -919,8 +928,10 @@ __global__ void __launch_bounds__(512, 1) k_residual_dense(const V *__restrict__
     extern __shared__ __align__(16) unsigned char dr_ring[];
     __shared__ unsigned hist[kHistBins];
     if ((finalize == 1 || finalize == 3) && (ctl->done || ctl->halt)) return;
-    const int lane = threadIdx.x & 31, pair = ST == 8 ? 0 : threadIdx.x >> 6;
-    const bool load = (threadIdx.x >> 5) & 1;
+    constexpr bool spread = ST == 3 || (ST == 6 && sizeof(V) < sizeof(T));
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool load = spread ? warp >= kDrMaxPairs : warp & 1;
+    const int pair = spread ? (warp - load) & (kDrMaxPairs - 1) : ST == 8 ? 0 : warp >> 1;
     for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) hist[i] = 0u;
     __syncthreads();
     double rr = 0.0;
@@ -3634,7 +3645,6 @@ int residual_grid(rorbk_ctx *h) {
 }
 
 // The rings of k_residual_dense: long stages and many of them for few pairs.
-constexpr int kDrMaxPairs = 8;
 template <typename T, typename V>
 static void configure_residual_dense() {
     cudaFuncSetAttribute(k_residual_dense<T, V, 512, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
