@@ -11,9 +11,9 @@
 //                  the last block completes the exact top-K set
 //   k_dyn_mark     gathers A_I, marks shared columns, Gram diagonal; the last
 //                  block factors G = A_I A_I^T + mu I on the coupled rows' small
-//                  components and solves for y, the first block done forms the
-//                  next draws
-//   k_dyn_scatter  the large components in one cluster, x += A_I^T y; ends the
+//                  components and on large ones that are shallow trees and solves
+//                  for y, the first block done forms the next draws
+//   k_dyn_scatter  the other large components in one cluster, x += A_I^T y; ends the
 //                  iteration, sets the loop condition
 //
 // Compute type T is double (the plain method) or float (the inner solve of
@@ -23,9 +23,9 @@
 // columns; column-ordered triangular solves), so the iterates reproduce the
 // FP64 definition exactly.  FP64 arithmetic on this part has a long latency,
 // so chains are kept short: the Cholesky of the coupled rows runs per
-// connected component, one warp each, or, for components above 32 rows, in one
-// thread-block cluster (cluster_chol.cuh); both perform the operations of the
-// whole-matrix factor on every entry in the same order.
+// connected component, one warp each, or, for components above 32 rows, level by
+// level (shallow trees) or in one thread-block cluster (cluster_chol.cuh); all
+// perform the operations of the whole-matrix factor on every entry in the same order.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -2490,10 +2490,11 @@ __global__ void __launch_bounds__(256) k_sd_wood(Mat<T> A, const T *__restrict__
 // ---- the dynamic update of a dense A -------------------------------------
 // Every row of I holds every column, so all of I is coupled and the Gram is
 // dense: G = A_I A_I^T + mu I (packed lower, D.g), each entry one fused chain
-// over ascending columns as in the definition; one block factors it and
-// solves (the same right-looking Cholesky and column-oriented solves as the
-// sparse coupled set); x += A_I^T y, each column summed over ascending rows
-// of I, then added.
+// over ascending columns as in the definition; one cluster factors it and
+// solves up to its largest order (cluster_chol.cuh; above it the grid, below), with the
+// operations of the right-looking Cholesky and the column-oriented solves of the
+// sparse coupled set; x += A_I^T y, each column summed over ascending rows of I,
+// then added.
 //
 // The FP64 Gram: one warp per patch of 4 rows x 8 columns of the lower triangle
 // (a lane per entry), on its own ring of stages of the 12 rows.  Bound by the
@@ -2574,10 +2575,10 @@ __global__ void __launch_bounds__(32) k_dyn_dense_gram(const double *__restrict_
 // G = A_I A_I^T + mu I from the FP32 copy of A: TF32 products accumulated in
 // FP32 by tcgen05.mma, in kTcRows x kTcRows tiles of the lower triangle.  Grid
 // block (t, s) takes tile t and the s-th share of the column chunks (kTcCols
-// columns each).  Per chunk it stages the tile's rows in shared memory as core
-// matrices (see umma_desc), one thread issues the chunk's MMAs into a TMEM
-// accumulator and commits them to an mbarrier, and the block waits before it
-// stages the next chunk.  The accumulator is written as an FP32 partial tile;
+// columns each).  It stages the tile's rows in shared memory as core matrices (see
+// umma_desc), half a chunk to a slot; one thread issues a slot's MMAs into a TMEM
+// accumulator and commits them to the slot's mbarrier, which is waited for before the
+// slot is filled again, two halves later.  The accumulator is written as an FP32 partial tile;
 // k_dyn_gram_reduce adds a tile's partials in split order in FP64, adds mu on
 // the diagonal and writes the packed G that the FP64 Cholesky reads.
 //
@@ -2745,7 +2746,9 @@ __global__ void __launch_bounds__(256) k_dyn_gram_reduce(const float *__restrict
     }
 }
 
-// Blocked factor of the dense Gram: panels of kPW columns.  The panel kernel
+// Blocked factor of a dense Gram too large for a cluster (orders above 543, or
+// above what the clusters that can be resident take; launch_dense_chol): panels of kPW
+// columns, over the grid.  The panel kernel
 // factors the panel's columns, right-looking inside the panel, and carries the
 // forward solve for them (z is the panel's extra column); the trailing kernel
 // (many blocks) applies the panel's columns to every later entry, in
@@ -2755,8 +2758,8 @@ __global__ void __launch_bounds__(256) k_dyn_gram_reduce(const float *__restrict
 constexpr int kPW = 32;
 
 // ---- the dynamic block in the n x n form (K >= n; Lemma 1) ----------------
-// G = A_I^T A_I + mu I, h = A_I^T r_I, y = G^{-1} h by the blocked Cholesky and
-// its solves (size n, z starting at h), then x_c += y_c.  The rows of I are
+// G = A_I^T A_I + mu I, h = A_I^T r_I, y = G^{-1} h by the same factor and
+// solves (size n, z starting at h), then x_c += y_c.  The rows of I are
 // first laid out as a dense K x n array (dw; unstored entries zero), so the
 // column sums run over the rows in ascending order as in the definition.
 __global__ void __launch_bounds__(256) k_dynw_rows(const int *__restrict__ rowptr, const int *__restrict__ col,
