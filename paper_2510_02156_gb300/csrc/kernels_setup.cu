@@ -562,7 +562,21 @@ __device__ __forceinline__ void spd_inverse_from_factor(double *G, double *Li, i
 // flags and S offsets; outputs W on S (row-major |S|^2 at w_ss + w_ptr[t]),
 // W_ii for uncoupled rows, and s_idx / s_pos.  Linv scratch has the layout of
 // w_ss.
+//
+// Two instances share the blocks: SMALL those of up to kSoSmall coupled rows, whose
+// factor and inverse, chains of dependent accesses, run in shared memory; the other
+// those above, whose matrices stay in global memory and live on the L1 cache.  What the
+// kernel may take as shared memory is lost to L1, so the second asks for a quarter of
+// it (kSoCarveout; 40% was 0 to 10% slower) and stages the entries only, and those only
+// where rows are long.  Value refreshes, everything in global memory / all blocks in one
+// launch with the first instance's shared memory / now: 640 blocks of 250 coupled rows
+// of five entries 25.4, 57.3, 21.9 ms; 90 blocks of 1,000 608, 990, 581; 19 blocks of 263
+// rows of a power-law system 13.6, 15.6, 9.9.
 constexpr int kSoStage = 8192;        // entries of a block staged for the merges of its rows
+constexpr int kSoSmall = 64;
+constexpr int kSoCarveout = 25;       // percent
+constexpr int kSoShort = 8;           // rows too short for staging to pay
+template <bool SMALL>
 __global__ void k_static_ops(const int *__restrict__ rowptr, const int *__restrict__ col,
                              const double *__restrict__ val, const int *__restrict__ off,
                              double mu, const unsigned char *__restrict__ coupled,
@@ -571,14 +585,16 @@ __global__ void k_static_ops(const int *__restrict__ rowptr, const int *__restri
                              double *__restrict__ w_ss, double *__restrict__ w_diag,
                              double *__restrict__ linv, const long long *__restrict__ wood_ptr,
                              int *__restrict__ status, int gram_ready, const double *__restrict__ rn, int stage,
-                             int mat) {
+                             int first) {
     extern __shared__ double so_val[];           // [stage] values, then columns, of the block's entries;
-                                                 // then, over them, two matrices of mat doubles together
+                                                 // SMALL: then, over them, the two matrices
     __shared__ int scan_scratch[33];
     __shared__ int bad;
     __shared__ double gdiag[kMaxBlockRows];
     const int t = blockIdx.x;
     const int r0 = off[t], s = off[t + 1] - r0;
+    const int sb = s_ptr[t], nS = s_ptr[t + 1] - sb;
+    if (SMALL ? nS > kSoSmall : nS < first) return;   // the other instance's
     if (wood_ptr && wood_ptr[t] >= 0) {          // the n x n form serves this block
         for (int a = threadIdx.x; a < s; a += blockDim.x) {
             s_pos[r0 + a] = -1;
@@ -586,7 +602,6 @@ __global__ void k_static_ops(const int *__restrict__ rowptr, const int *__restri
         }
         return;
     }
-    const int sb = s_ptr[t], nS = s_ptr[t + 1] - sb;
     double *G = w_ss + w_ptr[t];
     double *Li = linv + w_ptr[t];
     if (threadIdx.x == 0) bad = 0;
@@ -644,9 +659,7 @@ __global__ void k_static_ops(const int *__restrict__ rowptr, const int *__restri
             G[(long long)i * nS + j] = g;
         }
         __syncthreads();
-        if (2LL * nS * nS <= mat) {
-            // the factor and the inverse are chains of dependent accesses: in
-            // shared memory (over the staged entries) where both matrices fit
+        if constexpr (SMALL) {
             double *Gs = so_val, *Ls = so_val + nS * nS;
             for (int idx = threadIdx.x; idx < nS * nS; idx += blockDim.x) Gs[idx] = idx / nS >= idx % nS ? G[idx] : 0.0;
             __syncthreads();
@@ -1172,14 +1185,22 @@ rorbk_status build_setup(rorbk_ctx *h, const std::vector<int> &hrp, bool refresh
             k_dense_static_gram<<<dim3(nt * (nt + 1) / 2, k), kSgT * kSgT, 0, s>>>(h->val, h->off, n, h->mu,
                                                                                  h->ops.w_ptr, h->ops.w_ss);
         }
-        const int stage = dense_gram ? 0 : std::min(kSoStage, (h->bt.max_entries + 1) & ~1);
-        // two matrices of the largest coupled set, up to 64 rows (three blocks per SM)
-        const int mat = dense_gram ? 0 : 2 * std::min(h->ops.max_coupled, 64) * std::min(h->ops.max_coupled, 64);
-        cudaFuncSetAttribute(k_static_ops, cudaFuncAttributeMaxDynamicSharedMemorySize, kSoStage * 12);
-        k_static_ops<<<k, 256, std::max((size_t)stage * 12, (size_t)mat * 8), s>>>(h->rowptr, h->col, h->val, h->off, h->mu, coupled,
-                                                        h->ops.s_ptr, h->ops.w_ptr, h->ops.s_idx, h->ops.s_pos,
-                                                        h->ops.w_ss, h->ops.w_diag, linv, h->wood_ptr, flags,
-                                                        dense_gram ? 1 : 0, h->rn, stage, mat);
+        const int mc = h->ops.max_coupled, me = h->bt.max_entries;
+        auto ops = [&](auto kernel, int stage, size_t smem, int first) {
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSoStage * 12);
+            kernel<<<k, 256, smem, s>>>(h->rowptr, h->col, h->val, h->off, h->mu, coupled, h->ops.s_ptr, h->ops.w_ptr,
+                                        h->ops.s_idx, h->ops.s_pos, h->ops.w_ss, h->ops.w_diag, linv, h->wood_ptr, flags,
+                                        dense_gram ? 1 : 0, h->rn, stage, first);
+        };
+        if (!dense_gram) {
+            const int stage = std::min(kSoStage, (me + 1) & ~1), c = std::min(mc, kSoSmall);
+            ops(k_static_ops<true>, stage, std::max((size_t)stage * 12, (size_t)c * c * 16), 0);
+        }
+        if (dense_gram || mc > kSoSmall) {
+            const int stage = dense_gram || me > kSoStage || h->maxrow <= kSoShort ? 0 : (me + 1) & ~1;
+            cudaFuncSetAttribute(k_static_ops<false>, cudaFuncAttributePreferredSharedMemoryCarveout, kSoCarveout);
+            ops(k_static_ops<false>, stage, (size_t)stage * 12, dense_gram ? 0 : kSoSmall + 1);
+        }
         if (h->n_wood) {
             double *linv2 = sc.get<double>(wtot);
             if (!linv2) return fail(h, RORBK_ERR_OOM, "s >= n operator scratch");
