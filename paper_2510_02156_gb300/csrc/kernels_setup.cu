@@ -87,7 +87,9 @@ __device__ __forceinline__ int row_of_entry(const int *rowptr, int lo, int hi, i
     return lo;
 }
 
-// sort: entries that the launch's dynamic shared memory holds (a power of two).
+// sort: entries that the launch's dynamic shared memory holds (a power of two); 0:
+// the blocks above kBtSort, whose searches want the L1 cache that the shared memory
+// would take.
 __global__ void k_block_transpose(const int *__restrict__ rowptr, const int *__restrict__ col,
                                   const double *__restrict__ val, const int *__restrict__ off,
                                   int *__restrict__ bt_col, uint16_t *__restrict__ bt_row,
@@ -101,9 +103,10 @@ __global__ void k_block_transpose(const int *__restrict__ rowptr, const int *__r
     const int t = blockIdx.x;
     const int r0 = off[t], r1 = off[t + 1], s = r1 - r0;
     const int p0 = rowptr[r0], E = rowptr[r1] - p0;
+    if (sort ? E > sort : E <= kBtSort) return;
     for (int a = threadIdx.x; a < s; a += blockDim.x) flag[a] = 0;
 
-    if (E <= sort) {
+    if (sort) {
         const int np = next_pow2(max(E, 1));
         for (int e = threadIdx.x; e < np; e += blockDim.x)
             bt_keys[e] = e < E ? (unsigned long long)(unsigned)col[p0 + e] << 32 | (unsigned)e : ~0ull;
@@ -1086,9 +1089,12 @@ rorbk_status build_setup(rorbk_ctx *h, const std::vector<int> &hrp, bool refresh
                 h->bt.max_entries = std::max(h->bt.max_entries, hrp[h->h_off[t + 1]] - hrp[h->h_off[t]]);
         const int sort = std::min(kBtSort, next_pow2(std::max(1, h->bt.max_entries)));
         cudaFuncSetAttribute(k_block_transpose, cudaFuncAttributeMaxDynamicSharedMemorySize, kBtSort * 8);
-        k_block_transpose<<<k, 256, (size_t)sort * 8, s>>>(h->rowptr, h->col, h->val, h->off, h->bt.col, h->bt.row,
-                                                           h->bt.val, h->bt.off16, h->bt.seg, h->bt.seg_ptr, coupled,
-                                                           ncoupled, sort);
+        for (int so : {sort, 0}) {
+            if (!so && h->bt.max_entries <= kBtSort) break;
+            k_block_transpose<<<k, 256, (size_t)so * 8, s>>>(h->rowptr, h->col, h->val, h->off, h->bt.col, h->bt.row,
+                                                             h->bt.val, h->bt.off16, h->bt.seg, h->bt.seg_ptr, coupled,
+                                                             ncoupled, so);
+        }
     }
     if ((st = cuda_check(h, cudaGetLastError(), "block transpose"))) return st;
 
