@@ -571,15 +571,21 @@ __global__ void __launch_bounds__(1024, 1) k_static(Mat<T> A, const T *__restric
             return;
         }
         const int la = cur.la;
-        // the coupled rows' list and the first entries of this thread's row of W:
-        // in flight during the gather and the dot products
+        // the coupled rows' list and the first entries of this thread's row of W: in
+        // flight during the gather and the dot products of a staged block.  (Rows read
+        // from global memory want the registers for their own loads: one update
+        // of 30,000 x 1,001 in blocks of 254 rows took 950 us without these, 1,064
+        // with them held during the rows, 910 with them loaded behind the rows.)
         const int si = a < nS ? A.s_idx[sb + a] : 0;
         const T *Wr = A.w_ss + wb + (long long)max(cur.pos, 0) * nS;
         T wn[kWAhead];
+        auto first_of_w = [&]() {
 #pragma unroll
-        for (int u = 0; u < kWAhead; ++u) wn[u] = a < s && cur.pos >= 0 && u < nS ? __ldg(Wr + u) : T(0);
+            for (int u = 0; u < kWAhead; ++u) wn[u] = a < s && cur.pos >= 0 && u < nS ? __ldg(Wr + u) : T(0);
+        };
         T acc = T(0);
         if (staged) {
+            first_of_w();
             const Stage<T> st = stage_at<T>(sbase + sidx * static_stage_bytes<T>());
             // x at the block's columns: four loads in flight per thread
             for (int p = p0 + a; p < pend; p += 4 * (int)blockDim.x) {
@@ -603,6 +609,7 @@ __global__ void __launch_bounds__(1024, 1) k_static(Mat<T> A, const T *__restric
             // so the rows proceed side by side however long they are
 #pragma unroll 8
             for (int p = cur.q0; p < cur.q1; ++p) acc = Ar<T>::fma(A.val[p], x[(long long)A.col[p] * ld], acc);
+            first_of_w();
         }
         // the next block's per-row data, in flight during the solve below
         StaticRow<T> nxt{0, 0, 0, -1, T(0), T(0)};
