@@ -912,13 +912,13 @@ __global__ void __launch_bounds__(256, 4) k_residual(Mat<T> A, const T *__restri
 // of stages (dense_rows.cuh), row-major values, one block per SM.  W pairs per
 // block run, with longer and more stages the fewer they are, so that a short A
 // (few chains) keeps more bytes of each in flight.  A warp's number decides which
-// quarter of the SM issues it: from five pairs on, and where FP32 values are widened
-// from two on, the summing warps are the first eight and the copying warps the others, one
-// quarter further on, so that every quarter has its share of both.  (With the two kinds
-// taking turns the sums ran in two quarters.  Whole calls at 200,000 x 2,048: 760 us
-// in FP64 against 724, 1,233 against 822 over FP32 values, whose widening is integer
-// work; 15,000 rows of those 164 against 141.  Four chains of FP64 values, 15,000 rows, are
-// better off in turns: 117 us against 125.)
+// quarter of the SM issues it.  Where the pairs have more than one group each, and where
+// FP32 values are widened, the summing warps are the first eight and the copying warps the
+// others, one quarter further on, so that every quarter has its share of both.  (With
+// the two kinds taking turns the sums ran in two quarters.  Whole calls at 200,000 x
+// 2,048: 760 us in FP64 against 724, 1,233 against 822 over FP32 values, whose widening is
+// integer work; 15,000 rows of those 164 against 141.  Pairs with one group are better off
+// in turns: 15,000 x 2,048 in FP64 117 us against 125, 20,000 x 512 51 against 58.)
 // 200,000 x 2,048 FP32: 300 -> 262 us, 0.92 of measured HBM; 25,600 x 2,048 FP64:
 // 175 -> 117 us (bound by the FP64 rate: 107); 2,048 x 100,000: 8,300 -> 3,628 us
 // FP64, 4,280 -> 284 us FP32 (bound by the chains: 3,200 and 240).
@@ -931,18 +931,17 @@ template <typename T, typename V, int RB, int ST>
 __global__ void __launch_bounds__(512, 1) k_residual_dense(const V *__restrict__ val, int m, int n, int K,
                                                           const T *__restrict__ b, const T *__restrict__ x,
                                                           T *__restrict__ r, double *partials, unsigned *hist1,
-                                                          Ctl *ctl, int finalize, int W) {
+                                                          Ctl *ctl, int finalize, int W, int spread) {
     extern __shared__ __align__(16) unsigned char dr_ring[];
     __shared__ unsigned hist[kHistBins];
     if ((finalize == 1 || finalize == 3) && (ctl->done || ctl->halt)) return;
-    constexpr bool spread = ST == 3 || (ST == 6 && sizeof(V) < sizeof(T));
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool load = spread ? warp >= kDrMaxPairs : warp & 1;
-    const int pair = spread ? (warp - load) & (kDrMaxPairs - 1) : ST == 8 ? 0 : warp >> 1;
+    const int pair = spread ? (warp - load) & (kDrMaxPairs - 1) : warp >> 1;
     for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) hist[i] = 0u;
     __syncthreads();
     double rr = 0.0;
-    if (ST == 8 ? threadIdx.x < 64 : pair < W) {
+    if (pair < W) {
         const bool vec = ((long long)n * (int)sizeof(V)) % 16 == 0;
         const int nsl = (m + 31) / 32, Wt = gridDim.x * W, g = pair * gridDim.x + blockIdx.x;
         unsigned char *ring = dr_ring + (size_t)pair * ST * DenseStage<T, V, RB>::bytes;
@@ -3949,9 +3948,11 @@ template <>
 const float *row_major<float>(const rorbk_ctx *h) { return h->val32; }
 
 template <typename T, typename V, int RB, int ST>
-static void residual_dense_launch(rorbk_ctx *h, const T *b, const T *x, T *r, Ctl *ctl, int finalize, int g, int W) {
+static void residual_dense_launch(rorbk_ctx *h, const T *b, const T *x, T *r, Ctl *ctl, int finalize, int g, int W,
+                                  int per) {
+    const int spread = per > 1 && (sizeof(V) < sizeof(T) || per > W);
     k_residual_dense<T, V, RB, ST><<<g, 512, dense_res_smem<T, V, RB, ST>(W), h->stream>>>(
-        row_major<V>(h), (int)h->m, (int)h->n, h->K, b, x, r, h->partials, h->hist1, ctl, finalize, W);
+        row_major<V>(h), (int)h->m, (int)h->n, h->K, b, x, r, h->partials, h->hist1, ctl, finalize, W, spread);
 }
 
 // The residual kernel for this handle's format.  Dense: as many pairs of warps
@@ -3972,14 +3973,14 @@ static void residual_launch(rorbk_ctx *h, const Mat<T> &A, const T *b, const T *
         return;
     }
     const int nsl = (int)((h->m + 31) / 32), g = std::min(h->grid_res, nsl), per = (nsl + g - 1) / g;
-    if (per == 1) residual_dense_launch<T, V, 512, 8>(h, b, x, r, ctl, finalize, g, 1);
-    else if (per == 2) residual_dense_launch<T, V, 512, 6>(h, b, x, r, ctl, finalize, g, 2);
-    else if (per <= 4) residual_dense_launch<T, V, 256, 6>(h, b, x, r, ctl, finalize, g, per);
+    if (per == 1) residual_dense_launch<T, V, 512, 8>(h, b, x, r, ctl, finalize, g, 1, per);
+    else if (per == 2) residual_dense_launch<T, V, 512, 6>(h, b, x, r, ctl, finalize, g, 2, per);
+    else if (per <= 4) residual_dense_launch<T, V, 256, 6>(h, b, x, r, ctl, finalize, g, per, per);
     else {
         int W = kDrMaxPairs;
         for (int c = kDrMaxPairs - 1; c >= 5; --c)
             if ((per + c - 1) / c * c < (per + W - 1) / W * W) W = c;
-        residual_dense_launch<T, V, 256, 3>(h, b, x, r, ctl, finalize, g, W);
+        residual_dense_launch<T, V, 256, 3>(h, b, x, r, ctl, finalize, g, W, per);
     }
 }
 
