@@ -35,6 +35,23 @@ __device__ __forceinline__ void cp_async_elem(unsigned dst, const void *src) {
     static_assert(N == 4 || N == 8, "element copies");
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(N) : "memory");
 }
+// The same with an L2 eviction policy: lines that are the first to be evicted.
+__device__ __forceinline__ unsigned long long l2_stream_policy() {
+    unsigned long long p;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+__device__ __forceinline__ void cp_async16(unsigned dst, const void *src, int bytes, unsigned long long pol) {
+    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2, %3;" ::"r"(dst), "l"(src), "r"(bytes),
+                 "l"(pol)
+                 : "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_elem(unsigned dst, const void *src, unsigned long long pol) {
+    static_assert(N == 4 || N == 8, "element copies");
+    asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(N), "l"(pol)
+                 : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
@@ -45,10 +62,11 @@ template <> struct Pack16<double> { using type = double2; };
 
 // A pair of warps: acc_l = sum over j ascending of A0[l * n + j] x[j] (one fused
 // chain from 0) for the lanes l < rows, in the warp that calls dense_sum; the
-// other warp calls dense_copy for the same rows.  ring: ST stages of DenseStage<T, V, RB>::bytes.  vec: every
-// row starts on a 16-byte boundary (n * sizeof(V) % 16 == 0); else the rows are
-// copied value by value.  The pair meets at named barrier `bar` once per stage:
-// behind it stage k has landed and stage k - 1 is free.
+// other warp calls dense_copy for the same rows.  ring: ST stages of
+// DenseStage<T, V, RB>::bytes.  vec: every row starts on a 16-byte boundary
+// (n * sizeof(V) % 16 == 0); else the rows are copied value by value.  STREAM: A's
+// lines are the first that L2 evicts.  The pair meets at named barrier `bar` once
+// per stage: behind it stage k has landed and stage k - 1 is free.
 __device__ __forceinline__ void pair_sync(int bar) {
     __syncwarp();
     switch (bar) {                                    // an immediate barrier number
@@ -63,7 +81,7 @@ __device__ __forceinline__ void pair_sync(int bar) {
     }
 }
 
-template <typename T, typename V, int RB, int ST>
+template <typename T, typename V, int RB, int ST, bool STREAM = false>
 __device__ __forceinline__ void dense_copy(const V *__restrict__ A0, int rows, int n, const T *__restrict__ x,
                                            unsigned char *ring, bool vec, int bar) {
     using S = DenseStage<T, V, RB>;
@@ -73,6 +91,8 @@ __device__ __forceinline__ void dense_copy(const V *__restrict__ A0, int rows, i
     const int nst = (n + S::cols - 1) / S::cols;
     {
         const unsigned rb = smem_u32(ring);
+        unsigned long long pol = 0;
+        if constexpr (STREAM) pol = l2_stream_policy();
         const int ch = lane % (RB / 16), u0 = lane / (RB / 16);
         auto issue = [&](int k) {
             if (k < nst) {
@@ -84,7 +104,10 @@ __device__ __forceinline__ void dense_copy(const V *__restrict__ A0, int rows, i
                     unsigned dst = sb + u0 * S::pitch + ch * 16;
 #pragma unroll
                     for (int u = 0; u < 32; u += RP) {
-                        if (u + u0 < rows && bytes > 0) cp_async16(dst, src, bytes);
+                        if (u + u0 < rows && bytes > 0) {
+                            if constexpr (STREAM) cp_async16(dst, src, bytes, pol);
+                            else cp_async16(dst, src, bytes);
+                        }
                         src += (long long)RP * n;
                         dst += RP * S::pitch;
                     }
@@ -93,9 +116,11 @@ __device__ __forceinline__ void dense_copy(const V *__restrict__ A0, int rows, i
 #pragma unroll
                         for (int q = 0; q < S::cols / 32; ++q) {
                             const int c = c0 + 32 * q + lane;
-                            if (c < n)
-                                cp_async_elem<sizeof(V)>(sb + u * S::pitch + (32 * q + lane) * (int)sizeof(V),
-                                                         A0 + (long long)u * n + c);
+                            const unsigned d = sb + u * S::pitch + (32 * q + lane) * (int)sizeof(V);
+                            if (c < n) {
+                                if constexpr (STREAM) cp_async_elem<sizeof(V)>(d, A0 + (long long)u * n + c, pol);
+                                else cp_async_elem<sizeof(V)>(d, A0 + (long long)u * n + c);
+                            }
                         }
                 }
 #pragma unroll

@@ -150,6 +150,7 @@ struct rorbk_ctx {
     double mu = 0;
     int precision_built = 0;
     int num_sms = 0;
+    int l2_bytes = 0;
     int64_t bytes = 0;
     std::vector<void *> allocs;                       // memory this handle alone owns
     std::shared_ptr<rorbk::DevBlocks> shared_setup;   // set-up memory shared with clones

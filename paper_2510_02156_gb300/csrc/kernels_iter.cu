@@ -931,7 +931,8 @@ template <typename T, typename V, int RB, int ST>
 __global__ void __launch_bounds__(512, 1) k_residual_dense(const V *__restrict__ val, int m, int n, int K,
                                                           const T *__restrict__ b, const T *__restrict__ x,
                                                           T *__restrict__ r, double *partials, unsigned *hist1,
-                                                          Ctl *ctl, int finalize, int W, int spread) {
+                                                          Ctl *ctl, int finalize, int W, int spread,
+                                                          int stream) {
     extern __shared__ __align__(16) unsigned char dr_ring[];
     __shared__ unsigned hist[kHistBins];
     if ((finalize == 1 || finalize == 3) && (ctl->done || ctl->halt)) return;
@@ -946,8 +947,12 @@ __global__ void __launch_bounds__(512, 1) k_residual_dense(const V *__restrict__
         const int nsl = (m + 31) / 32, Wt = gridDim.x * W, g = pair * gridDim.x + blockIdx.x;
         unsigned char *ring = dr_ring + (size_t)pair * ST * DenseStage<T, V, RB>::bytes;
         if (load) {
-            for (int sl = g; sl < nsl; sl += Wt)
-                dense_copy<T, V, RB, ST>(val + (long long)sl * 32 * n, min(32, m - sl * 32), n, x, ring, vec, 1 + pair);
+            for (int sl = g; sl < nsl; sl += Wt) {
+                const V *A0 = val + (long long)sl * 32 * n;
+                const int rows = min(32, m - sl * 32);
+                if (ST == 3 && sizeof(V) == sizeof(T) && stream) dense_copy<T, V, RB, ST, ST == 3>(A0, rows, n, x, ring, vec, 1 + pair);
+                else dense_copy<T, V, RB, ST>(A0, rows, n, x, ring, vec, 1 + pair);
+            }
         } else {
             for (int sl = g; sl < nsl; sl += Wt) {
                 const int row = sl * 32 + lane;
@@ -3951,8 +3956,15 @@ template <typename T, typename V, int RB, int ST>
 static void residual_dense_launch(rorbk_ctx *h, const T *b, const T *x, T *r, Ctl *ctl, int finalize, int g, int W,
                                   int per) {
     const int spread = per > 1 && (sizeof(V) < sizeof(T) || per > W);
+    // An A as large as L2 would leave none of the iteration's other data there: where the
+    // pairs work through several groups its lines go first.  (FP32 60,000 x 2,048 126 ->
+    // 115 us, 30,000 x 1,001 77 -> 66; the initial solution of 30,000 x 1,001, whose
+    // block's data then stay in L2, 356 -> 207.  Over widened FP32 values it costs 2%, in
+    // the one-group pairs of few long rows 6%.)
+    const int stream = 4 * h->m * h->n * (int64_t)sizeof(V) > 3 * (int64_t)h->l2_bytes;
     k_residual_dense<T, V, RB, ST><<<g, 512, dense_res_smem<T, V, RB, ST>(W), h->stream>>>(
-        row_major<V>(h), (int)h->m, (int)h->n, h->K, b, x, r, h->partials, h->hist1, ctl, finalize, W, spread);
+        row_major<V>(h), (int)h->m, (int)h->n, h->K, b, x, r, h->partials, h->hist1, ctl, finalize, W, spread,
+        stream);
 }
 
 // The residual kernel for this handle's format.  Dense: as many pairs of warps

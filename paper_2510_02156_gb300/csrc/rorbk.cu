@@ -431,6 +431,7 @@ rorbk_status rorbk_setup(const rorbk_matrix *A, const rorbk_partition *part, dou
     cudaGetDevice(&h->device);
     h->stream = (cudaStream_t)opt.stream;
     cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
+    cudaDeviceGetAttribute(&h->l2_bytes, cudaDevAttrL2CacheSize, h->device);
     h->m = m; h->n = n; h->nnz = nnz; h->k = k;
     h->format = A->format; h->vdtype = A->dtype;
     h->K = (int)(m / k);
