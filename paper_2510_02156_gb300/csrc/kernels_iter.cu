@@ -937,12 +937,13 @@ __global__ void __launch_bounds__(512, 1) k_residual_dense(const V *__restrict__
     __shared__ unsigned hist[kHistBins];
     if ((finalize == 1 || finalize == 3) && (ctl->done || ctl->halt)) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool load = spread ? warp >= kDrMaxPairs : warp & 1;
-    const int pair = spread ? (warp - load) & (kDrMaxPairs - 1) : warp >> 1;
+    const bool sp = ST < 8 && spread;
+    const bool load = sp ? warp >= kDrMaxPairs : warp & 1;
+    const int pair = ST == 8 ? 0 : sp ? (warp - load) & (kDrMaxPairs - 1) : warp >> 1;
     for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) hist[i] = 0u;
     __syncthreads();
     double rr = 0.0;
-    if (pair < W) {
+    if (ST == 8 ? threadIdx.x < 64 : pair < W) {
         const bool vec = ((long long)n * (int)sizeof(V)) % 16 == 0;
         const int nsl = (m + 31) / 32, Wt = gridDim.x * W, g = pair * gridDim.x + blockIdx.x;
         unsigned char *ring = dr_ring + (size_t)pair * ST * DenseStage<T, V, RB>::bytes;
