@@ -29,12 +29,13 @@
 //     others apply the finished rows of the solution further up.
 // Two cluster barriers per panel order the traffic through L2.
 //
-// Measured (16 blocks, one launch): order 256 321 us (mixed form's factor
-// 237 us), order 100 121 us, order 40 51 us, order 500 866 us; with the whole
-// trailing update awaited 348, 128, 54 and 995 us.  At order 256 about 356 kcycles of
-// 622 are the 256 columns and 100 the backward solve.  Before: 15 grid-wide launches
-// and a one-block backward solve, 1,003 us at order 256 (dense A); the sparse
-// dynamic block, factored by one block of threads, 2,230 us at about 230 coupled
+// Measured (16 blocks, one launch; 8 at order 100, 4 at 40): order 256 329 us (mixed
+// form's factor 237 us), order 100 123 us, order 40 50 us, order 500 861 us; with one
+// remainder per quotient in the panel, which does not round every one, 321, 121, 51 and
+// 866, of order 256's 622 kcycles about 356 in the 256 columns and 100 in the backward
+// solve; with the whole trailing update awaited 348, 128, 54 and 995 us.  Before: 15
+// grid-wide launches and a one-block backward solve, 1,003 us at order 256 (dense A); the
+// sparse dynamic block, factored by one block of threads, 2,230 us at about 230 coupled
 // rows.
 //
 // Order of operations.  Every entry receives g = fma(-L_aj, L_bj, g) over

@@ -919,9 +919,10 @@ __global__ void __launch_bounds__(256, 4) k_residual(Mat<T> A, const T *__restri
 // 2,048: 760 us in FP64 against 724, 1,233 against 822 over FP32 values, whose widening is
 // integer work; 15,000 rows of those 164 against 141.  Pairs with one group are better off
 // in turns: 15,000 x 2,048 in FP64 117 us against 125, 20,000 x 512 51 against 58.)
-// 200,000 x 2,048 FP32: 300 -> 262 us, 0.92 of measured HBM; 25,600 x 2,048 FP64:
-// 175 -> 117 us (bound by the FP64 rate: 107); 2,048 x 100,000: 8,300 -> 3,628 us
-// FP64, 4,280 -> 284 us FP32 (bound by the chains: 3,200 and 240).
+// 200,000 x 2,048 in a launch list: FP32 300 -> 259 us (0.9 of measured HBM with a cold
+// L2), FP64 704 -> 699 us (bound by the FP64 rate); 25,600 x 2,048 FP64: 175 -> 117 us
+// (the FP64 rate: 107); 2,048 x 100,000: 8,300 -> 3,628 us FP64, 4,280 -> 284 us FP32 (bound
+// by the chains: 3,200 and 240).
 constexpr int kDrMaxPairs = 8;
 
 template <typename T, typename V, int RB, int ST>
@@ -3836,9 +3837,9 @@ static cudaError_t cluster_launch(cudaStream_t st, void (*kernel)(A...), dim3 gr
 }
 
 // Blocks of the cluster that factors a Gram of order up to K (0: none is
-// needed or none can be resident).  Measured at order 256: 321 us with 16
-// blocks, 361 us with 8 (the trailing updates); at order 100 both take 121 us,
-// so 8 serve orders up to 128 and a block of columns, whose clusters run side
+// needed or none can be resident).  Measured with one remainder per quotient:
+// at order 256 321 us with 16 blocks, 361 us with 8 (the trailing updates); at order
+// 100 both take 121 us, so 8 serve orders up to 128 and a block of columns, whose clusters run side
 // by side.  Orders up to 64 have one small trailing update: 4 blocks.
 int chol_cluster_blocks(rorbk_ctx *h) {
     const bool dense = h->format == RORBK_FORMAT_DENSE || h->K >= h->n;
@@ -3972,7 +3973,7 @@ static void residual_dense_launch(rorbk_ctx *h, const T *b, const T *x, T *r, Ct
 // per SM as there are groups of 32 rows for it.  From five on (four keep the
 // FP64 unit busy) the count that leaves the fewest idle in the last round: a
 // lone chain runs at a quarter of the SM's FP64 rate (200,000 rows, 42 groups
-// per SM: 775 us with 8 pairs, 732 with 7).
+// per SM, before the warps were spread: 775 us with 8 pairs, 732 with 7).
 template <typename T, typename V>
 static void residual_launch(rorbk_ctx *h, const Mat<T> &A, const T *b, const T *x, T *r, Ctl *ctl,
                             int finalize) {
