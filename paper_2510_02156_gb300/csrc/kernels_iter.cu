@@ -919,8 +919,8 @@ __global__ void __launch_bounds__(256, 4) k_residual(Mat<T> A, const T *__restri
 // 2,048: 760 us in FP64 against 724, 1,233 against 822 over FP32 values, whose widening is
 // integer work; 15,000 rows of those 164 against 141.  Pairs with one group are better off
 // in turns: 15,000 x 2,048 in FP64 117 us against 125, 20,000 x 512 51 against 58.)
-// 200,000 x 2,048 in a launch list: FP32 300 -> 259 us (0.9 of measured HBM with a cold
-// L2), FP64 704 -> 699 us (bound by the FP64 rate); 25,600 x 2,048 FP64: 175 -> 117 us
+// 200,000 x 2,048 in a launch list: FP32 300 -> 249 us (0.9 of measured HBM with a cold
+// L2), FP64 704 -> 693 us (bound by the FP64 rate); 25,600 x 2,048 FP64: 175 -> 117 us
 // (the FP64 rate: 107); 2,048 x 100,000: 8,300 -> 3,628 us FP64, 4,280 -> 284 us FP32 (bound
 // by the chains: 3,200 and 240).
 constexpr int kDrMaxPairs = 8;
