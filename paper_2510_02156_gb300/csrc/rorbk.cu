@@ -596,7 +596,8 @@ rorbk_status rorbk_update_values(rorbk_handle h, const void *values, int32_t dty
         }
         cudaFree(tmp);
     }
-    if (!st) st = build_setup(h, std::vector<int>(), true);
+    if (!st && (st = build_setup(h, std::vector<int>(), true)))
+        cudaStreamSynchronize(s);           // the caller's values are no longer read
     if (!st && h->values_version) ++*h->values_version;
     // this handle's own column-major copy now; those of handles sharing the
     // set-up at their next incremental solve
