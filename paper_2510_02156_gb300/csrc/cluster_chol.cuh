@@ -15,9 +15,8 @@
 //     dealt over the cluster, every block factors the diagonal block itself
 //     (identical operations), so a panel needs no communication;
 //   - inside a column two warps form the pivot and divide, with 1 / sqrt(d) taken
-//     first and root and quotients from it by fused remainders (pivot.cuh: 13
-//     dependent FP64 operations, the column's last update included, and no call to
-//     sqrt or to a division), while six warps apply
+//     first and root and quotients from it by fused remainders (pivot.cuh; no call
+//     to sqrt or to a division), while six warps apply
 //     the previous column to the columns after the next, from registers;
 //   - the trailing update of a panel runs over all warps of the cluster (a lane
 //     per column, a few rows per warp) from a copy of the panel in shared memory;
@@ -29,13 +28,12 @@
 //     others apply the finished rows of the solution further up.
 // Two cluster barriers per panel order the traffic through L2.
 //
-// Measured (16 blocks, one launch; 8 at order 100, 4 at 40): order 256 329 us (mixed
-// form's factor 237 us), order 100 123 us, order 40 50 us, order 500 861 us; with one
-// remainder per quotient in the panel, which does not round every one, 321, 121, 51 and
-// 866, of order 256's 622 kcycles about 356 in the 256 columns and 100 in the backward
-// solve; with the whole trailing update awaited 348, 128, 54 and 995 us.  Before: 15
-// grid-wide launches and a one-block backward solve, 1,003 us at order 256 (dense A); the
-// sparse dynamic block, factored by one block of threads, 2,230 us at about 230 coupled
+// Measured (16 blocks, one launch; 8 at order 100, 4 at 40): order 256 313 us (mixed
+// form's factor 237 us), order 100 116 us, order 40 47 us, order 500 837 us; with the
+// whole trailing update awaited 348, 128, 54 and 995 us.  At order 256 about 356 kcycles of
+// 622 are the 256 columns and 100 the backward solve.  Before: 15 grid-wide launches
+// and a one-block backward solve, 1,003 us at order 256 (dense A); the sparse
+// dynamic block, factored by one block of threads, 2,230 us at about 230 coupled
 // rows.
 //
 // Order of operations.  Every entry receives g = fma(-L_aj, L_bj, g) over
@@ -163,7 +161,7 @@ __device__ __forceinline__ void cc_panel(double *Ld, double *R, int w, int nr, d
                 q = v * rl;
             } else {
                 const Pivot pv = pivot(d);
-                q = pivot_div_early(v, pv);
+                q = pivot_div(v, pv);
                 rl = pv.rl;
                 dg = pv.l;
             }

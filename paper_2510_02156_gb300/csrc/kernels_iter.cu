@@ -3837,7 +3837,7 @@ static cudaError_t cluster_launch(cudaStream_t st, void (*kernel)(A...), dim3 gr
 }
 
 // Blocks of the cluster that factors a Gram of order up to K (0: none is
-// needed or none can be resident).  Measured with one remainder per quotient:
+// needed or none can be resident).  Measured (an earlier form of the panel):
 // at order 256 321 us with 16 blocks, 361 us with 8 (the trailing updates); at order
 // 100 both take 121 us, so 8 serve orders up to 128 and a block of columns, whose clusters run side
 // by side.  Orders up to 64 have one small trailing update: 4 blocks.

@@ -3,8 +3,8 @@
 // GB300's FP64 square root and division take 611 and 581 cycles where a
 // multiply-add takes 64, and every column of a factor waits for one of each.
 // Here one approximation of 1 / sqrt(d) serves both, and fused remainders round
-// them (P. W. Markstein, IBM J. Res. Dev. 34, 1990): eight dependent operations to
-// the root, four more to the quotient.
+// them (P. W. Markstein, IBM J. Res. Dev. 34, 1990): eight operations to the root, five
+// more to the quotient.
 //
 // Bounds (u = 2^-53; relative errors; the hardware's approximation of the
 // reciprocal square root is good to 20 bits):
@@ -26,11 +26,11 @@
 //     between two numbers and, next to one, q is half a unit away from it; so the rounding of
 //     q + r rl is that of v / l while L^2 (1 + 2^-48) < 2^106.  divisor_ok keeps the
 //     mantissas closest to all ones, where that fails, out.
-//     - pivot_div: q = v rl is within 1.5 units, next to a middle within half.
-//     - pivot_div_early: v y is not behind l and rl, but up to three units away
-//       (the errors of y, of l and of the product), and its remainder not exact:
-//       the first correction, by y, brings it within half a unit and 2^-48, the
-//       second rounds it.
+//     So q = v rl (pivot_div): within 1.5 units, next to a middle within half.  (v y, which
+//     need not wait for l, is up to three units away, and its remainder not exact.  A
+//     warp issues an FP64 instruction every 64 cycles whatever depends on what, so
+//     the wait costs nothing: 313 against 312 us at order 256, and 329 with a second
+//     correction behind v y.)
 // root_ok, divisor_ok and the test of v's exponent keep every intermediate
 // normal; other operands take sqrt and the division themselves.
 #pragma once
@@ -120,10 +120,6 @@ __device__ __forceinline__ Pivot pivot(double d) {
 #endif
 __device__ __forceinline__ double pivot_div(double v, const Pivot &p) {      // RN(v / l)
     return quotient_rn(v, __dmul_rn(v, p.rl), p.l, p.rl, p.ok);
-}
-__device__ __forceinline__ double pivot_div_early(double v, const Pivot &p) {      // RN(v / l), v y formed beside l
-    const double q0 = __dmul_rn(v, p.y);
-    return quotient_rn(v, __fma_rn(__fma_rn(-q0, p.l, v), p.y, q0), p.l, p.rl, p.ok);
 }
 
 }  // namespace rorbk
